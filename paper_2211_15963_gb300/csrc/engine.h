@@ -82,13 +82,11 @@ __host__ __device__ __forceinline__ void philox4x64_10(unsigned long long c[4], 
   }
 }
 
-constexpr int kTile = 1024;         // neurons per update block
-constexpr int kUpdThreads = 256;    // four neurons per thread
+constexpr int kTile = 1024;         // neurons per tile: the unit of instance placement
+constexpr int kUpdThreads = 128;    // four neurons per thread: half a tile
 constexpr int kDelThreads = 256;
 constexpr int kMaxThr = 16;         // Poisson inversion thresholds
-constexpr int kTileRegions = 8;     // region constants staged in shared memory
 
-// 16-byte multiples: the update kernel moves these with bulk copies
 // (laid out as 16-byte vectors: the update kernel reads them with 128-bit loads)
 struct alignas(16) RegionConst {
   float g[4];                        // channel conductance scales

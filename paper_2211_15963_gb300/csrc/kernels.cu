@@ -68,6 +68,7 @@ __device__ __forceinline__ int find_region(const int32_t* __restrict__ ro, int R
 #endif
 constexpr int kWalkU = DBNET_WALK_CHUNKS;
 constexpr int kSegGroup = 32;  // spikes per transposition group of the segment-ring copy
+constexpr int kTileWarps = kTile / 128;  // warps of an update tile, 128 neurons each
 constexpr int kMaxPhases = 8;  // rank phases of the arrival items (see k_deliver)
 
 __device__ __forceinline__ unsigned long long l2_policy_first() {
@@ -140,7 +141,7 @@ __device__ double bw_euler(double* x, double z, const InstDesc& d) {
   return d.V0 * (k1 * (1.0 - q2) + k2 * (1.0 - q2 / v2) + k3 * (1.0 - v2));
 }
 
-__global__ void __launch_bounds__(kUpdThreads) k_init_state(EngineDev e, int inst, int first_tile) {
+__global__ void __launch_bounds__(kTile / 4) k_init_state(EngineDev e, int inst, int first_tile) {
   const InstDesc& d = e.insts[inst];
   const int64_t gi0 = (int64_t)(first_tile + blockIdx.x) * kTile + threadIdx.x * 4;
   const int32_t li0 = (int32_t)(gi0 - d.base);
@@ -222,22 +223,171 @@ __device__ __forceinline__ float normal_from_word(unsigned long long w) {
   return sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
 }
 
+// Where an iteration's accumulators lie: slot a mod acc_slots (one slot, two,
+// or the emission ring).
+__device__ __forceinline__ int2* acc_of(const EngineDev& e, unsigned long long g) {
+  const unsigned n = (unsigned)e.acc_slots;
+  const unsigned slot = n <= 2u ? (unsigned)g & (n - 1u) : (unsigned)(g % (unsigned long long)n);
+  return e.acc + (size_t)slot * (size_t)e.stride * (e.four ? 2 : 1);
+}
+
+// a / b for step counts: in 32 bits while they fit
+__device__ __forceinline__ long long div_steps(long long a, int b) {
+  return (unsigned long long)a >> 32 ? a / b : (long long)((uint32_t)a / (uint32_t)b);
+}
+
+// Region constants of a thread's four neurons: one region's for all (ONE), or
+// each neuron's own.
+template <bool ONE>
+struct QuadConst {
+  const RegionConst* p;  // the tile's first region
+  int r[ONE ? 1 : 4];    // the neurons' regions, counted from it
+  __device__ __forceinline__ const RegionConst& of(int k) const { return ONE ? *p : p[r[ONE ? 0 : k]]; }
+};
+
+// What the membrane step of a thread's four neurons leaves: bit k of spk and
+// cls for a spike of neuron k and its inhibitory class.
+struct QuadSpikes {
+  unsigned spk = 0, cls = 0;
+};
+
+// One Euler step of the thread's four neurons (m of them exist).  The traces
+// go channel by channel over the four, so that only one channel's constants
+// and one float4 of traces are live at a time, and each float4 is stored as
+// soon as it is updated.
+template <bool EXT, bool FOUR, bool ONE>
+__device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDesc& d, const QuadConst<ONE>& rc,
+                                                int m, int64_t gi0, int32_t li0, long long n,
+                                                float4 V4, const float4 (&J4)[4], uchar4 rf, const int4 (&A)[FOUR ? 4 : 2]) {
+  unsigned long long x[4] = {(unsigned long long)n, (unsigned long long)(li0 >> 2), 0ull, 0ull};
+  philox4x64_10(x, d.seed, d.net_id);
+  // background: Poisson count by integer inversion of 32 Philox bits (the
+  // thresholds are non-decreasing: count them up to the first miss), added
+  // to AMPA and NMDA
+  int dq[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const RegionConst& p = rc.of(k);
+    const uint32_t uu = (uint32_t)(x[k] >> 32);
+    const int n_thr = __ldg(&p.n_thr);
+    int c = 0;
+    while (c < n_thr && uu >= __ldg(&p.thr[c])) ++c;
+    dq[k] = c * __ldg(&p.q_ext);
+  }
+  const float v[4] = {V4.x, V4.y, V4.z, V4.w};
+  float Isyn[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {  // the membrane sees the old V and traces
+    const float jo[4] = {J4[u].x, J4[u].y, J4[u].z, J4[u].w};
+    float jn[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const RegionConst& p = rc.of(k);
+      const float gj = __fmul_rn(__ldg(&p.g[u]), jo[k]);
+      const float dv = __fsub_rn(__ldg(&p.Vu[u]), v[k]);
+      Isyn[k] = __fadd_rn(Isyn[k], __fmul_rn(gj, dv));
+      // traces: decay, then this step's arrivals
+      const int4 Ak = FOUR ? A[k] : A[k >> 1];
+      const int q = FOUR ? (u == 0 ? Ak.x : u == 1 ? Ak.y : u == 2 ? Ak.z : Ak.w)
+                         : ((k & 1) ? (u < 2 ? Ak.z : Ak.w) : (u < 2 ? Ak.x : Ak.y));
+      const float xu = __fmul_rn(__int2float_rn(u < 2 ? q + dq[k] : q), d.inv_two_S);
+      jn[k] = __fadd_rn(__fmul_rn(__ldg(&p.dec[u]), jo[k]), xu);
+    }
+    if (m == 4) {
+      __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + gi0), make_float4(jn[0], jn[1], jn[2], jn[3]));
+    } else {  // the last neurons of an instance: the padding keeps its values
+      __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + gi0),
+             make_float4(jn[0], m > 1 ? jn[1] : jo[1], m > 2 ? jn[2] : jo[2], jo[3]));
+    }
+  }
+  // the background current and the injected-current factors, only where the
+  // instance has them (a request server's engine runs this variant for
+  // every request)
+  const bool ou = EXT && (d.ext & kExtOU), het = EXT && (d.ext & kExtHet);
+  float4 B4 = make_float4(0.f, 0.f, 0.f, 0.f), F4 = make_float4(1.f, 1.f, 1.f, 1.f);
+  if (ou) B4 = __ldcs(reinterpret_cast<const float4*>(e.Ibg + gi0));
+  if (het) F4 = __ldg(reinterpret_cast<const float4*>(e.fext + gi0));
+  float ib[4] = {B4.x, B4.y, B4.z, B4.w};
+  const float fe[4] = {F4.x, F4.y, F4.z, F4.w};
+  unsigned long long xo[4] = {0ull, 0ull, 0ull, 0ull};
+  if (ou) {  // the OU noise: stream 4
+    xo[0] = (unsigned long long)n;
+    xo[1] = (unsigned long long)(li0 >> 2);
+    xo[2] = 4ull;
+    philox4x64_10(xo, d.seed, d.net_id);
+  }
+  float vo[4];
+  int rr[4] = {rf.x, rf.y, rf.z, rf.w};
+  QuadSpikes out;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    vo[k] = v[k];
+    if (k >= m) continue;
+    const RegionConst& p = rc.of(k);
+    const float4 M = __ldg(reinterpret_cast<const float4*>(&p.dtC));     // dtC gL VL Vth
+    const float4 Q = __ldg(reinterpret_cast<const float4*>(&p.Vreset));  // Vreset Iext n_ref q_ext
+    const float leak = __fmul_rn(M.y, __fsub_rn(v[k], M.z));
+    float I = __fsub_rn(Isyn[k], leak);
+    float4 OUc = make_float4(0.f, 0.f, 0.f, 0.f);  // mu, dt/tau, sigma sqrt(2 dt/tau), bits
+    if (EXT && d.ext) OUc = __ldg(reinterpret_cast<const float4*>(&p.ou_mu));
+    const int xb = __float_as_int(OUc.w);
+    // injected current, scaled by the neuron's factor where heterogeneous
+    const float ie = (EXT && (xb & kExtHet)) ? __fmul_rn(Q.y, fe[k]) : Q.y;
+    I = __fadd_rn(I, ie);
+    if (EXT && (xb & kExtOU)) I = __fadd_rn(I, ib[k]);  // I_bg before this step
+    const float vn = __fadd_rn(v[k], __fmul_rn(I, M.x));
+    if (EXT && (xb & kExtOU)) {  // Eq. 1, Euler-Maruyama
+      const float xi = normal_from_word(xo[k]);
+      const float t1 = __fmul_rn(__fsub_rn(OUc.x, ib[k]), OUc.y);
+      ib[k] = __fadd_rn(ib[k], t1);
+      ib[k] = __fadd_rn(ib[k], __fmul_rn(OUc.z, xi));
+    }
+    // refractory clamp, threshold, reset
+    if (rr[k] > 0) {
+      vo[k] = Q.x;
+      rr[k] -= 1;
+    } else if (vn >= M.w) {
+      vo[k] = Q.x;
+      rr[k] = __float_as_int(Q.z);
+      out.spk |= 1u << k;
+      if (li0 + k >= __ldg(&p.exc_end)) out.cls |= 1u << k;
+    } else {
+      vo[k] = vn;
+    }
+  }
+  __stcs(reinterpret_cast<float4*>(e.V + gi0), make_float4(vo[0], vo[1], vo[2], vo[3]));
+  __stcs(reinterpret_cast<uchar4*>(e.ref + gi0),
+         make_uchar4((unsigned char)rr[0], (unsigned char)rr[1], (unsigned char)rr[2], (unsigned char)rr[3]));
+  if (ou) __stcs(reinterpret_cast<float4*>(e.Ibg + gi0), make_float4(ib[0], ib[1], ib[2], ib[3]));
+  return out;
+}
+
+// One warp's 128 neurons of a tile, in the iteration sr names.
+//
 // EXT: also the kExt* terms of the instances that have them: the background
 // OU current and the per-neuron injected-current factor.  FOUR: the
 // accumulators hold four channels per neuron (two weights per edge); the
 // background drive adds to both AMPA and NMDA.
 //
-// One tile of the iteration sr names; the block's threads call it together.
+// Bound: the state's traffic (58 bytes a neuron and step) on large networks,
+// the latency of the loads on small ones.  The warps of a tile share
+// nothing, so the kernel has no block barrier: a warp's region constants
+// come through the L1 (one 176-byte row, the same for most warps of an SM),
+// its Philox rounds run under its state loads, and a warp without spikes
+// ends after its stores.  A tile inside one region (most) reads its
+// constants once for four neurons.  Measured against blocks of 256 that
+// staged constants in shared memory behind a barrier, one neuron after the
+// other: 51.0 us against 59.8 us at 5 M neurons (5.7 TB/s of 290 MB),
+// 25.9 against 30.1 us at 2 M.  Seven blocks of 128 (72 registers) beat six
+// (53.2 us) and eight (64 registers, spills: 51.3 us, and 56.1 against
+// 53.2 us with 50,000 spikes a step); an L2 prefetch of the state 304 to
+// 1,216 tiles ahead changed nothing.
 template <bool EXT, bool FOUR>
-__device__ __forceinline__ void update_tile(const EngineDev& e, const StepRef& sr, int tile) {
-  __shared__ RegionConst s_rc[kTileRegions];
-  __shared__ uint32_t s_wtot[kUpdThreads / 32];
-  __shared__ uint32_t s_hbase;
-  __shared__ unsigned long long s_rbase;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+__device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& sr, int tile, int warp) {
+  const int lane = threadIdx.x & 31;
   // state loads first: they depend only on the tile, and the arrays cover
   // every padded tile
-  const int64_t gi0 = (int64_t)tile * kTile + threadIdx.x * 4;
+  const int64_t gi0 = (int64_t)tile * kTile + warp * 128 + lane * 4;
   // (state is streamed once per step: evict-first, so that the delivery's
   // working set keeps the L2)
   const float4 V4 = __ldcs(reinterpret_cast<const float4*>(e.V + gi0));
@@ -245,155 +395,48 @@ __device__ __forceinline__ void update_tile(const EngineDev& e, const StepRef& s
 #pragma unroll
   for (int u = 0; u < 4; ++u) J4[u] = __ldcs(reinterpret_cast<const float4*>(e.J + u * e.stride + gi0));
   const uchar4 rf = __ldcs(reinterpret_cast<const uchar4*>(e.ref + gi0));
-  float4 B4 = make_float4(0.f, 0.f, 0.f, 0.f), F4 = make_float4(1.f, 1.f, 1.f, 1.f);
-  if (EXT) {
-    B4 = __ldcs(reinterpret_cast<const float4*>(e.Ibg + gi0));
-    F4 = __ldg(reinterpret_cast<const float4*>(e.fext + gi0));
-  }
-  // this step's arrivals, per channel (AMPA, NMDA, GABA_A, GABA_B) of the
-  // thread's four neurons, from the accumulator slot of this iteration
+  const int4 ti = __ldg(e.tile_info + tile);  // instance, first region, regions touched
+  // this step's arrivals: one int4 per neuron (AMPA, NMDA, GABA_A, GABA_B)
+  // or per two (E, I of each), from the accumulator slot of this iteration
   const unsigned long long g = step_of(sr);
-  int2* const accs = e.acc + (e.acc_slots > 1 ? (size_t)(g % (unsigned long long)e.acc_slots) : 0) *
-                                 (size_t)e.stride * (FOUR ? 2 : 1);
-  int4 A[4];
-  if (FOUR) {
+  constexpr int kA = FOUR ? 4 : 2;
+  int4* const accs = reinterpret_cast<int4*>(acc_of(e, g)) + (FOUR ? gi0 : gi0 / 2);
+  int4 A[kA];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) A[k] = *reinterpret_cast<const int4*>(accs + 2 * gi0 + 2 * k);
-  } else {
-    const int4 a01 = *reinterpret_cast<const int4*>(accs + gi0);
-    const int4 a23 = *reinterpret_cast<const int4*>(accs + gi0 + 2);
-    A[0] = make_int4(a01.x, a01.x, a01.y, a01.y);
-    A[1] = make_int4(a01.z, a01.z, a01.w, a01.w);
-    A[2] = make_int4(a23.x, a23.x, a23.y, a23.y);
-    A[3] = make_int4(a23.z, a23.z, a23.w, a23.w);
-  }
+  for (int k = 0; k < kA; ++k) A[k] = __ldcg(accs + k);
 
-  const int4 ti = e.tile_info[tile];  // instance, first region, regions touched
   if (sr.next && threadIdx.x == 0) *sr.next = g + 1ull;
   if (ti.x < 0) return;  // unused tile
-  const int inst = ti.x, r0 = ti.y, nr = ti.z;
+  const int inst = ti.x, r0 = ti.y;
   const InstDesc& d = e.insts[inst];
   const long long n = (long long)(g - d.g0);
-  const bool active = e.dyn[inst].active != 0 && n < d.n_end;
-  if (nr <= kTileRegions) {
-    const uint32_t* src = reinterpret_cast<const uint32_t*>(d.rc + r0);
-    uint32_t* dst = reinterpret_cast<uint32_t*>(s_rc);
-    const int words = nr * (int)(sizeof(RegionConst) / 4);
-    for (int w = threadIdx.x; w < words; w += blockDim.x) dst[w] = src[w];
-  }
-  __syncthreads();
-  const RegionConst* rcp = nr <= kTileRegions ? s_rc : d.rc + r0;
-
+  if (e.dyn[inst].active == 0 || n >= d.n_end) return;
   const int32_t li0 = (int32_t)(gi0 - d.base);
-  unsigned spk = 0;       // bit k: neuron li0 + k spiked
-  unsigned cls_bits = 0;  // bit k: that neuron is inhibitory
-  int reg[4] = {0, 0, 0, 0};
-
-  if (active && li0 < d.N) {
+  const int m = d.N - li0 < 4 ? d.N - li0 : 4;  // neurons of the thread that exist
+  const RegionConst* rcp = d.rc + r0;
+  QuadConst<true> one{rcp, {0}};
+  QuadConst<false> each{rcp, {0, 0, 0, 0}};
+  QuadSpikes qs;
+  if (m > 0) {
 #pragma unroll
-    for (int k = 0; k < (FOUR ? 4 : 2); ++k)
-      *reinterpret_cast<int4*>(accs + (FOUR ? 2 : 1) * gi0 + 2 * k) = make_int4(0, 0, 0, 0);
-    unsigned long long x[4] = {(unsigned long long)n, (unsigned long long)(li0 >> 2), 0ull, 0ull};
-    philox4x64_10(x, d.seed, d.net_id);
-    float ib[4] = {B4.x, B4.y, B4.z, B4.w};
-    const float fe[4] = {F4.x, F4.y, F4.z, F4.w};
-    unsigned long long xo[4] = {0ull, 0ull, 0ull, 0ull};
-    if (EXT && (d.ext & kExtOU)) {  // the OU noise: stream 4
-      xo[0] = (unsigned long long)n;
-      xo[1] = (unsigned long long)(li0 >> 2);
-      xo[2] = 4ull;
-      philox4x64_10(xo, d.seed, d.net_id);
+    for (int k = 0; k < kA; ++k) accs[k] = make_int4(0, 0, 0, 0);
+    if (ti.z == 1) {  // the whole tile lies in one region
+      qs = quad_step<EXT, FOUR, true>(e, d, one, m, gi0, li0, n, V4, J4, rf, A);
+    } else {
+      int r = 0;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        if (k < m)
+          while (li0 + k >= __ldg(&rcp[r].end)) ++r;
+        each.r[k] = r;
+      }
+      qs = quad_step<EXT, FOUR, false>(e, d, each, m, gi0, li0, n, V4, J4, rf, A);
     }
-
-    float v[4] = {V4.x, V4.y, V4.z, V4.w};
-    float j[4][4] = {{J4[0].x, J4[0].y, J4[0].z, J4[0].w},
-                     {J4[1].x, J4[1].y, J4[1].z, J4[1].w},
-                     {J4[2].x, J4[2].y, J4[2].z, J4[2].w},
-                     {J4[3].x, J4[3].y, J4[3].z, J4[3].w}};
-    int rr[4] = {rf.x, rf.y, rf.z, rf.w};
-    int r = 0;  // relative to r0
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int32_t li = li0 + k;
-      if (li >= d.N) break;
-      while (li >= rcp[r].end) ++r;
-      reg[k] = r0 + r;
-      const RegionConst& p = rcp[r];
-      const float4 G = *reinterpret_cast<const float4*>(p.g);
-      const float4 VU = *reinterpret_cast<const float4*>(p.Vu);
-      const float4 DE = *reinterpret_cast<const float4*>(p.dec);
-      const float4 M = *reinterpret_cast<const float4*>(&p.dtC);     // dtC gL VL Vth
-      const float4 Q = *reinterpret_cast<const float4*>(&p.Vreset);  // Vreset Iext n_ref q_ext
-      const int4 W = *reinterpret_cast<const int4*>(&p.n_thr);       // n_thr exc_end start end
-      // background: Poisson count by integer inversion of 32 Philox bits
-      // (the thresholds are non-decreasing: count them up to the first miss)
-      const uint32_t uu = (uint32_t)(x[k] >> 32);
-      int c = 0;
-      while (c < W.x && uu >= p.thr[c]) ++c;
-      const int dq = c * __float_as_int(Q.w);
-      const int a0 = A[k].x + dq, a1 = A[k].y + dq;  // the drive feeds AMPA and NMDA
-      // membrane with the old V and traces
-      const float vk = v[k];
-      const float gu[4] = {G.x, G.y, G.z, G.w}, vu[4] = {VU.x, VU.y, VU.z, VU.w};
-      float Isyn = 0.0f;
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const float gj = __fmul_rn(gu[u], j[u][k]);
-        const float dv = __fsub_rn(vu[u], vk);
-        Isyn = __fadd_rn(Isyn, __fmul_rn(gj, dv));
-      }
-      const float leak = __fmul_rn(M.y, __fsub_rn(vk, M.z));
-      float I = __fsub_rn(Isyn, leak);
-      float4 OUc = make_float4(0.f, 0.f, 0.f, 0.f);  // mu, dt/tau, sigma sqrt(2 dt/tau), bits
-      if (EXT && d.ext) OUc = *reinterpret_cast<const float4*>(&p.ou_mu);
-      const int xb = __float_as_int(OUc.w);
-      // injected current, scaled by the neuron's factor where heterogeneous
-      const float ie = (EXT && (xb & kExtHet)) ? __fmul_rn(Q.y, fe[k]) : Q.y;
-      I = __fadd_rn(I, ie);
-      if (EXT && (xb & kExtOU)) I = __fadd_rn(I, ib[k]);  // I_bg before this step
-      const float vn = __fadd_rn(vk, __fmul_rn(I, M.x));
-      if (EXT && (xb & kExtOU)) {  // Eq. 1, Euler-Maruyama
-        const float xi = normal_from_word(xo[k]);
-        const float t1 = __fmul_rn(__fsub_rn(OUc.x, ib[k]), OUc.y);
-        ib[k] = __fadd_rn(ib[k], t1);
-        ib[k] = __fadd_rn(ib[k], __fmul_rn(OUc.z, xi));
-      }
-      // traces: decay, then this step's arrivals
-      const float x0 = __fmul_rn(__int2float_rn(a0), d.inv_two_S);
-      const float x1 = FOUR ? __fmul_rn(__int2float_rn(a1), d.inv_two_S) : x0;
-      const float x2 = __fmul_rn(__int2float_rn(A[k].z), d.inv_two_S);
-      const float x3 = FOUR ? __fmul_rn(__int2float_rn(A[k].w), d.inv_two_S) : x2;
-      j[0][k] = __fadd_rn(__fmul_rn(DE.x, j[0][k]), x0);
-      j[1][k] = __fadd_rn(__fmul_rn(DE.y, j[1][k]), x1);
-      j[2][k] = __fadd_rn(__fmul_rn(DE.z, j[2][k]), x2);
-      j[3][k] = __fadd_rn(__fmul_rn(DE.w, j[3][k]), x3);
-      // refractory clamp, threshold, reset
-      if (rr[k] > 0) {
-        v[k] = Q.x;
-        rr[k] -= 1;
-      } else if (vn >= M.w) {
-        v[k] = Q.x;
-        rr[k] = __float_as_int(Q.z);
-        spk |= 1u << k;
-        if (li >= W.y) cls_bits |= 1u << k;
-      } else {
-        v[k] = vn;
-      }
-    }
-    __stcs(reinterpret_cast<float4*>(e.V + gi0), make_float4(v[0], v[1], v[2], v[3]));
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-      __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + gi0),
-             make_float4(j[u][0], j[u][1], j[u][2], j[u][3]));
-    __stcs(reinterpret_cast<uchar4*>(e.ref + gi0),
-           make_uchar4((unsigned char)rr[0], (unsigned char)rr[1], (unsigned char)rr[2],
-                       (unsigned char)rr[3]));
-    if (EXT && (d.ext & kExtOU))
-      __stcs(reinterpret_cast<float4*>(e.Ibg + gi0), make_float4(ib[0], ib[1], ib[2], ib[3]));
   }
+  const unsigned spk = qs.spk, cls_bits = qs.cls;
 
-  // ---- spikes: one ring append, spike and raster count per block ---------
-  if (!__syncthreads_or(spk != 0)) return;
+  // ---- spikes: one ring append, spike and raster count per warp ----------
+  if (!__any_sync(kFull, spk != 0)) return;
   const int nsp = __popc(spk);
   int ps = nsp;
 #pragma unroll
@@ -401,28 +444,23 @@ __device__ __forceinline__ void update_tile(const EngineDev& e, const StepRef& s
     const int t = __shfl_up_sync(kFull, ps, o);
     if (lane >= o) ps += t;
   }
-  if (lane == 31) s_wtot[warp] = (uint32_t)ps;
-  __syncthreads();
   // the ring slot of the step at which these spikes are handed on: this
   // step, or with spike binning the last step of its bin
   const unsigned long long rel =
-      d.bin_sp ? d.g0 + (unsigned long long)((n / d.spb + 1) * d.spb - 1) : g;
-  const int slot = (int)(rel % (unsigned long long)e.D);
-  if (threadIdx.x == 0) {
-    uint32_t tot = 0;
-    for (int w = 0; w < kUpdThreads / 32; ++w) {
-      const uint32_t c = s_wtot[w];
-      s_wtot[w] = tot;  // exclusive prefix
-      tot += c;
-    }
-    s_hbase = atomicAdd(e.hcount + slot, tot);
-    atomicAdd(&e.dyn[inst].spikes, (unsigned long long)tot);
-    s_rbase = d.raster_cap > 0 ? atomicAdd(&e.dyn[inst].raster_count, (unsigned long long)tot) : 0ull;
+      d.bin_sp ? d.g0 + (unsigned long long)((div_steps(n, d.spb) + 1) * d.spb - 1) : g;
+  const int slot = (int)((rel >> 32) ? rel % (unsigned long long)e.D : (uint32_t)rel % (uint32_t)e.D);
+  uint32_t hbase = 0;
+  unsigned long long rbase = 0;
+  if (lane == 31) {
+    hbase = atomicAdd(e.hcount + slot, (uint32_t)ps);
+    atomicAdd(&e.dyn[inst].spikes, (unsigned long long)ps);
+    if (d.raster_cap > 0) rbase = atomicAdd(&e.dyn[inst].raster_count, (unsigned long long)ps);
   }
-  __syncthreads();
+  hbase = __shfl_sync(kFull, hbase, 31);
+  rbase = __shfl_sync(kFull, rbase, 31);
   if (spk) {
-    uint64_t pos = (uint64_t)s_hbase + s_wtot[warp] + (uint32_t)(ps - nsp);
-    unsigned long long rpos = s_rbase + s_wtot[warp] + (unsigned long long)(ps - nsp);
+    uint64_t pos = (uint64_t)hbase + (uint32_t)(ps - nsp);
+    unsigned long long rpos = rbase + (unsigned long long)(ps - nsp);
     uint32_t* hslot = e.hist + (size_t)slot * (size_t)e.hist_cap;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
@@ -432,7 +470,7 @@ __device__ __forceinline__ void update_tile(const EngineDev& e, const StepRef& s
       else
         atomicOr(e.flags, kFlagHistOverflow);
       ++pos;
-      atomicAdd(&e.cnt[d.rbase + reg[k]], 1);
+      atomicAdd(&e.cnt[d.rbase + r0 + each.r[k]], 1);
       if (d.raster_cap > 0) {
         if (rpos < (unsigned long long)d.raster_cap) {
           d.raster_step[rpos] = (int32_t)n;
@@ -445,8 +483,9 @@ __device__ __forceinline__ void update_tile(const EngineDev& e, const StepRef& s
 }
 
 template <bool EXT, bool FOUR>
-__global__ void __launch_bounds__(kUpdThreads, 4) k_update(EngineDev e, StepRef sr) {
-  update_tile<EXT, FOUR>(e, sr, blockIdx.x);
+__global__ void __launch_bounds__(kUpdThreads, 7) k_update(EngineDev e, StepRef sr) {
+  const int w = blockIdx.x * (kUpdThreads / 32) + (threadIdx.x >> 5);
+  update_warp<EXT, FOUR>(e, sr, w / kTileWarps, w % kTileWarps);
 }
 
 __device__ __forceinline__ uint32_t edge_delay(const uint32_t* col, const uint8_t* dl, int shift,
@@ -936,10 +975,8 @@ __global__ void __launch_bounds__(kDelThreads, 2)
     deliver_body<FOUR, SINGLE, true>(e, sr, kPartAll, blockIdx.x, gridDim.x);
     target += gridDim.x;
     if (!grid_barrier(count, target, limit_ns, e.flags)) return;
-    for (int t = blockIdx.x; t < e.n_tiles; t += gridDim.x) {
-      __syncthreads();  // the previous tile's block-shared values are read
-      update_tile<EXT, FOUR>(e, sr, t);
-    }
+    for (int t = blockIdx.x; t < e.n_tiles; t += gridDim.x)
+      update_warp<EXT, FOUR>(e, sr, t, threadIdx.x >> 5);
     target += gridDim.x;
     if (!grid_barrier(count, target, limit_ns, e.flags)) return;
   }
@@ -1084,16 +1121,17 @@ int g_deliver_grid = 0;
 
 void launch_init_state(const EngineDev& e, int inst, int n_tiles_inst, int first_tile,
                        cudaStream_t s) {
-  if (n_tiles_inst > 0) k_init_state<<<n_tiles_inst, kUpdThreads, 0, s>>>(e, inst, first_tile);
+  if (n_tiles_inst > 0) k_init_state<<<n_tiles_inst, kTile / 4, 0, s>>>(e, inst, first_tile);
 }
 
 void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s) {
+  const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads);
   if (e.four) {
-    if (e.any_ext) k_update<true, true><<<e.n_tiles, kUpdThreads, 0, s>>>(e, sr);
-    else k_update<false, true><<<e.n_tiles, kUpdThreads, 0, s>>>(e, sr);
+    if (e.any_ext) k_update<true, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
+    else k_update<false, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
   } else {
-    if (e.any_ext) k_update<true, false><<<e.n_tiles, kUpdThreads, 0, s>>>(e, sr);
-    else k_update<false, false><<<e.n_tiles, kUpdThreads, 0, s>>>(e, sr);
+    if (e.any_ext) k_update<true, false><<<blocks, kUpdThreads, 0, s>>>(e, sr);
+    else k_update<false, false><<<blocks, kUpdThreads, 0, s>>>(e, sr);
   }
 }
 
