@@ -158,7 +158,12 @@ typedef struct {
  *                    hold at most one tile each) -- runs 64 steps timed by
  *                    CUDA events, three times each in turn (after the first
  *                    round those over twice the best drop out), and the
- *                    smallest total is kept.
+ *                    smallest total is kept.  These turns time per-step
+ *                    delivery; an engine that delivers otherwise (see
+ *                    emit_delay) does so before and after them, and one more
+ *                    turn of 64 steps, after the tuning is reported done,
+ *                    keeps it unless the best per-step shape was faster by
+ *                    a tenth.
  *                    Results depend on none of these choices (integer
  *                    accumulation).  Default 2000 (200 ms at dt 0.1 ms, past
  *                    the onset).
@@ -182,7 +187,11 @@ typedef struct {
  *                    it fits a third of the free device memory) and a
  *                    spike's edges of delay >= emit_delay go straight into
  *                    the slot of their arrival step, its short segments read
- *                    in one pass.  -1 (default): none; d >= 1: delays >= d;
+ *                    in one pass.  -1 (default): the engine's own rule --
+ *                    every edge at emission where that ring stays in the L2
+ *                    (48 MB), else in windows of a few steps, a row's edges
+ *                    due in a window read as one segment --; d >= 1: delays
+ *                    >= d at emission, the others in their own step;
  *                    0: the delays from which every (row, delay) segment
  *                    holds fewer than 4 edges on average (estimated from a
  *                    sample of rows at create), kept only if the autotuner
@@ -202,9 +211,11 @@ typedef struct {
  *                    steps in one cooperative launch (the same delivery and
  *                    update device code, separated by grid barriers whose
  *                    waits give up after 1 s with DBNET_ETIMEOUT), which
- *                    saves the two launches per step where a step's kernels
- *                    are short; DBNET_SCHEDULE_AUTO (default): sequential
- *                    until the autotuner times all three.
+ *                    saves the launches where a step's kernels
+ *                    are short; DBNET_SCHEDULE_AUTO (default): by the
+ *                    engine's size, until and after the autotuner times all
+ *                    three (see autotune_at).  The pipelined schedule
+ *                    delivers each delay in its own step.
  *   deliver_blocks   blocks of the delivery grid (>= 2; on the persistent
  *                    schedule at most the co-resident blocks, else
  *                    DBNET_EINVAL at the first step), and the autotuner then
@@ -245,11 +256,12 @@ typedef struct {
   int32_t deliver_blocks;    /* delivery grid in use */
   int32_t autotuned;         /* 1 once the autotuner has chosen that grid */
   int32_t two_weights;       /* 1: four accumulator channels (two weights per edge) */
-  int32_t seg_ring;          /* spikes per step whose segments the delivery reads
-                                from its delay-major ring; a step's later spikes
-                                (and graphs with u32 segment tables) are resolved
-                                from the graph's own tables */
-  int32_t emit_delay;        /* delays >= this are added at emission (0: none) */
+  int32_t seg_ring;          /* spikes per step whose segments per-step delivery
+                                reads from its delay-major ring; a step's later
+                                spikes (and graphs with u32 segment tables) are
+                                resolved from the graph's own tables */
+  int32_t emit_delay;        /* the emission threshold the options asked for
+                                and the engine uses (0: none) */
   int32_t schedule;          /* DBNET_SCHEDULE_SEQUENTIAL, _PIPELINED or
                                 _PERSISTENT: the schedule in use */
 } dbnet_stats_t;

@@ -181,9 +181,10 @@ std::shared_ptr<GraphDev> upload_graph(const dbnet_graph_t* g, cudaStream_t s) {
     }
     gd->emit_from = E > 0 ? from : 0;
   }
-  const int32_t per16 = gd->seg_kind == kSeg16 ? 8 : 4;  // entries per 16 bytes
-  gd->seg_stride = (gd->max_delay + per16 - 1) / per16 * per16;
-  const int64_t seg_bytes = (int64_t)N * gd->seg_stride * (gd->seg_kind == kSeg16 ? 2 : 4);
+  gd->shift = N <= (1 << 24) ? 24 : N <= (1 << 28) ? 28 : 32;  // delay bits of the records
+  const int32_t count_b = gd->seg_kind == kSeg16 ? 2 : 4;
+  gd->seg_bytes = (kSegHead + gd->max_delay * count_b + 15) / 16 * 16;
+  const int64_t seg_bytes = (int64_t)N * gd->seg_bytes;
 
   gd->row_ptr.alloc(N + 1);
   gd->ro.alloc(R + 1);
@@ -217,14 +218,14 @@ std::shared_ptr<GraphDev> upload_graph(const dbnet_graph_t* g, cudaStream_t s) {
       int32_t j1 = j0 + 1;
       while (j1 < N && g->row_ptr[j1 + 1] - g->row_ptr[j0] <= cap) ++j1;
       const int64_t e0 = g->row_ptr[j0], ne = g->row_ptr[j1] - e0;
-      if (ne > 0) {
+      {
         stage.copy(col_st.p, g->col + e0, sizeof(int32_t) * ne);
         stage.copy(d_st.p, g->delay + e0, ne);
         stage.copy(w_st.p, static_cast<const uint8_t*>(g->weight) + e0 * wsz, ne * wsz);
         if (gd->two_w) stage.copy(w2_st.p, static_cast<const uint8_t*>(g->weight2) + e0 * wsz, ne * wsz);
         launch_ingest(N, j0, j1, e0, gd->row_ptr.p, col_st.p, w_st.p,
                       gd->two_w ? w2_st.p : nullptr, g->weight_dtype, d_st.p,
-                      gd->rec.p, gd->max_delay, gd->seg_stride, gd->seg.p, gd->seg_kind, indeg.p,
+                      gd->rec.p, gd->shift, gd->max_delay, gd->seg_bytes, gd->seg.p, gd->seg_kind, indeg.p,
                       scal.p + 0, scal.p + 2, s);
         CK(cudaGetLastError());
       }
@@ -437,7 +438,7 @@ void Engine::init(const std::vector<InstSpec>& specs, void* user_stream) {
   }
   // with spike binning a spike waits up to spb - 1 steps for its bin to end
   init_pool(n, tiles, regions, dmax_all + 1 + bin_lead(specs[0].opt), specs[0].opt, user_stream,
-            any_ext, four, emit_from > dmax_all ? 0 : emit_from);
+            any_ext, four, emit_from > dmax_all ? 0 : emit_from, true);
   int64_t t = 0;
   int32_t r = 0;
   for (int k = 0; k < n; ++k) {
@@ -451,7 +452,7 @@ void Engine::init(const std::vector<InstSpec>& specs, void* user_stream) {
 
 void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D,
                        const dbnet_options_t& common, void* user_stream, bool any_ext,
-                       bool four, int32_t emit_from) {
+                       bool four, int32_t emit_from, bool n_tiles_fixed) {
   if (user_stream) {
     stream = (cudaStream_t)user_stream;
     own_stream = false;
@@ -474,18 +475,53 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   Ibg.alloc(stride);
   fext.alloc(stride);
   ref.alloc(stride);
-  // accumulators: one slot, or a ring of D slots when long delays may be
-  // handed on at emission (and the ring takes at most a third of the free
-  // memory)
+  // which kernel adds a spike's edges, and the accumulator ring it needs
+  dev = EngineDev{};
+  const int32_t lead = bin_lead(common);
+  if (lead >= D - 1) raise(DBNET_EINVAL, "the spike bin is longer than the ring");
+  dev.bin_lead = lead;
+  dev.dmax = D - 1 - lead;
+  size_t free_b = 0, total_b = 0;
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  const double slot_b = (double)stride * (four ? 16.0 : 8.0);
+  auto pow2 = [](int32_t n) {
+    int32_t p = 1;
+    while (p < n) p *= 2;
+    return p;
+  };
   // (two slots at least: the pipelined schedule delivers into step g + 1's
   // slot while the update reads step g's)
   int32_t slots = 2;
+  dev.mode = kPerStep;
+  const int32_t D0 = D;  // ring slots that per-step delivery needs
+  const bool tunes = common.autotune_at >= 0 && !(common.deliver_blocks > 0 && common.schedule != DBNET_SCHEDULE_AUTO);
   if (emit_from > 0) {
-    size_t free_b = 0, total_b = 0;
-    CK(cudaMemGetInfo(&free_b, &total_b));
-    const double ring_b = (double)D * (double)stride * 8.0 * (four ? 2.0 : 1.0);
-    if (ring_b <= (double)free_b / 3.0) slots = D;
+    if (pow2(D) * slot_b <= (double)free_b / 3.0) slots = pow2(D);
     else emit_from = 0;
+  }
+  // (a request server's instances have bins of their own each, so that there
+  // is no step at which its mode could change)
+  if (common.emit_delay < 0 && common.schedule != DBNET_SCHEDULE_PIPELINED && (lead == 0 || n_tiles_fixed)) {
+    // delay bits that every graph of the engine has in its records
+    const int bits = stride <= (int64_t(1) << 24) ? 8 : stride <= (int64_t(1) << 28) ? 4 : 0;
+    auto fits = [&](int32_t n) { return (bits == 8 || n <= (bits == 4 ? 16 : 0)) && n * slot_b <= (double)free_b / 4.0; };
+    // Steps per window: the longer the window the fewer the pieces of rows,
+    // as long as its accumulators stay in the L2 (see k_windows).  Where the
+    // update adds its own spikes' edges (small networks, bound by launches)
+    // the longest; with spike binning, whose ring is a bin longer, four.
+    dev.push_now = tiles <= kPushTiles;
+    int32_t W = dev.push_now ? (lead > 0 ? 4 : kWindow) : 4 * slot_b <= kWindowRingBytes ? 4 : 2;
+    W = std::min(W, pow2(dev.dmax));
+    const int32_t all = pow2(D), win = pow2(W + lead);
+    if (fits(all) && all * slot_b <= kEmitRingBytes) {
+      dev.mode = kAtEmission;
+      slots = all;
+    } else if (fits(win)) {
+      dev.mode = kWindows;
+      dev.wmask = W - 1;
+      slots = win;
+      D = dev.dmax + W + lead;  // a window's slots are cleared before its first update
+    }
   }
   acc.alloc((four ? 2 : 1) * stride * (int64_t)slots);  // int2 per neuron, or int4 with four channels
   // the second stream of the pipelined schedule, ahead of the first
@@ -502,7 +538,7 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   CK(cudaMemsetAsync(J.p, 0, sizeof(float) * 4 * stride, stream));
   CK(cudaMemsetAsync(ref.p, 0, stride, stream));
   CK(cudaMemsetAsync(acc.p, 0, sizeof(int2) * (four ? 2 : 1) * stride * (size_t)slots, stream));
-  if (slots > 1) {
+  if (dev.mode == kPerStep || tunes) {
     slot_emit.alloc(D);
     CK(cudaMemsetAsync(slot_emit.p, 0xFF, sizeof(uint16_t) * D, stream));  // none yet
   }
@@ -511,7 +547,7 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   tile_info.alloc(tiles);
   closed.alloc(regions);
   region_inst.alloc(regions);
-  cnt.alloc(regions);
+  cnt.alloc(2 * (int64_t)regions);
   bw.alloc(4 * (int64_t)regions);
   ylast.alloc(regions);
   CK(cudaMemsetAsync(desc.p, 0, sizeof(InstDesc) * n_inst, stream));
@@ -523,31 +559,45 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   CK(cudaMemcpyAsync(tile_info.p, no_tiles_h.data(), sizeof(int4) * tiles, cudaMemcpyHostToDevice, stream));
   CK(cudaMemsetAsync(region_inst.p, 0xFF, sizeof(int32_t) * regions, stream));  // -1: unused
   CK(cudaMemsetAsync(closed.p, 0, sizeof(long long) * regions, stream));
-  CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * regions, stream));
+  CK(cudaMemsetAsync(cnt.p, 0, sizeof(int32_t) * 2 * regions, stream));
   CK(cudaMemsetAsync(bw.p, 0, sizeof(double) * 4 * regions, stream));
   CK(cudaMemsetAsync(ylast.p, 0, sizeof(double) * regions, stream));
   // spike ring: a slot per step of the longest delay, each able to hold every neuron
-  hist.alloc((int64_t)D * stride);
+  if (dev.mode != kAtEmission || tunes) hist.alloc((int64_t)D * stride);
   hcount.alloc(D);
   CK(cudaMemsetAsync(hcount.p, 0, sizeof(uint32_t) * D, stream));
   // delay-major segment ring: room for seg_cap spikes per step -- a 64th of
   // the neurons (at least 4096), within a sixteenth of the free memory; a
   // step's spikes beyond seg_cap (and instances with u32 tables) take the
   // direct path
-  const int32_t dcap = D - 1;
-  int64_t seg_cap = 0;
-  {
-    size_t free_b = 0, total_b = 0;
+  auto ring = [&](int32_t per, DevBuf<uint16_t>& counts, DevBuf<int64_t>& rows, bool wanted) {
     CK(cudaMemGetInfo(&free_b, &total_b));
     const int64_t budget = (int64_t)(free_b / 16);
-    const int64_t per_spike = (int64_t)D * dcap * 2 + (int64_t)D * 8;
+    const int64_t per_spike = (int64_t)D * per * 2 + (int64_t)D * 8;
     const int64_t want = std::max<int64_t>(4096, stride / 64);
-    seg_cap = std::min<int64_t>(std::min(stride, want), budget / per_spike) / 32 * 32;
-    if (seg_cap < 1024) seg_cap = 0;  // too little room to be worth it
-  }
-  if (seg_cap > 0) {
-    hseg.alloc((int64_t)D * dcap * seg_cap);
-    hr0.alloc((int64_t)D * seg_cap);
+    int64_t cap = std::min<int64_t>(std::min(stride, want), budget / per_spike) / 32 * 32;
+    if (cap < 1024) cap = 0;  // too little room to be worth it
+    if (cap > 0 && wanted) {
+      counts.alloc((int64_t)D * per * cap);
+      rows.alloc((int64_t)D * cap);
+    }
+    return cap;
+  };
+  // per-step delivery (the engine's mode, or while the launch shapes are
+  // tuned) and windows each have a ring of their own
+  Delivery per{kPerStep, 0, 0, 1, D0 - 1, 0, nullptr, nullptr};
+  ring_cap = ring(per.dcap, hseg, hr0, dev.mode == kPerStep || tunes);
+  per.seg_cap = ring_cap;
+  per.hseg = hseg.p;
+  per.hr0 = hr0.p;
+  Delivery fast{dev.mode, dev.wmask, dev.push_now, 1, 0, 0, nullptr, nullptr};
+  if (dev.mode == kWindows) {  // a bound per window and one more
+    fast.dcap = (dev.dmax + dev.wmask) / (dev.wmask + 1) + 1;
+    // (where most items lie beyond the first windows)
+    if (!dev.push_now && dev.dmax > 2 * (dev.wmask + 1) && n_inst <= 65535)
+      fast.seg_cap = ring(fast.dcap, wseg, wr0, true);
+    fast.hseg = wseg.p;
+    fast.hr0 = wr0.p;
   }
   base.alloc(2);
   events.alloc(2);  // [0] events counted by the deliveries, [1] scratch for the pending ones
@@ -556,7 +606,6 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   CK(cudaMemsetAsync(events.p, 0, sizeof(unsigned long long), stream));
   CK(cudaMemsetAsync(flags.p, 0, sizeof(unsigned), stream));
 
-  dev = EngineDev{};
   dev.V = V.p;
   dev.J = J.p;
   dev.Ibg = Ibg.p;
@@ -571,13 +620,14 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
     int dev_id = 0, l2 = 0;
     CK(cudaGetDevice(&dev_id));
     CK(cudaDeviceGetAttribute(&l2, cudaDevAttrL2CacheSize, dev_id));
-    // one accumulator slot larger than a quarter of the L2: deliver in
-    // rank phases, each touching about an eighth of the regions at a time
-    const double slot_b = (double)stride * (four ? 16.0 : 8.0);
-    dev.phases = slot_b > 0.25 * (double)l2 ? 8 : 1;
+    // accumulators (of a window, or one slot) larger than a quarter of the
+    // L2: deliver in rank phases, each touching about an eighth of the
+    // regions at a time
+    per.phases = slot_b > 0.25 * (double)l2 ? 8 : 1;
+    fast.phases = slot_b * (dev.wmask + 1) > 0.25 * (double)l2 ? 8 : 1;
   }
   dev.d_emit = emit_from > 0 ? emit_from : D + 1;
-  dev.slot_emit = slots > 1 ? slot_emit.p : nullptr;
+  dev.slot_emit = slot_emit.p;
   emit_cand = emit_from;
   emit_phase = (emit_from > 0 && common.emit_delay == 0 && common.autotune_at >= 0) ? 0 : 2;
   dev.insts = desc.p;
@@ -585,18 +635,13 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   dev.tile_info = tile_info.p;
   dev.closed = closed.p;
   dev.cnt = cnt.p;
+  dev.cnt_stride = regions;
   dev.bw = bw.p;
   dev.ylast = ylast.p;
   dev.region_inst = region_inst.p;
   dev.hist = hist.p;
   dev.hcount = hcount.p;
   dev.hist_cap = stride;
-  dev.hseg = hseg.p;
-  dev.hr0 = hr0.p;
-  dev.seg_cap = seg_cap;
-  dev.dcap = dcap;
-  dev.bin_lead = bin_lead(common);
-  if (dev.bin_lead >= D - 1) raise(DBNET_EINVAL, "the spike bin is longer than the ring");
   dev.D = D;
   dev.events = events.p;
   dev.flags = flags.p;
@@ -607,7 +652,15 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   total_R = 0;
   del_grid = common.deliver_blocks > 0 ? common.deliver_blocks : deliver_grid();
   pbar.alloc(1);
+  use(per);
   persist_max = persist_max_grid(dev);
+  if (fast.mode != kPerStep) {
+    use(fast);
+    persist_max = std::min(persist_max, persist_max_grid(dev));
+  }
+  dev.since = 0;
+  per_step = per;
+  rule = fast;
   fixed_schedule = common.schedule;
   pipelined = common.schedule == DBNET_SCHEDULE_PIPELINED;
   persistent = common.schedule == DBNET_SCHEDULE_PERSISTENT;
@@ -639,9 +692,12 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
     const size_t n_sched = fixed_schedule == DBNET_SCHEDULE_AUTO ? 3 : 1;
     if (tune_grid.size() * n_sched > 1) {
       tune_ms.assign(3 * tune_grid.size(), 0.0);  // each grid on each schedule
+      tune_last.assign(3 * tune_grid.size(), kDropped);
       tune_pending = true;
     }
   }
+  rule_grid = del_grid;
+  rule_persistent = persistent;
   CK(cudaGetLastError());
 }
 
@@ -652,7 +708,7 @@ void Engine::place(int k, const InstSpec& sp, int32_t first_tile, int32_t rbase,
   if (k < 0 || k >= cap_inst || first_tile < 0 || first_tile + nt > cap_tiles || rbase < 0 ||
       rbase + g.R > cap_R)
     raise(DBNET_EINVAL, "instance placement outside the engine's capacity");
-  if (g.max_delay + dev.bin_lead >= dev.D) raise(DBNET_EINVAL, "a delay is longer than the engine's ring");
+  if (g.max_delay > dev.dmax) raise(DBNET_EINVAL, "a delay is longer than the engine's ring");
   if (bin_lead(sp.opt) != dev.bin_lead) raise(DBNET_EINVAL, "spike binning differs from the engine's");
   if (g.two_w && !dev.four)
     raise(DBNET_EUNSUPPORTED, "two weights per edge need an engine with four accumulator channels");
@@ -687,7 +743,7 @@ void Engine::place(int k, const InstSpec& sp, int32_t first_tile, int32_t rbase,
   d.seg = g.seg.p;
   d.seg_kind = g.seg_kind;
   d.dmax = g.max_delay;
-  d.seg_stride = g.seg_stride;
+  d.seg_bytes = g.seg_bytes;
   for (const auto& p : sp.params) d.ext |= ext_bits(p);
   if (d.ext && !dev.any_ext)
     raise(DBNET_EUNSUPPORTED, "this engine was built without the OU current or injected-current factors");
@@ -706,8 +762,8 @@ void Engine::place(int k, const InstSpec& sp, int32_t first_tile, int32_t rbase,
   d.N = g.N;
   d.R = g.R;
   d.rbase = rbase;
-  d.shift = 32;
-  d.tmask = 0xFFFFFFFFu;
+  d.shift = g.shift;
+  d.tmask = g.shift < 32 ? (1u << g.shift) - 1u : 0xFFFFFFFFu;
   d.two_S = std::ldexp(1.0f, S);
   d.inv_two_S = std::ldexp(1.0f, -S);
   d.spb = (int32_t)std::lrint(o.bin_ms / o.dt_ms);
@@ -746,7 +802,8 @@ void Engine::place(int k, const InstSpec& sp, int32_t first_tile, int32_t rbase,
                      cudaMemcpyHostToDevice, stream));
   CK(cudaMemcpyAsync(bw.p + 4 * (int64_t)rbase, ih.stage_bw.data(), sizeof(double) * 4 * g.R,
                      cudaMemcpyHostToDevice, stream));
-  CK(cudaMemsetAsync(cnt.p + rbase, 0, sizeof(int32_t) * g.R, stream));
+  for (int k2 = 0; k2 < 2; ++k2)
+    CK(cudaMemsetAsync(cnt.p + (int64_t)k2 * cap_R + rbase, 0, sizeof(int32_t) * g.R, stream));
   CK(cudaMemsetAsync(ylast.p + rbase, 0, sizeof(double) * g.R, stream));
   CK(cudaMemsetAsync(closed.p + rbase, 0, sizeof(long long) * g.R, stream));
   launch_init_state(dev, k, nt, first_tile, stream);
@@ -816,7 +873,8 @@ void Engine::check() const {
 // kChunk steps in two halves: the first half finds its iteration at
 // base[0] + i and its last update writes base[1]; the second half reads
 // base[1] and its last update writes base[0] for the next replay.
-// kChunk steps.  Sequential: delivery then update, per step.  Pipelined:
+// Sequential: the delivery the mode has, then the update, per step (windows:
+// replays start at a window's first step).  Pipelined:
 // the short part of step g's delivery, then step g's update beside the long
 // part of step g + 1's delivery (a fork onto the second stream and a join),
 // so that the latency-bound delivery runs under the bandwidth-bound update;
@@ -831,7 +889,9 @@ void Engine::capture() {
     const StepRef rd{base.p + h, (unsigned long long)off, nullptr};
     const StepRef ru{base.p + h, (unsigned long long)off, off == half - 1 ? base.p + (1 - h) : nullptr};
     if (!pipelined) {
-      launch_deliver(dev, del_grid, rd, stream);
+      if (dev.mode == kPerStep) launch_deliver(dev, del_grid, rd, stream);
+      if (dev.mode == kWindows && ((i & dev.wmask) == 0 || !dev.push_now))
+        launch_windows(dev, del_grid, rd, (i & dev.wmask) == 0, stream);
       launch_update(dev, ru, stream);
       continue;
     }
@@ -861,11 +921,18 @@ void Engine::step(int64_t n) {
       n -= tune_emit(n);
       continue;
     }
-    if (tune_pending && g_host >= tune_at) {  // then the grid
+    if (tune_pending && g_host >= tune_at && (dev.mode == kPerStep || (n >= kChunk && may_switch()))) {  // then the grid
+      if (dev.mode != kPerStep) to_per_step();
       n -= tune_steps(n);
       continue;
     }
-    const int64_t k = (tune_pending || emit_pending) ? std::min<int64_t>(n, (int64_t)(tune_at - g_host)) : n;
+    if (weigh_rule) {  // and whether the best of them beats the mode the rule chose
+      n -= weigh_steps(n);
+      continue;
+    }
+    int64_t k = n;
+    if ((tune_pending || emit_pending) && g_host < tune_at) k = std::min<int64_t>(n, (int64_t)(tune_at - g_host));
+    else if (tune_pending && n >= kChunk) k = 1;  // to the start of a window
     run_plain(k);
     n -= k;
   }
@@ -960,6 +1027,7 @@ int64_t Engine::tune_steps(int64_t n) {
   float ms = 0.0f;
   CK(cudaEventElapsedTime(&ms, tune_ev[0], tune_ev[1]));
   tune_ms[(size_t)c] += ms;
+  tune_last[(size_t)c] = ms;
   finish_turn(C);
   return kChunk;
 }
@@ -976,8 +1044,93 @@ void Engine::finish_turn(int C) {
     if (tune_ms[(size_t)k] < tune_ms[(size_t)best]) best = k;
   set_shape(tune_grid[(size_t)(best / 3)], best % 3);
   tune_pending = false;
+  weigh_rule = rule.mode != kPerStep;
 }
 
+void Engine::use(const Delivery& m) {
+  dev.mode = m.mode;
+  dev.wmask = m.wmask;
+  dev.push_now = m.push_now;
+  dev.phases = m.phases;
+  dev.dcap = m.dcap;
+  dev.seg_cap = m.seg_cap;
+  dev.hseg = m.hseg;
+  dev.hr0 = m.hr0;
+  dev.since = g_host > 0 ? g_host - 1ull : 0ull;  // what this mode counts and copies itself
+  drop_graph();
+}
+
+void Engine::drop_graph() {
+  if (!gexec) return;
+  CK(cudaStreamSynchronize(stream));
+  CK(cudaGraphExecDestroy(gexec));
+  gexec = nullptr;
+}
+
+// The mode may change before step g_host: a window starts there, and no
+// earlier spike waits for the end of its bin.
+bool Engine::may_switch() const {
+  return !long_pending && (g_host & (unsigned long long)rule.wmask) == 0ull &&
+         g_host % (unsigned long long)(dev.bin_lead + 1) == 0ull;
+}
+
+// From the rule's mode to per-step delivery (where the mode may change).
+void Engine::to_per_step() {
+  if (dev.mode == kAtEmission) {  // its ring lists no spikes
+    CK(cudaMemsetAsync(hcount.p, 0, sizeof(uint32_t) * dev.D, stream));
+  } else if (dev.seg_cap == 0) {  // the last window's spikes but the newest, which k_deliver counts
+    const long long from = (long long)g_host - dev.wmask - 1;
+    launch_count_events(dev, std::max<long long>(from, (long long)dev.since), (long long)g_host - 2, events.p, stream);
+  }
+  use(per_step);
+  persistent = fixed_schedule == DBNET_SCHEDULE_PERSISTENT;
+}
+
+// From per-step delivery to the rule's mode (where the mode may change).
+void Engine::to_rule() {
+  if (rule.mode == kAtEmission && g_host > 0) {
+    launch_hand_over(dev, deliver_grid(), g_host, stream);
+    CK(cudaMemsetAsync(hcount.p, 0, sizeof(uint32_t) * dev.D, stream));
+  }
+  use(rule);
+  del_grid = rule_grid;
+  pipelined = false;
+  persistent = rule_persistent;
+}
+
+// The tuner's last turn: one chunk of the rule's mode against the chosen
+// per-step shape's last one (the activity grows over the first rounds); the
+// rule's mode stays unless that was faster by a tenth.
+int64_t Engine::weigh_steps(int64_t n) {
+  if (dev.mode == kPerStep) {
+    if (!may_switch()) {
+      direct_step();
+      return 1;
+    }
+    best_shape = {del_grid, persistent ? 2 : pipelined ? 1 : 0};
+    for (size_t i = 0; i < tune_grid.size(); ++i)
+      if (tune_grid[i] == del_grid) best_ms = tune_last[3 * i + (size_t)best_shape.sched];
+    to_rule();
+  }
+  if (n < kChunk || !aligned()) {
+    const int64_t k = n < kChunk ? n : 1;
+    run_plain(k);
+    return k;
+  }
+  if (!gexec && !persistent) capture();
+  CK(cudaEventRecord(tune_ev[0], stream));
+  run_plain(kChunk);
+  CK(cudaEventRecord(tune_ev[1], stream));
+  CK(cudaEventSynchronize(tune_ev[1]));
+  float ms = 0.0f;
+  CK(cudaEventElapsedTime(&ms, tune_ev[0], tune_ev[1]));
+  weigh_rule = false;
+  if ((double)ms > 1.1 * best_ms && may_switch()) {
+    to_per_step();
+    set_shape(best_shape.grid, best_shape.sched);
+  }
+  return kChunk;
+}
 
 
 void Engine::set_shape(int grid, int sched) {
@@ -1008,7 +1161,8 @@ void Engine::run_plain(int64_t n) {
     }
     return;
   }
-  if (n >= kChunk && !pipelined && long_pending) {  // the pending long part first
+  // the pending long part, or the rest of a window, first
+  while (n >= kChunk && ((!pipelined && long_pending) || !aligned())) {
     direct_step();
     --n;
   }
@@ -1027,13 +1181,24 @@ void Engine::run_plain(int64_t n) {
   for (; n > 0; --n) direct_step();
 }
 
-// One step by direct launches: the delivery (only its short part when the
-// long part is already enqueued), then the update.
-void Engine::direct_step() {
+// A captured chunk may start here: at the first step of a window.
+bool Engine::aligned() const {
+  return dev.mode != kWindows || (g_host & (unsigned long long)dev.wmask) == 0ull;
+}
+
+// The delivery of step g_host, where its mode has one (only the short part
+// when the long part is already enqueued).
+void Engine::direct_delivery() {
   const StepRef sr{nullptr, g_host, nullptr};
-  launch_deliver(dev, del_grid, sr, stream, long_pending ? kPartShort : kPartAll);
-  launch_update(dev, sr, stream);
+  if (dev.mode == kPerStep) launch_deliver(dev, del_grid, sr, stream, long_pending ? kPartShort : kPartAll);
+  if (dev.mode == kWindows && (aligned() || !dev.push_now)) launch_windows(dev, del_grid, sr, aligned(), stream);
   long_pending = false;
+}
+
+// One step by direct launches.
+void Engine::direct_step() {
+  direct_delivery();
+  launch_update(dev, StepRef{nullptr, g_host, nullptr}, stream);
   ++g_host;
 }
 
@@ -1050,8 +1215,7 @@ void Engine::step_timed(int64_t n, double* ms) {
       for (int i = 0; i < b; ++i, ++g_host) {
         const StepRef sr{nullptr, g_host, nullptr};
         CK(cudaEventRecord(ev[3 * i], stream));
-        launch_deliver(dev, del_grid, sr, stream, long_pending ? kPartShort : kPartAll);
-        long_pending = false;
+        direct_delivery();
         CK(cudaEventRecord(ev[3 * i + 1], stream));
         launch_update(dev, sr, stream);
         CK(cudaEventRecord(ev[3 * i + 2], stream));
@@ -1418,7 +1582,7 @@ int dbnet_stats(dbnet_t* h, dbnet_stats_t* out) {
     out->packed_edges = ih.graph->packed ? 1 : 0;
     out->weights_rounded = ih.graph->rounded ? 1 : 0;
     out->deliver_blocks = e.del_grid;
-    out->seg_ring = ih.graph->seg_kind == kSeg16 ? (int32_t)e.dev.seg_cap : 0;
+    out->seg_ring = ih.graph->seg_kind == kSeg16 ? (int32_t)e.ring_cap : 0;
     out->emit_delay = e.dev.d_emit <= e.dev.D ? e.dev.d_emit : 0;
     out->schedule = e.persistent ? DBNET_SCHEDULE_PERSISTENT
                    : e.pipelined ? DBNET_SCHEDULE_PIPELINED : DBNET_SCHEDULE_SEQUENTIAL;

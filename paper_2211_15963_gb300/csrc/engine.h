@@ -13,31 +13,50 @@
 //   or, in an engine with four channels, acc[2i], acc[2i+1] (AMPA, NMDA |
 //   GABA_A, GABA_B: one int4 per neuron)
 // Edges of an instance (CSR by source, rows sorted by delay), either
-//   rec[3e], rec[3e+1], rec[3e+2] u16 = target low, target high, BF16 weight
+//   rec[3e], rec[3e+1], rec[3e+2] u16 = word low, word high, BF16 weight
 //     (interleaved 6-byte records: a short segment is one contiguous read), or,
-//   with two weights per edge, rec[4e .. 4e+3] u16 = target low, target high,
+//   with two weights per edge, rec[4e .. 4e+3] u16 = word low, word high,
 //     BF16 weight, BF16 second weight (8-byte records, one load each), or,
 //   for graphs the caller keeps (the allocation-free entry point), arrays
 //   col[e] u32 = target, w[e] u16 BF16 bit pattern, delay[e] u8
-//   seg[j * seg_stride + k] u16/u32 = number of edges of row j with
-//                       delay <= k + 1, k < dmax (the per-delay segment
-//                       table; seg_stride pads rows to 16 bytes)
-// Iteration g of an engine runs k_deliver then k_update; the bin that ends
-// with iteration g - 1 is closed (Balloon-Windkessel step, BOLD sample) at
-// the start of k_deliver(g), one region per thread.
-// Spike ring: D slots; slot n mod D lists the spikes handed on at step n
-//   (their own step, or the last step of their bin with spike binning) as
-//   global index | class << 31, with a count per slot.  At step n the
-//   delivery reads slots n - d (d = 1..D-1) and applies, for each listed
-//   spike, the segment of its row whose delay is exactly d (arrival time).
-// Long delays at emission: when d_emit <= the longest delay, the
-//   accumulators form a ring of D slots (slot a mod D collects the arrivals
-//   of step a); at step n the delivery adds, for every spike handed on at
-//   step n - 1, its edges of delay d >= d_emit straight into slot n - 1 + d,
-//   each (spike, delay) segment read as it lies in the row, so that the
-//   short segments of long delays cost one coalesced pass instead of one
-//   resolution each; arrival time keeps the delays below d_emit.  The
-//   update of step n reads and clears slot n.
+//   A record's word holds the target in its low `shift` bits and the delay
+//   above them: the whole delay when the graph has at most 2^24 neurons
+//   (shift 24), its low four bits up to 2^28 (shift 28), none beyond.
+//   The segment table: row j, of seg_bytes (a multiple of 16), holds the
+//   row's first and last edge (two int64) and, for k < dmax, the number of
+//   its edges with delay <= k + 1 (u16, or u32 for rows of 65,536 edges on).
+// The accumulators are a ring of acc_slots (a power of two): slot a mod
+// acc_slots collects the arrivals of step a, and the update of step a reads
+// and clears it.  A spike handed on at step s reaches the target of an edge
+// of delay d at step s + d; which kernel adds the edge is the engine's mode:
+//   kAtEmission  the update that emits a spike adds its whole row.  No spike
+//                ring, one launch per step.
+//   kWindows     steps go in windows of W = wmask + 1 (aligned to multiples
+//                of W).  The update that emits a spike adds the edges that
+//                come due inside the window in which it is handed on -- the
+//                start of its row --, and k_windows, before the first update
+//                of a window, adds for every spike handed on earlier the
+//                edges due in the window: one contiguous segment of W delays
+//                of its row.
+//   kPerStep     k_deliver, before every update, adds the edges due in that
+//                step, one segment of one delay per spike and step (the
+//                pipelined schedule, explicit emission thresholds, and
+//                graphs of more than 2^28 neurons).
+// Iteration g runs [k_windows or k_deliver,] k_update; the bin that ends
+// with iteration g - 1 is closed (Balloon-Windkessel step, BOLD sample) by
+// the first blocks of k_update(g), one region per thread; bins count into
+// two sets of region counters in turn.
+// An engine may change between kPerStep and another mode at the start of a
+// window: arrivals before that step are in the accumulators, later ones are
+// not (kAtEmission: they are, or are handed over at once).
+// Spike ring (not kAtEmission): D slots; slot n mod D lists the spikes
+//   handed on at step n (their own step, or the last step of their bin with
+//   spike binning) as global index | class << 31, with a count per slot.
+// kPerStep only:
+// Long delays at emission: when d_emit <= the longest delay, k_deliver(n)
+//   adds, for every spike handed on at step n - 1, its edges of delay d >=
+//   d_emit straight into the slot of step n - 1 + d; arrival time keeps the
+//   delays below d_emit.
 // Delay-major segment ring (u16 tables only): k_deliver(n) copies, for the
 //   first seg_cap spikes of step n - 1, the row start into hr0[slot][k] and
 //   the row's segment counts into hseg[slot][d][k] (d < dcap), so that the
@@ -112,13 +131,15 @@ enum : int32_t {
   kSeg32 = 2,
 };
 
+constexpr int kSegHead = 16;  // bytes before a segment-table row's counts
+
 struct alignas(16) InstDesc {
   const int64_t* row_ptr;
   const uint16_t* rec;           // interleaved records, or nullptr for col/w/delay
   const uint32_t* col;
   const uint16_t* w;
   const uint8_t* delay;          // col/w/delay: caller-held arrays (allocation-free runs)
-  const void* seg;               // [N][seg_stride] segment table, or nullptr
+  const void* seg;               // [N][seg_bytes] segment table, or nullptr
   const int32_t* region_offsets; // [R+1], local
   const RegionConst* rc;         // [R]
   double* bold;                  // [bold_cap][R]
@@ -130,11 +151,11 @@ struct alignas(16) InstDesc {
   uint64_t seed, net_id;
   unsigned long long g0;         // engine iteration at which this instance's step 0 ran
   long long n_end;               // steps it runs: later iterations leave it unchanged
-  int32_t N, R, rbase, shift;    // shift, tmask: the col/w/delay form (targets col & tmask)
+  int32_t N, R, rbase, shift;    // an edge word: target = word & tmask, delay = word >> shift
   uint32_t tmask;
   float two_S, inv_two_S;
   int32_t spb, bins_per_tr;
-  int32_t seg_kind, dmax, seg_stride, ext;  // ext: kExt* bits of any region
+  int32_t seg_kind, dmax, seg_bytes, ext;  // ext: kExt* bits of any region
   int32_t two_w, bin_sp;         // two_w: 8-byte records with a second weight; bin_sp:
                                  //   spikes handed on at the end of their bin
   double h_bw, z_scale, kappa, gamma, tau, alpha, rho, V0;
@@ -162,6 +183,9 @@ enum : unsigned {
   kFlagTimeout = 2u,       // a grid barrier of the persistent stepper gave up waiting
 };
 
+// Which kernel adds a spike's edges (see above).
+enum : int32_t { kPerStep = 0, kWindows = 1, kAtEmission = 2 };
+
 struct EngineDev {
   float* V;
   float* J;
@@ -170,7 +194,14 @@ struct EngineDev {
   uint8_t* ref;
   int2* acc;             // [acc_slots][stride] (int2, or int4 with four channels)
   int64_t stride;
-  int32_t acc_slots;     // 1, or D when long delays are handed on at emission
+  int32_t acc_slots;     // a power of two
+  int32_t mode;          // kPerStep, kWindows or kAtEmission
+  int32_t wmask;         // kWindows: steps per window - 1 (a power of two less one)
+  int32_t push_now;      // kWindows: the update adds its spikes' edges due in the window
+  int32_t keep_counts;   // k_windows leaves the ring's counts alone (handing over, see below)
+  unsigned long long since;  // spikes handed on at earlier steps were counted, and are
+                         //   missing from the segment ring, for they came in another mode
+  int32_t dmax;          // longest delay the rings hold
   int32_t d_emit;        // delays >= d_emit are added at emission into the slot
                          //   of their arrival step (D + 1: none)
   uint16_t* slot_emit;   // [D] d_emit in force when each ring slot's spikes were
@@ -178,7 +209,8 @@ struct EngineDev {
   const InstDesc* insts;
   InstDyn* dyn;
   const int4* tile_info;  // per tile: instance, first region (local), regions touched, 0
-  int32_t* cnt;          // [total_R] spikes in the current bin
+  int32_t* cnt;          // [2][cnt_stride] spikes in the bins of even and odd index
+  int32_t cnt_stride;
   double* bw;            // [total_R][4]
   double* ylast;         // [total_R]
   const int32_t* region_inst;
@@ -206,6 +238,9 @@ void launch_init_state(const EngineDev& e, int inst, int n_tiles_inst, int first
 void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s);
 enum : int { kPartAll = 0, kPartLong = 1, kPartShort = 2 };  // see k_deliver
 void launch_deliver(const EngineDev& e, int grid, StepRef sr, cudaStream_t s, int part = kPartAll);
+// kWindows: the arrivals of the window that starts with the iteration sr names
+// (first), or what the previous step's spikes add to the rest of a window
+void launch_windows(const EngineDev& e, int grid, StepRef sr, bool first, cudaStream_t s);
 // closes the bin that ends with iteration g - 1 (if any) for every region
 void launch_close(const EngineDev& e, unsigned long long g, cudaStream_t s);
 void launch_set_base(unsigned long long* base, unsigned long long g, cudaStream_t s);
@@ -226,12 +261,18 @@ cudaError_t launch_barrier_probe(int grid, unsigned extra, int rounds, unsigned 
                                  unsigned* count, unsigned* flags, cudaStream_t s);
 void launch_ingest(int32_t N, int32_t j0, int32_t j1, int64_t e_base, const int64_t* row_ptr,
                    const int32_t* col_in, const void* w_in, const void* w2_in, int32_t w_dtype,
-                   const uint8_t* delay_in, uint16_t* rec, int32_t dmax, int32_t seg_stride,
-                   void* seg, int32_t seg_kind, int32_t* indeg, unsigned* wmax_bits, unsigned* err,
-                   cudaStream_t s);
+                   const uint8_t* delay_in, uint16_t* rec, int32_t shift, int32_t dmax,
+                   int32_t seg_bytes, void* seg, int32_t seg_kind, int32_t* indeg,
+                   unsigned* wmax_bits, unsigned* err, cudaStream_t s);
+// the spike ring's arrivals from iteration g on, all at once (the engine's
+// accumulator ring must hold every delay): from kPerStep to kAtEmission
+void launch_hand_over(const EngineDev& e, int grid, unsigned long long g, cudaStream_t s);
+// the out-degrees of the spikes handed on at steps r0 .. r1 into *out
+void launch_count_events(const EngineDev& e, long long r0, long long r1, unsigned long long* out, cudaStream_t s);
 void launch_max_reduce(const int32_t* a, int64_t n, unsigned* out, cudaStream_t s);
-// adds to *out the out-degrees of the spikes handed on at steps g - 1 ..
-// g - 1 + bin_lead, which no delivery has counted yet
+// adds to *out the out-degrees of the spikes that no delivery has counted
+// yet: those handed on from the start of the last window (kPerStep: at step
+// g - 1) to step g - 1 + bin_lead; none when they are counted at emission
 void launch_pending_events(const EngineDev& e, unsigned long long g, unsigned long long* out,
                            cudaStream_t s);
 

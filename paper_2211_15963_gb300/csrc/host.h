@@ -183,11 +183,12 @@ struct GraphDev {
   int64_t E = 0;
   std::vector<int32_t> ro_h, nexc_h;
   DevBuf<int64_t> row_ptr;
-  DevBuf<uint16_t> rec;  // [3E] interleaved (target lo, target hi, BF16 weight),
+  DevBuf<uint16_t> rec;  // [3E] interleaved (word lo, word hi, BF16 weight),
                          // or [4E] with a second BF16 weight per edge
   DevBuf<int32_t> ro;
-  DevBuf<uint8_t> seg;  // [N][seg_stride] u16 or u32 segment table
-  int32_t seg_kind = 0, seg_stride = 0;
+  DevBuf<uint8_t> seg;  // [N][seg_bytes] segment table with u16 or u32 counts
+  int32_t seg_kind = 0, seg_bytes = 0;
+  int32_t shift = 24;  // where a record's delay bits start (engine.h)
   bool packed = true;  // edges held as interleaved records
   bool rounded = false;
   bool two_w = false;  // a second weight per edge (8-byte records)
@@ -225,8 +226,30 @@ struct InstHost {
   InstDyn stage_dyn{};
 };
 
+// How an engine adds a spike's edges: the mode's fields of EngineDev.
+struct Delivery {
+  int32_t mode, wmask, push_now, phases, dcap;
+  int64_t seg_cap;
+  uint16_t* hseg;
+  int64_t* hr0;
+};
+
 struct Engine {
   static constexpr int kChunk = 64;
+  // Most steps per delivery window (a power of two that divides kChunk / 2).
+  static constexpr int kWindow = 8;
+  // The accumulator ring up to which every edge is added at emission: it
+  // stays in the L2 beside the state (one kernel a step: 7.8 against 13.2 us
+  // a step at 10,000 neurons, 12.4 against 16.6 at 30,000).
+  static constexpr double kEmitRingBytes = 48.0 * 1048576.0;
+  // A window's accumulators up to which it is four steps long (half the L2).
+  static constexpr double kWindowRingBytes = 64.0 * 1048576.0;
+  // Tiles up to which the update adds its own spikes' edges due in the window
+  // (a separate kernel else): while all its blocks are resident at once, the
+  // few warps that stay for their spikes delay no other.  Inside / outside
+  // measured 11.7 / 13.6 us a step at 150,000 neurons and 12.1 / 14.4 at
+  // 300,000; 38.5 / 26.5 us for the update alone at 2 M.
+  static constexpr int kPushTiles = 532;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   std::vector<InstHost> inst;
@@ -241,8 +264,9 @@ struct Engine {
   DevBuf<long long> closed;
   DevBuf<double> bw, ylast;
   DevBuf<uint32_t> hist, hcount;
-  DevBuf<uint16_t> hseg;
-  DevBuf<int64_t> hr0;
+  DevBuf<uint16_t> hseg, wseg;  // segment rings of per-step delivery and of windows
+  DevBuf<int64_t> hr0, wr0;
+  int64_t ring_cap = 0;  // spikes per step that the segment ring holds, where the mode has one
   DevBuf<unsigned long long> base, events;  // base: the two graph-half iteration words
   DevBuf<unsigned> flags;
   unsigned long long g_host = 0;            // iterations enqueued so far
@@ -257,8 +281,26 @@ struct Engine {
   bool tune_pending = false;
   unsigned long long tune_at = 0;
   int tune_done = 0;                  // steps timed so far
+  // The mode that a rule on the engine's size chose (kPerStep: none), in
+  // which it runs but for the tuner's turns, which time per-step delivery;
+  // a last turn weighs the best of those against it.
+  Delivery rule{}, per_step{};
+  int rule_grid = 0;
+  bool rule_persistent = false;
+  bool weigh_rule = false;
+  double best_ms = kDropped;          // the best per-step shape's last turn
+  struct Shape {
+    int grid, sched;
+  } best_shape{};
+  void use(const Delivery& m);
+  void drop_graph();
+  bool may_switch() const;
+  void to_per_step();
+  void to_rule();
+  int64_t weigh_steps(int64_t n);
   std::vector<int> tune_grid;         // candidates
   std::vector<double> tune_ms;        // chunk time per candidate (grid-major, schedule)
+  std::vector<double> tune_last;      // of its latest turn
   cudaEvent_t tune_ev[2] = {nullptr, nullptr};
   // pipelined schedule: the long part of step g + 1's delivery beside step
   // g's update on a second stream; long_pending: that part of step g_host is
@@ -277,6 +319,8 @@ struct Engine {
   int persist_max = 0;
   bool persist_tunable = false;  // the tuner may weigh the persistent schedule
   DevBuf<unsigned> pbar;
+  bool aligned() const;
+  void direct_delivery();
   void direct_step();
   // sched: 0 sequential, 1 pipelined, 2 persistent
   void set_shape(int grid, int sched);
@@ -311,10 +355,11 @@ struct Engine {
   // per-neuron injected-current factors; four: four accumulator channels
   // per neuron, so that instances may carry two weights per edge.
   // emit_from: delays >= it may be handed on at emission (0: never; the
-  // accumulators then have one slot).
+  // accumulators then have one slot).  n_tiles_fixed: every tile is placed
+  // before the first step and stays.
   void init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D,
                  const dbnet_options_t& common, void* user_stream, bool any_ext,
-                 bool four = false, int32_t emit_from = 0);
+                 bool four = false, int32_t emit_from = 0, bool n_tiles_fixed = false);
   int64_t tune_emit(int64_t n);
   // Put instance k on tiles [first_tile, +tiles of its graph) and region
   // slots [rbase, +R): its constants, buffers and initial state; its step 0

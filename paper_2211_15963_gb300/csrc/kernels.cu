@@ -9,25 +9,22 @@
 //              injected-current factors; k_update<., true> reads four
 //              accumulator channels (two weights per edge) instead of the
 //              two classes.
-//   k_close / the head of k_deliver: the per-bin Balloon-Windkessel step
-//              (Extended Data Table 4) and the BOLD sample, one region per
-//              thread.
-//   k_deliver  push delivery (Supplementary Algorithm 2) at arrival time: for
-//              every spike of step n - d (d = 1..D-1, from the spike ring)
-//              the edges of its row with delay exactly d -- one contiguous
-//              segment, read from the delay-major segment ring that the
-//              leading blocks fill for the previous step's spikes (or from
-//              the graph's segment table) -- are added to this step's
-//              fixed-point accumulators, the warp's segments laid end to end
-//              so that consecutive lanes read consecutive edge records;
-//              k_deliver<true> adds an edge's two weights to the channel pair
-//              of the source's class with one 64-bit atomic.
+//   k_close / the first blocks of k_update: the per-bin Balloon-Windkessel
+//              step (Extended Data Table 4) and the BOLD sample, one region
+//              per thread.
+//   push delivery (Supplementary Algorithm 2) into the ring of fixed-point
+//              accumulators, by the engine's mode (engine.h): k_update adds
+//              the edges of the spikes it emits that come due soon (or all),
+//              k_windows those of earlier spikes due in the next few steps,
+//              k_deliver those due in one step.  In each, a warp lays the
+//              segments of its 32 spikes end to end so that consecutive lanes
+//              read consecutive edge records; with two weights per edge an
+//              edge adds both to the channel pair of the source's class with
+//              one 64-bit atomic.
 //
-// Both kernels find their iteration through a StepRef (a base word in device
-// memory plus an offset), so a captured CUDA graph of (deliver, update) pairs
-// is valid for any step.  The bin that ends with an iteration is closed (BW
-// step, BOLD sample) by the next k_deliver, or by k_close at the end of a
-// step call.
+// The kernels find their iteration through a StepRef (a base word in device
+// memory plus an offset), so a captured CUDA graph of steps is valid for any
+// aligned step.
 //
 // The FP32 neuron arithmetic is written with explicit round-to-nearest
 // intrinsics in a fixed order so that no operation is fused or reordered; the
@@ -196,8 +193,9 @@ __device__ void close_region(const EngineDev& e, int gr, unsigned long long g) {
   if (e.closed[gr] >= (long long)g) return;
   const int r = gr - dk.rbase;
   const double nr = (double)(dk.rc[r].end - dk.rc[r].start);
-  const double z = dk.z_scale * (double)e.cnt[gr] / nr;
-  e.cnt[gr] = 0;
+  int32_t* const cnt = e.cnt + ((nk / dk.spb) & 1) * e.cnt_stride + gr;  // that bin's
+  const double z = dk.z_scale * (double)*cnt / nr;
+  *cnt = 0;
   const double y = bw_euler(e.bw + 4 * gr, z, dk);
   e.ylast[gr] = y;
   const long long b = (nk + 1) / dk.spb;  // bins completed
@@ -223,17 +221,156 @@ __device__ __forceinline__ float normal_from_word(unsigned long long w) {
   return sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
 }
 
-// Where an iteration's accumulators lie: slot a mod acc_slots (one slot, two,
-// or the emission ring).
+// Where an iteration's accumulators lie.
 __device__ __forceinline__ int2* acc_of(const EngineDev& e, unsigned long long g) {
-  const unsigned n = (unsigned)e.acc_slots;
-  const unsigned slot = n <= 2u ? (unsigned)g & (n - 1u) : (unsigned)(g % (unsigned long long)n);
-  return e.acc + (size_t)slot * (size_t)e.stride * (e.four ? 2 : 1);
+  return e.acc + (size_t)((unsigned)g & (unsigned)(e.acc_slots - 1)) * (size_t)e.stride * (e.four ? 2 : 1);
 }
 
 // a / b for step counts: in 32 bits while they fit
 __device__ __forceinline__ long long div_steps(long long a, int b) {
   return (unsigned long long)a >> 32 ? a / b : (long long)((uint32_t)a / (uint32_t)b);
+}
+
+__device__ __forceinline__ uint32_t edge_delay(const uint32_t* col, const uint8_t* dl, int shift,
+                                               int64_t e) {
+  return dl ? (uint32_t)__ldg(dl + e) : (__ldg(col + e) >> shift);
+}
+
+// first edge in [lo, hi) whose delay is >= d (rows are sorted by delay)
+__device__ int64_t first_delay_at_least(const uint32_t* col, const uint8_t* dl, int shift,
+                                        int64_t lo, int64_t hi, uint32_t d) {
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (edge_delay(col, dl, shift, mid) < d) lo = mid + 1; else hi = mid;
+  }
+  return lo;
+}
+
+// What the walk needs of an instance.
+struct EdgeView {
+  const uint16_t* rec;
+  const uint32_t* col;
+  const uint16_t* w;
+  const uint8_t* delay;
+  int64_t base;
+  uint32_t tmask;
+  int32_t shift, two_w;
+  float two_S;
+  __device__ __forceinline__ explicit EdgeView(const InstDesc& d)
+      : rec(d.rec), col(d.col), w(d.w), delay(d.delay), base(d.base), tmask(d.tmask), shift(d.shift),
+        two_w(d.two_w), two_S(d.two_S) {}
+};
+
+// Adds the warp's segments -- nseg edge records from e0 on, of a row of
+// instance inst (UNI: the first) whose spike was handed on at a step with low
+// bits key >> 1 and has class key & 1 -- each edge into the accumulator slot
+// of its arrival step.  The segments are laid end to end: consecutive lanes
+// take consecutive records (coalesced), and kWalkU chunks of 32 records are
+// loaded before the first of their reductions.  A chunk's owners come from
+// one word: the lanes whose segment starts in the chunk set its bit (a warp
+// OR), and a record belongs to the item whose rank among the non-empty ones
+// is the number of starts up to it; the items lie by rank in s_item (32 a
+// warp), so that an owner's data is one 16-byte read.  (A shuffle search per
+// chunk took 5 + 5 shuffles and more than twice the instructions, and the
+// walk is bound by its issue slots.)  Called by the whole warp.
+//
+// FOUR: four accumulator channels per neuron; an edge adds its two weights
+// (the one weight twice for one-weight records) to the channel pair of the
+// source's class with one 64-bit atomic.  Every channel sum stays below 2^31
+// (the fixed-point scale is chosen so), so the low word never carries into
+// the high one.
+template <bool FOUR, bool UNI>
+__device__ __forceinline__ void walk_segments(const EngineDev& e, const InstDesc* insts, int4* s_item,
+                                              int64_t e0, uint32_t nseg, int inst, uint32_t key,
+                                              unsigned long long pol_rec, unsigned long long pol_acc) {
+  const int lane = threadIdx.x & 31;
+  uint32_t incl = nseg;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t x = __shfl_up_sync(kFull, incl, o);
+    if (lane >= o) incl += x;
+  }
+  const uint32_t total = __shfl_sync(kFull, incl, 31);
+  if (total == 0u) return;
+  const uint32_t ex = incl - nseg;
+  const unsigned full = __ballot_sync(kFull, nseg != 0u);
+  if (nseg != 0u) {
+    const int64_t b = e0 - (int64_t)ex;  // record of edge fi of the walk: b + fi
+    s_item[__popc(full & ((1u << lane) - 1u))] = make_int4((int)(uint32_t)b, (int)(b >> 32), (int)key, inst);
+  }
+  __syncwarp();
+  const uint32_t smask = (uint32_t)e.acc_slots - 1u;
+  const unsigned upto = 0xffffffffu >> (31 - lane);  // this lane and those before
+  const EdgeView v0(insts[0]);
+  int begun = -1;  // items that start before the chunk, less one
+  for (uint32_t f = 0; f < total; f += 32u * kWalkU) {  // warp-uniform
+    uint32_t tg[kWalkU], wv[kWalkU], ky[kWalkU];
+    int ic[kWalkU];
+#pragma unroll
+    for (int u = 0; u < kWalkU; ++u) {
+      const uint32_t at = ex - (f + 32u * u);
+      const unsigned starts = __reduce_or_sync(kFull, nseg != 0u && at < 32u ? 1u << at : 0u);
+      const int owner = begun + __popc(starts & upto);
+      begun += __popc(starts);
+      const uint32_t fi = f + 32u * u + lane;
+      ky[u] = 0u;
+      ic[u] = -1;
+      if (fi < total) {
+        const int4 it = s_item[owner];
+        ky[u] = (uint32_t)it.z;
+        ic[u] = UNI ? 0 : it.w;
+        const int64_t ei = (int64_t)(((uint64_t)(uint32_t)it.y << 32) | (uint32_t)it.x) + (int64_t)fi;
+        const EdgeView v(UNI ? v0 : EdgeView(insts[ic[u]]));
+        if (FOUR && v.two_w) {  // 8-byte record: word, weight | second weight << 16
+          const uint2 r4 = ld_stream_u64(reinterpret_cast<const uint2*>(v.rec) + ei, pol_rec);
+          tg[u] = r4.x;
+          wv[u] = r4.y;
+        } else if (v.rec) {
+          // 6-byte record at byte 6 ei: two aligned words cover it (the
+          // record array carries 8 bytes of padding at its end)
+          const size_t byte = 6 * (size_t)ei;
+          const uint32_t* w4 = reinterpret_cast<const uint32_t*>(
+              reinterpret_cast<const unsigned char*>(v.rec) + (byte & ~size_t(3)));
+          const uint32_t w0 = ld_stream_u32(w4, pol_rec), w1 = ld_stream_u32(w4 + 1, pol_rec);
+          const uint32_t sh = (uint32_t)(byte & 3u) * 8u;  // 0 or 16
+          tg[u] = __funnelshift_r(w0, w1, sh);
+          const uint32_t wb = (w1 >> sh) & 0xFFFFu;
+          wv[u] = wb | (wb << 16);
+        } else {
+          tg[u] = __ldg(v.col + ei) | ((uint32_t)__ldg(v.delay + ei) << v.shift);
+          const uint32_t wb = __ldg(v.w + ei);
+          wv[u] = wb | (wb << 16);
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kWalkU; ++u) {
+      if (ic[u] < 0) continue;
+      const EdgeView v(UNI ? v0 : EdgeView(insts[ic[u]]));
+      const uint32_t slot = ((ky[u] >> 1) + (tg[u] >> v.shift)) & smask;
+      const size_t at = (size_t)slot * (size_t)e.stride + (size_t)v.base + (tg[u] & v.tmask);
+      const int q = __float2int_rn(__fmul_rn(__uint_as_float(wv[u] << 16), v.two_S));
+      if (FOUR) {
+        const int q2 = __float2int_rn(__fmul_rn(__uint_as_float(wv[u] & 0xFFFF0000u), v.two_S));
+        red_add_u64(reinterpret_cast<unsigned long long*>(e.acc) + 2 * at + (ky[u] & 1u),
+                    ((unsigned long long)(uint32_t)q2 << 32) | (uint32_t)q, pol_acc);
+      } else {
+        red_add_s32(reinterpret_cast<int*>(e.acc) + 2 * at + (ky[u] & 1u), q, pol_acc);
+      }
+    }
+  }
+  __syncwarp();  // s_item is read
+}
+
+// Row j of the segment table: a header with the row's first and last edge,
+// then the counts.  One look-up per item reads both from one DRAM page.
+__device__ __forceinline__ const unsigned char* seg_row(const InstDesc& dd, int64_t j) {
+  return static_cast<const unsigned char*>(dd.seg) + j * (int64_t)dd.seg_bytes;
+}
+// Edges of a row of delay <= d, for 1 <= d <= dmax, from its table row.
+__device__ __forceinline__ uint32_t edges_up_to(const InstDesc& dd, const unsigned char* row, int d) {
+  return dd.seg_kind == kSeg16 ? (uint32_t)__ldg(reinterpret_cast<const uint16_t*>(row + kSegHead) + d - 1)
+                               : __ldg(reinterpret_cast<const uint32_t*>(row + kSegHead) + d - 1);
 }
 
 // Region constants of a thread's four neurons: one region's for all (ONE), or
@@ -383,7 +520,8 @@ __device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDe
 // 53.2 us with 50,000 spikes a step); an L2 prefetch of the state 304 to
 // 1,216 tiles ahead changed nothing.
 template <bool EXT, bool FOUR>
-__device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& sr, int tile, int warp) {
+__device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& sr, int tile, int warp,
+                                            int4* s_item) {
   const int lane = threadIdx.x & 31;
   // state loads first: they depend only on the tile, and the arrays cover
   // every padded tile
@@ -435,7 +573,7 @@ __device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& s
   }
   const unsigned spk = qs.spk, cls_bits = qs.cls;
 
-  // ---- spikes: one ring append, spike and raster count per warp ----------
+  // ---- spikes: counts, ring append, and the edges that are due soon -------
   if (!__any_sync(kFull, spk != 0)) return;
   const int nsp = __popc(spk);
   int ps = nsp;
@@ -444,63 +582,103 @@ __device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& s
     const int t = __shfl_up_sync(kFull, ps, o);
     if (lane >= o) ps += t;
   }
-  // the ring slot of the step at which these spikes are handed on: this
-  // step, or with spike binning the last step of its bin
-  const unsigned long long rel =
-      d.bin_sp ? d.g0 + (unsigned long long)((div_steps(n, d.spb) + 1) * d.spb - 1) : g;
-  const int slot = (int)((rel >> 32) ? rel % (unsigned long long)e.D : (uint32_t)rel % (uint32_t)e.D);
+  const int total = __shfl_sync(kFull, ps, 31);
+  // the step at which these spikes are handed on: this step, or with spike
+  // binning the last step of its bin
+  const long long bin = div_steps(n, d.spb);
+  const unsigned long long rel = d.bin_sp ? d.g0 + (unsigned long long)((bin + 1) * d.spb - 1) : g;
+  const int slot = e.mode == kAtEmission ? 0
+                   : (int)((rel >> 32) ? rel % (unsigned long long)e.D : (uint32_t)rel % (uint32_t)e.D);
+  int32_t* const cnt = e.cnt + (bin & 1) * e.cnt_stride + d.rbase + r0;
   uint32_t hbase = 0;
   unsigned long long rbase = 0;
   if (lane == 31) {
-    hbase = atomicAdd(e.hcount + slot, (uint32_t)ps);
+    if (e.mode != kAtEmission) hbase = atomicAdd(e.hcount + slot, (uint32_t)ps);
     atomicAdd(&e.dyn[inst].spikes, (unsigned long long)ps);
     if (d.raster_cap > 0) rbase = atomicAdd(&e.dyn[inst].raster_count, (unsigned long long)ps);
+    if (ti.z == 1) atomicAdd(cnt, ps);
   }
   hbase = __shfl_sync(kFull, hbase, 31);
   rbase = __shfl_sync(kFull, rbase, 31);
-  if (spk) {
-    uint64_t pos = (uint64_t)hbase + (uint32_t)(ps - nsp);
-    unsigned long long rpos = rbase + (unsigned long long)(ps - nsp);
-    uint32_t* hslot = e.hist + (size_t)slot * (size_t)e.hist_cap;
+  // the longest delay whose edges this warp adds: up to the end of the window
+  // in which the spikes are handed on, or every delay
+  const int dnow = e.mode == kAtEmission ? d.dmax
+                   : e.push_now ? min(e.wmask - (int)((unsigned)rel & (unsigned)e.wmask), d.dmax)
+                                : 0;
+  unsigned long long ev = 0;
+  // spike i of the warp goes to lane i mod 32: its owner by a shuffle search
+  // over the inclusive counts, its neuron the owner's bit of that rank
+  for (int i0 = 0; i0 < total; i0 += 32) {
+    const int i = i0 + lane;
+    int o = 0;
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      if (!(spk & (1u << k))) continue;
-      if (pos < (uint64_t)e.hist_cap)
-        hslot[pos] = (uint32_t)(gi0 + k) | (((cls_bits >> k) & 1u) << 31);
-      else
-        atomicOr(e.flags, kFlagHistOverflow);
-      ++pos;
-      atomicAdd(&e.cnt[d.rbase + r0 + each.r[k]], 1);
-      if (d.raster_cap > 0) {
-        if (rpos < (unsigned long long)d.raster_cap) {
-          d.raster_step[rpos] = (int32_t)n;
-          d.raster_id[rpos] = li0 + k;
+    for (int step = 16; step > 0; step >>= 1) {
+      const int v = __shfl_sync(kFull, ps, o + step - 1);
+      if (v <= i) o += step;
+    }
+    o = o < 32 ? o : 31;
+    unsigned bits = __shfl_sync(kFull, spk, o);
+    const unsigned inh = __shfl_sync(kFull, cls_bits, o);
+    int rank = i - (__shfl_sync(kFull, ps, o) - __popc(bits));
+    const int rk = ti.z == 1 ? 0 : -1;
+    int64_t e0 = 0;
+    uint32_t nseg = 0, key = 0;
+    int k = 0;
+    if (i < total) {
+      while (rank-- > 0) bits &= bits - 1u;
+      k = __ffs(bits) - 1;
+      const int32_t lo = li0 - lane * 4 + o * 4 + k;  // the neuron
+      const unsigned cl = (inh >> k) & 1u;
+      if (e.mode != kAtEmission) {
+        const uint64_t pos = (uint64_t)hbase + (uint32_t)i;
+        if (pos < (uint64_t)e.hist_cap)
+          e.hist[(size_t)slot * (size_t)e.hist_cap + pos] = (uint32_t)(d.base + lo) | (cl << 31);
+        else
+          atomicOr(e.flags, kFlagHistOverflow);
+      }
+      if (d.raster_cap > 0 && rbase + (unsigned)i < (unsigned long long)d.raster_cap) {
+        d.raster_step[rbase + (unsigned)i] = (int32_t)n;
+        d.raster_id[rbase + (unsigned)i] = lo;
+      }
+      if (rk < 0) {
+        int r = 0;
+        while (lo >= __ldg(&rcp[r].end)) ++r;
+        atomicAdd(cnt + r, 1);
+      }
+      if (dnow > 0) {
+        key = ((uint32_t)rel << 1) | cl;
+        if (e.mode == kAtEmission) {  // the whole row
+          e0 = __ldg(d.row_ptr + lo);
+          nseg = (uint32_t)(__ldg(d.row_ptr + lo + 1) - e0);
+          ev += nseg;
+        } else {
+          const unsigned char* row = seg_row(d, lo);
+          e0 = __ldg(reinterpret_cast<const longlong2*>(row)).x;
+          nseg = edges_up_to(d, row, dnow);
         }
-        ++rpos;
       }
     }
+    if (dnow > 0)
+      walk_segments<FOUR, true>(e, &d, s_item + (threadIdx.x >> 5) * 32, e0, nseg, 0, key, l2_policy_first(), l2_policy_last());
+  }
+  if (e.mode == kAtEmission) {  // the synaptic events of these spikes
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
+    if (lane == 0 && ev) atomicAdd(e.events, ev);
   }
 }
 
 template <bool EXT, bool FOUR>
 __global__ void __launch_bounds__(kUpdThreads, 7) k_update(EngineDev e, StepRef sr) {
-  const int w = blockIdx.x * (kUpdThreads / 32) + (threadIdx.x >> 5);
-  update_warp<EXT, FOUR>(e, sr, w / kTileWarps, w % kTileWarps);
-}
-
-__device__ __forceinline__ uint32_t edge_delay(const uint32_t* col, const uint8_t* dl, int shift,
-                                               int64_t e) {
-  return dl ? (uint32_t)__ldg(dl + e) : (__ldg(col + e) >> shift);
-}
-
-// first edge in [lo, hi) whose delay is >= d (rows are sorted by delay)
-__device__ int64_t first_delay_at_least(const uint32_t* col, const uint8_t* dl, int shift,
-                                        int64_t lo, int64_t hi, uint32_t d) {
-  while (lo < hi) {
-    const int64_t mid = (lo + hi) >> 1;
-    if (edge_delay(col, dl, shift, mid) < d) lo = mid + 1; else hi = mid;
+  const int n_close = (e.total_R + kUpdThreads - 1) / kUpdThreads;
+  if ((int)blockIdx.x < n_close) {  // close the bins that ended with the previous iteration
+    const int gr = blockIdx.x * kUpdThreads + threadIdx.x;
+    if (gr < e.total_R) close_region(e, gr, step_of(sr));
+    return;
   }
-  return lo;
+  const int w = (blockIdx.x - n_close) * (kUpdThreads / 32) + (threadIdx.x >> 5);
+  __shared__ int4 s_item[kUpdThreads];
+  update_warp<EXT, FOUR>(e, sr, w / kTileWarps, w % kTileWarps, s_item);
 }
 
 // Stage one of resolving an item (spike k of the ring slot of step g - d,
@@ -525,8 +703,7 @@ struct ItemLoads {
 // part: kPartAll does the whole delivery of iteration g.  The pipelined
 // schedule splits it: kPartLong, the arrival items of delays >= 2, which
 // read only spikes of steps <= g - 2 and so run beside the update of
-// iteration g - 1; then kPartShort after that update: the bin close, the
-// ring bookkeeping, the segment-ring copy of step g - 1's spikes, the
+// iteration g - 1; then kPartShort after that update: the ring bookkeeping, the segment-ring copy of step g - 1's spikes, the
 // delay-1 items and the emission items.
 // Loads of the spike and segment rings: through the read-only path when
 // the rings are written only by earlier launches; from the L2 (coherent,
@@ -558,10 +735,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
   const int D = e.D;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int gtid = bid * blockDim.x + threadIdx.x;
-  // close the bin that ended with the previous iteration, one region per thread
   const bool do_short = part != kPartLong, do_long = part != kPartShort;
-  if (do_short)
-    for (int gr = gtid; gr < e.total_R; gr += nblk * blockDim.x) close_region(e, gr, g);
   // the slot that the updates from this iteration on fill (a bin later with
   // spike binning) was last read by the previous iteration; the slot handed
   // on at g - 1 gets its long delays now, at emission, when d_emit allows
@@ -610,8 +784,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
             if (dd.seg_kind == kSeg16) {
               const int64_t j = gidx - dd.base;
               r0 = __ldg(dd.row_ptr + j);
-              row = reinterpret_cast<const uint4*>(static_cast<const uint16_t*>(dd.seg) +
-                                                   j * dd.seg_stride);
+              row = reinterpret_cast<const uint4*>(seg_row(dd, j) + kSegHead);
               nq = (dd.dmax + 7) >> 3;
             }
           }
@@ -645,9 +818,8 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
   const int bB = bid - nA, nB = nblk - nA;  // item blocks
 
   // spikes handed on at step g - d for d = threadIdx.x + 1, and their
-  // exclusive prefix (delays up to D - 1 - bin_lead: the later slots hold
-  // bins still filling)
-  const int dlim = D - 1 - e.bin_lead;
+  // exclusive prefix
+  const int dlim = e.dmax;
   unsigned long long c = 0;
   const int dme = threadIdx.x + 1;
   if (dme <= dlim && g >= (unsigned long long)dme && (dme == 1 ? do_short : do_long)) {
@@ -714,7 +886,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
   }
   const unsigned long long W = W_arr + c1e * (unsigned long long)ne;
   const unsigned long long acc_elems = (unsigned long long)e.stride * (FOUR ? 2 : 1);
-  const uint32_t aslot_now = e.acc_slots > 1 ? (uint32_t)(g % (unsigned long long)e.acc_slots) : 0u;
+  const uint32_t aslot_now = (uint32_t)g & ((uint32_t)e.acc_slots - 1u);
   __syncthreads();
 
   const unsigned long long pol_rec = l2_policy_first(), pol_acc = l2_policy_last();
@@ -730,7 +902,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
       p.k = (uint32_t)(te / (unsigned long long)ne);
       p.d = (uint32_t)e.d_emit + (uint32_t)(te % (unsigned long long)ne);
       p.slot = (uint32_t)s1;
-      p.aslot = (uint32_t)((g - 1ull + p.d) % (unsigned long long)e.acc_slots);
+      p.aslot = (uint32_t)(g - 1ull + p.d) & ((uint32_t)e.acc_slots - 1u);
       p.ent = ld_ring<PERSIST>(e.hist + (size_t)p.slot * (size_t)e.hist_cap + p.k);
       return;
     }
@@ -748,7 +920,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
     p.k = (uint32_t)((unsigned long long)q * s_cnt[lo] / (unsigned long long)Q + (tq - s_pre[q][lo]));
     p.slot = (uint32_t)((g - p.d) % (unsigned long long)D);
     p.ent = ld_ring<PERSIST>(e.hist + (size_t)p.slot * (size_t)e.hist_cap + p.k);
-    if (p.d >= 2u && p.k < cap) {  // from the delay-major ring (coalesced across lanes)
+    if (p.d >= 2u && p.k < cap && g - p.d >= e.since) {  // from the delay-major ring (coalesced across lanes)
       p.ring = true;
       p.r0 = ld_ring<PERSIST>(e.hr0 + p.slot * cap + p.k);
       const uint16_t* H = e.hseg + ((size_t)p.slot * (size_t)e.dcap) * cap + p.k;
@@ -792,12 +964,12 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
       b = (int64_t)p.b;
     } else if (dd.seg_kind == kSeg16) {
       r0 = __ldg(dd.row_ptr + j);
-      const uint16_t* T = static_cast<const uint16_t*>(dd.seg) + j * dd.seg_stride;
+      const uint16_t* T = reinterpret_cast<const uint16_t*>(seg_row(dd, j) + kSegHead);
       a = d >= 2 ? (int64_t)__ldg(T + d - 2) : 0;
       b = (int64_t)__ldg(T + d - 1);
     } else if (dd.seg_kind == kSeg32) {
       r0 = __ldg(dd.row_ptr + j);
-      const uint32_t* T = static_cast<const uint32_t*>(dd.seg) + j * dd.seg_stride;
+      const uint32_t* T = reinterpret_cast<const uint32_t*>(seg_row(dd, j) + kSegHead);
       a = d >= 2 ? (int64_t)__ldg(T + d - 2) : 0;
       b = (int64_t)__ldg(T + d - 1);
     } else {
@@ -855,9 +1027,9 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
           if (fi < total) {
             const InstDesc& dd = e.insts[SINGLE ? 0 : (ic[u] & 0x7FFFFF)];
             const int64_t ei = q0 + (int64_t)(fi - qx);
-            if (FOUR && dd.two_w) {  // 8-byte record: target, weight | second weight << 16
+            if (FOUR && dd.two_w) {  // 8-byte record: word, weight | second weight << 16
               const uint2 r4 = ld_stream_u64(reinterpret_cast<const uint2*>(dd.rec) + ei, pol_rec);
-              tg[u] = r4.x;
+              tg[u] = r4.x & dd.tmask;
               wv[u] = r4.y;
             } else if (dd.rec) {
               // 6-byte record at byte 6 ei: two aligned words cover it (the
@@ -867,7 +1039,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
                   reinterpret_cast<const unsigned char*>(dd.rec) + (byte & ~size_t(3)));
               const uint32_t w0 = ld_stream_u32(w4, pol_rec), w1 = ld_stream_u32(w4 + 1, pol_rec);
               const uint32_t sh = (uint32_t)(byte & 3u) * 8u;  // 0 or 16
-              tg[u] = __funnelshift_r(w0, w1, sh);
+              tg[u] = __funnelshift_r(w0, w1, sh) & dd.tmask;
               const uint32_t wb = (w1 >> sh) & 0xFFFFu;
               wv[u] = wb | (wb << 16);
             } else {
@@ -901,6 +1073,295 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
   if (lane == 0 && ev) atomicAdd(e.events, ev);
+}
+
+// A row in the bounds ring: first edge (47 bits), class, instance (16 bits).
+constexpr unsigned long long kRowMask = (1ull << 47) - 1ull;
+constexpr unsigned long long kNoRow = ~0ull;
+
+// The window bounds of step g - 1's spikes into the ring, one warp per spike,
+// warps w0, w0 + n, ...: for the spike of rank k, its row into hr0[slot][k],
+// and into hseg[slot][j][k] the number of its edges with delay below the
+// first of window j (of W delays; the first window starts at the next
+// multiple of W).  The items of later windows then read 12 bytes next to
+// their neighbours' each, where the row and table look-ups of an item are
+// three random DRAM accesses: at the 37 G a second measured for those, they
+// cost more than the edges (of a window kernel of 285 us for 21.6 M edges,
+// 128 us were left without its edge reads and reductions).  Counts the
+// synaptic events of those spikes: the out-degree of each, once (Supp. Alg. 2
+// pushes every out-edge once).
+template <bool PERSIST>
+__device__ __forceinline__ void copy_bounds(const EngineDev& e, unsigned long long g, uint32_t w0, uint32_t n,
+                                            unsigned long long& ev) {
+  if (g == 0ull) return;
+  const int lane = threadIdx.x & 31;
+  const uint32_t sl = (uint32_t)((g - 1ull) % (unsigned long long)e.D);
+  const uint32_t h = PERSIST ? __ldcg(e.hcount + sl) : e.hcount[sl];
+  const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap, cap = (uint32_t)e.seg_cap;
+  const int W = e.wmask + 1;
+  const int first = W - (int)((unsigned)(g - 1ull) & (unsigned)e.wmask);  // delay at the next window's start
+  for (uint32_t k = w0; k < c; k += n) {
+    const uint32_t ent = ld_ring<PERSIST>(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
+    const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
+    const int inst = e.n_inst == 1 ? 0 : e.tile_info[gidx / kTile].x;
+    unsigned long long packed = kNoRow;
+    if (inst >= 0) {
+      const InstDesc& dd = e.insts[inst];
+      const unsigned char* row = seg_row(dd, gidx - dd.base);
+      if (dd.seg_kind == kSeg16 && k < cap)
+        for (int j = lane; j < e.dcap; j += 32) {
+          const int d = first + j * W - 1;  // the last delay before window j
+          e.hseg[(sl * (size_t)e.dcap + j) * cap + k] =
+              (uint16_t)(d < 1 ? 0u : edges_up_to(dd, row, d < dd.dmax ? d : dd.dmax));
+        }
+      const longlong2 r = __ldg(reinterpret_cast<const longlong2*>(row));
+      if (lane == 0) ev += (unsigned long long)(r.y - r.x);
+      if (dd.seg_kind == kSeg16)
+        packed = (unsigned long long)r.x | ((unsigned long long)(ent >> 31) << 47) | ((unsigned long long)inst << 48);
+    }
+    if (lane == 0 && k < cap) reinterpret_cast<unsigned long long*>(e.hr0)[sl * (size_t)cap + k] = packed;
+  }
+}
+
+// kWindows: the arrivals of steps g .. g + W - 1, W = wmask + 1, from the
+// spikes handed on before step g, as block bid of nblk; the block's threads
+// call it together.  Bucket t holds the spikes of step g - 1 - t, and an item
+// (a spike of bucket t) is the segment of its row with delays t + 1 .. t + W.
+//
+// Bound: random DRAM accesses (some 37 G a second measured) and the
+// reductions into the accumulators (212 G/s while they lie in the L2, 34 to
+// 58 G/s beyond).  A window of W delays reads a row in pieces W times as long
+// as one step's would be, W times less often, so the items and the sectors
+// that hold a piece's few records fall with W, and the accumulators grow with
+// it: W = 4 / 2 / 1 measured 33.8 / 35.0 / 43.2 us a step at 2 M neurons and
+// in-degree 1,000 (16 MB of accumulators per step; 45.3 us with one delay per
+// step and kernel), 49.9 / 45.2 / 50.9 us at 5 M and 400 (40 MB; 60.2 us).
+template <bool FOUR, bool SINGLE, bool PERSIST>
+__device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned long long g, int bid, int nblk) {
+  // items of phase q and bucket t start at s_pre[q][t] of the phase
+  __shared__ uint32_t s_pre[kMaxPhases][256];
+  __shared__ uint32_t s_wsum[kMaxPhases][kDelThreads / 32];
+  __shared__ uint32_t s_items[kMaxPhases];     // of the phase
+  __shared__ uint32_t s_unit[kMaxPhases + 1];  // warp units before the phase
+  __shared__ uint32_t s_cnt[256];
+  __shared__ int4 s_item[kDelThreads];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned long long D = (unsigned long long)e.D;
+  const int W = e.wmask + 1;
+  // the slots that the updates of this window fill (a bin later with spike
+  // binning): their spikes' last arrivals lie before step g
+  if (bid == 0 && (int)threadIdx.x < W && !e.keep_counts)
+    e.hcount[(g + (unsigned long long)e.bin_lead + threadIdx.x) % D] = 0u;
+  const uint32_t top = (uint32_t)((g + D - 1ull) % D);  // ring slot of step g - 1
+  const auto ring_of = [&](int t) {                     // and of step g - 1 - t
+    return top >= (uint32_t)t ? top - (uint32_t)t : top + (uint32_t)D - (uint32_t)t;
+  };
+  unsigned long long ev = 0;
+  // buckets t0 .. t0 + nb - 1 at a time, so that their spikes count in 32 bits
+  // (all of them at once up to some 20 M neurons)
+  const int n_buckets = e.dmax;
+  const int at_once = (int)min((long long)n_buckets, 0xFFFFFFC0ll / (long long)e.hist_cap);
+  for (int t0 = 0; t0 < n_buckets; t0 += at_once) {
+  const int nb = min(at_once, n_buckets - t0);
+  uint32_t c = 0;
+  const int tme = threadIdx.x;
+  if (tme < nb && g >= (unsigned long long)(t0 + tme) + 1ull) {
+    const uint32_t sl = ring_of(t0 + tme);
+    const uint32_t h = PERSIST ? __ldcg(e.hcount + sl) : e.hcount[sl];
+    c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
+  }
+  // Phases: the update appends each step's spikes roughly in tile order, so
+  // a spike's rank in its slot follows its region.  Taking the items rank
+  // phase by rank phase (phase q: ranks [q c/Q, (q+1) c/Q) of every slot)
+  // keeps the warps in flight on a narrow band of regions, so the
+  // within-region edges (most of them) add into a slice of the accumulators
+  // that stays in the L2 even when all of them do not fit.
+  const int Qb = e.phases > 1 ? 3 : 0, Q = 1 << Qb;
+  s_cnt[threadIdx.x] = c;
+  uint32_t incl[kMaxPhases], own[kMaxPhases];
+#pragma unroll
+  for (int q = 0; q < kMaxPhases; ++q) {
+    own[q] = q < Q ? (uint32_t)(((q + 1ull) * c >> Qb) - ((unsigned long long)q * c >> Qb)) : 0u;
+    incl[q] = own[q];
+    if (q < Q) {  // block-uniform
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t t = __shfl_up_sync(kFull, incl[q], o);
+        if (lane >= o) incl[q] += t;
+      }
+    }
+    if (lane == 31) s_wsum[q][warp] = incl[q];
+  }
+  __syncthreads();
+  if (threadIdx.x < kMaxPhases) {  // warp offsets within each phase
+    uint32_t acc = 0;
+    for (int w = 0; w < kDelThreads / 32; ++w) {
+      const uint32_t t = s_wsum[threadIdx.x][w];
+      s_wsum[threadIdx.x][w] = acc;
+      acc += t;
+    }
+    s_items[threadIdx.x] = acc;
+  }
+  __syncthreads();
+  // items per unit: 32, or fewer when that would leave warps without one
+  uint32_t all = 0;
+  for (int q = 0; q < Q; ++q) all += s_items[q];
+  int ub = 5;
+  while (ub > 0 && (all >> ub) < (uint32_t)nblk * (kDelThreads / 32)) --ub;
+  if (threadIdx.x == 0) {
+    s_unit[0] = 0u;
+    for (int q = 0; q < kMaxPhases; ++q) s_unit[q + 1] = s_unit[q] + ((s_items[q] + (1u << ub) - 1u) >> ub);
+  }
+#pragma unroll
+  for (int q = 0; q < kMaxPhases; ++q) s_pre[q][threadIdx.x] = s_wsum[q][warp] + incl[q] - own[q];
+  __syncthreads();
+  const uint32_t n_units = s_unit[kMaxPhases];
+  const unsigned long long pol_rec = l2_policy_first(), pol_acc = l2_policy_last();
+
+  // A unit of 32 items is four runs of eight consecutive ones, a quarter of
+  // the phase apart: the buckets hold segments of very different lengths
+  // (short delays within a region, long ones across), so every unit gets an
+  // even share, and a run's bounds lie side by side in the ring.
+  struct Item {
+    unsigned long long row;  // packed row of the bounds ring, kNoRow: not there
+    uint32_t a, b, k;
+    int t;  // bucket, -1: none
+  };
+  const uint32_t cap = (uint32_t)e.seg_cap;
+  auto fetch = [&](uint32_t u) {
+    Item it{kNoRow, 0u, 0u, 0u, -1};
+    if (u >= n_units || lane >= (1 << ub)) return it;
+    int q = 0;  // the phase: the largest q < Q with s_unit[q] <= u
+    for (int step = kMaxPhases / 2; step > 0; step >>= 1)
+      if (q + step < Q && s_unit[q + step] <= u) q += step;
+    const uint32_t U = s_unit[q + 1] - s_unit[q], v = u - s_unit[q];
+    const uint32_t x = ub == 5 ? ((uint32_t)lane >> 3) * (U * 8u) + v * 8u + (lane & 7) : (v << ub) + lane;
+    if (x >= s_items[q]) return it;
+    int lo = 0;  // the bucket: the largest with s_pre[q][lo] <= x
+#pragma unroll
+    for (int step = 128; step > 0; step >>= 1)
+      if (lo + step < nb && s_pre[q][lo + step] <= x) lo += step;
+    it.k = (uint32_t)((unsigned long long)q * s_cnt[lo] >> Qb) + (x - s_pre[q][lo]);
+    it.t = t0 + lo;
+    if (it.t > 0 && it.k < cap && g - 1ull - (unsigned long long)it.t >= e.since) {  // window it.t / W of its slot
+      const size_t sl = ring_of(it.t);
+      const uint16_t* B = e.hseg + (sl * (size_t)e.dcap + (uint32_t)it.t / (uint32_t)W) * cap + it.k;
+      it.row = ld_ring<PERSIST>(reinterpret_cast<const unsigned long long*>(e.hr0) + sl * cap + it.k);
+      it.a = ld_ring<PERSIST>(B);
+      it.b = ld_ring<PERSIST>(B + cap);
+    }
+    return it;
+  };
+  // an item's segment: from the ring, or from its row of the segment table
+  auto resolve = [&](const Item& it, int64_t& e0, uint32_t& n, int& inst, uint32_t& key) {
+    e0 = 0;
+    n = 0u;
+    inst = 0;
+    key = 0u;
+    if (it.t < 0) return;
+    const int d0 = it.t + 1;
+    key = (uint32_t)(g - (unsigned long long)d0) << 1;
+    if (it.row != kNoRow) {
+      e0 = (int64_t)(it.row & kRowMask) + it.a;
+      n = it.b - it.a;
+      inst = SINGLE ? 0 : (int)(it.row >> 48);
+      key |= (uint32_t)(it.row >> 47) & 1u;
+      return;
+    }
+    const uint32_t ent = ld_ring<PERSIST>(e.hist + (size_t)ring_of(it.t) * (size_t)e.hist_cap + it.k);
+    const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
+    key |= ent >> 31;
+    if (!SINGLE) {
+      inst = e.tile_info[gidx / kTile].x;
+      if (inst < 0) {  // never for a listed spike: tiles are reused D steps late
+        inst = 0;
+        return;
+      }
+    }
+    const InstDesc& dd = e.insts[inst];
+    const int d1 = it.t + W < dd.dmax ? it.t + W : dd.dmax;
+    const unsigned char* row = seg_row(dd, gidx - dd.base);
+    const longlong2 r = __ldg(reinterpret_cast<const longlong2*>(row));
+    if (cap == 0u && it.t < W && g - (unsigned long long)d0 >= e.since) ev += (unsigned long long)(r.y - r.x);
+    if (d0 > d1) return;
+    const uint32_t a = d0 >= 2 ? edges_up_to(dd, row, d0 - 1) : 0u;
+    e0 = r.x + a;
+    n = edges_up_to(dd, row, d1) - a;
+  };
+  const uint32_t stride = (uint32_t)nblk * (kDelThreads / 32);
+  uint32_t u = (uint32_t)bid * (kDelThreads / 32) + warp;
+  Item next = fetch(u);
+  for (; u < n_units; u += stride) {  // warp-uniform
+    const Item it = next;
+    next = fetch(u + stride);  // its loads fly while this unit's edges are walked
+    int64_t e0;
+    uint32_t n, key;
+    int inst;
+    resolve(it, e0, n, inst, key);
+    walk_segments<FOUR, SINGLE>(e, e.insts, s_item + warp * 32, e0, n, inst, key, pol_rec, pol_acc);
+  }
+  __syncthreads();
+  }
+  if (e.seg_cap > 0)
+    copy_bounds<PERSIST>(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, (uint32_t)nblk * (kDelThreads / 32), ev);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
+  if (lane == 0 && ev) atomicAdd(e.events, ev);
+}
+
+// kWindows, inside a window: the edges of the spikes handed on at step g - 1
+// that come due by the window's end, the start of their rows.  A warp takes 32
+// of the spikes, or fewer when that would leave warps without one; four
+// dependent loads (count, ring entry, table row, records) bound it.
+template <bool FOUR, bool SINGLE, bool PERSIST>
+__device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long long g, int bid, int nblk,
+                                             int4* s_item) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int left = e.wmask + 1 - (int)((unsigned)g & (unsigned)e.wmask);  // steps to the window's end
+  const uint32_t sl = (uint32_t)((g - 1ull) % (unsigned long long)e.D);
+  const uint32_t h = PERSIST ? __ldcg(e.hcount + sl) : __ldg(e.hcount + sl);
+  const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
+  const uint32_t warps = (uint32_t)nblk * (kDelThreads / 32);
+  int ub = 5;
+  while (ub > 0 && (c >> ub) < warps) --ub;
+  const uint32_t n_units = (uint32_t)(((unsigned long long)c + (1u << ub) - 1u) >> ub);
+  for (uint32_t u = (uint32_t)bid * (kDelThreads / 32) + warp; u < n_units; u += warps) {
+    const uint32_t k = (u << ub) + lane;
+    int64_t e0 = 0;
+    uint32_t nseg = 0, key = 0;
+    int inst = 0;
+    if (lane < (1 << ub) && k < c) {
+      const uint32_t ent = ld_ring<PERSIST>(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
+      const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
+      if (!SINGLE) inst = e.tile_info[gidx / kTile].x;
+      if (inst >= 0) {
+        const InstDesc& dd = e.insts[inst];
+        const unsigned char* row = seg_row(dd, gidx - dd.base);
+        e0 = __ldg(reinterpret_cast<const longlong2*>(row)).x;
+        nseg = edges_up_to(dd, row, left < dd.dmax ? left : dd.dmax);
+        key = ((uint32_t)(g - 1ull) << 1) | (ent >> 31);
+      } else {
+        inst = 0;
+      }
+    }
+    walk_segments<FOUR, SINGLE>(e, e.insts, s_item + warp * 32, e0, nseg, inst, key, l2_policy_first(),
+                                l2_policy_last());
+  }
+  if (e.seg_cap == 0) return;
+  unsigned long long ev = 0;
+  copy_bounds<PERSIST>(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, warps, ev);
+  if (lane == 0 && ev) atomicAdd(e.events, ev);
+}
+
+template <bool FOUR, bool SINGLE>
+__global__ void __launch_bounds__(kDelThreads, 4) k_windows(EngineDev e, StepRef sr) {
+  deliver_windows<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x);
+}
+
+template <bool FOUR, bool SINGLE>
+__global__ void __launch_bounds__(kDelThreads, 4) k_rest(EngineDev e, StepRef sr) {
+  __shared__ int4 s_item[kDelThreads];
+  deliver_rest<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x, s_item);
 }
 
 template <bool FOUR, bool SINGLE>
@@ -960,23 +1421,34 @@ __device__ bool grid_barrier(unsigned* count, unsigned target, unsigned long lon
 }
 
 // The persistent stepper: iterations g0 .. g0 + nsteps - 1 in one
-// cooperative launch, each the delivery (the whole grid, as in k_deliver)
-// and the update (tiles dealt round robin over the blocks), with a grid
-// barrier after each.  The same device functions as the two-launch step do
+// cooperative launch, each the delivery where the mode has one (the whole
+// grid) and the update (tiles dealt round robin over the blocks), with a grid
+// barrier after each.  The same device functions as the launched step do
 // the work, so the results are identical bit for bit; a barrier that gives
 // up ends the launch (kFlagTimeout stays set for the host).
-template <bool EXT, bool FOUR, bool SINGLE>
+template <bool EXT, bool FOUR, bool SINGLE, bool PER_STEP>
 __global__ void __launch_bounds__(kDelThreads, 2)
     k_persist(EngineDev e, unsigned long long g0, int nsteps, unsigned* count,
               unsigned long long limit_ns) {
+  __shared__ int4 s_item[kDelThreads];
   unsigned target = 0;
   for (int s = 0; s < nsteps; ++s) {
-    const StepRef sr{nullptr, g0 + (unsigned long long)s, nullptr};
-    deliver_body<FOUR, SINGLE, true>(e, sr, kPartAll, blockIdx.x, gridDim.x);
-    target += gridDim.x;
-    if (!grid_barrier(count, target, limit_ns, e.flags)) return;
+    const unsigned long long g = g0 + (unsigned long long)s;
+    const StepRef sr{nullptr, g, nullptr};
+    const bool due = PER_STEP || (e.mode == kWindows && (!e.push_now || ((unsigned)g & (unsigned)e.wmask) == 0u));
+    if (due) {
+      if (PER_STEP) deliver_body<FOUR, SINGLE, true>(e, sr, kPartAll, blockIdx.x, gridDim.x);
+      else if (((unsigned)g & (unsigned)e.wmask) == 0u)
+        deliver_windows<FOUR, SINGLE, true>(e, g, blockIdx.x, gridDim.x);
+      else deliver_rest<FOUR, SINGLE, true>(e, g, blockIdx.x, gridDim.x, s_item);
+      target += gridDim.x;
+      if (!grid_barrier(count, target, limit_ns, e.flags)) return;
+    }
+    for (int gr = (gridDim.x - 1 - blockIdx.x) * kDelThreads + threadIdx.x; gr < e.total_R;
+         gr += gridDim.x * kDelThreads)
+      close_region(e, gr, g);  // the last blocks: the first ones have the most tiles
     for (int t = blockIdx.x; t < e.n_tiles; t += gridDim.x)
-      update_warp<EXT, FOUR>(e, sr, t, threadIdx.x >> 5);
+      update_warp<EXT, FOUR>(e, sr, t, threadIdx.x >> 5, s_item);
     target += gridDim.x;
     if (!grid_barrier(count, target, limit_ns, e.flags)) return;
   }
@@ -1018,17 +1490,19 @@ __device__ __forceinline__ uint16_t staged_bf16(const void* w_in, int32_t w_dtyp
 // from e_base on: warp per source row.  Checks every edge (target range,
 // delay >= 1 and non-decreasing within the row, weights finite and
 // non-negative after rounding to BF16), counts in-degrees, and writes
-//   rec[3e .. 3e+2] = target low 16 bits, target high 16 bits, BF16 weight
+//   rec[3e .. 3e+2] = word low 16 bits, word high 16 bits, BF16 weight
+//   (word: target | delay << shift, the delay's bits that fit)
 //   (with second weights w2_in: rec[4e .. 4e+3], the second weight last)
-//   seg[j * seg_stride + k] = number of edges of row j with delay <= k + 1
+//   row j of the segment table: first and last edge, then for k < dmax the
+//   number of edges with delay <= k + 1
 // (the segment table must be zero on entry; entries below the row's first
 // delay stay zero).
 __global__ void k_ingest(int32_t N, int32_t j0, int32_t j1, int64_t e_base,
                          const int64_t* __restrict__ row_ptr, const int32_t* __restrict__ col_in,
                          const void* __restrict__ w_in, const void* __restrict__ w2_in,
                          int32_t w_dtype, const uint8_t* __restrict__ delay_in,
-                         uint16_t* __restrict__ rec,
-                         int32_t dmax, int32_t seg_stride, void* seg, int32_t kind,
+                         uint16_t* __restrict__ rec, int32_t shift,
+                         int32_t dmax, int32_t seg_bytes, void* seg, int32_t kind,
                          int32_t* indeg, unsigned* wmax_bits, unsigned* err) {
   const int lane = threadIdx.x & 31;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1043,7 +1517,7 @@ __global__ void k_ingest(int32_t N, int32_t j0, int32_t j1, int64_t e_base,
       if (d < 1u) my_err |= kErrDelayRange;
       if (e > a && delay_in[e - 1] > d) my_err |= kErrDelayOrder;
       const uint16_t wb = staged_bf16(w_in, w_dtype, e, my_err, my_wmax);
-      const uint32_t tu = (uint32_t)t;
+      const uint32_t tu = (uint32_t)t | (shift < 32 ? (uint32_t)d << shift : 0u);
       if (w2_in) {
         const uint16_t wb2 = staged_bf16(w2_in, w_dtype, e, my_err, my_wmax);
         reinterpret_cast<uint2*>(rec)[e_base + e] = make_uint2(tu, (uint32_t)wb | ((uint32_t)wb2 << 16));
@@ -1057,8 +1531,10 @@ __global__ void k_ingest(int32_t N, int32_t j0, int32_t j1, int64_t e_base,
     }
     // segment counts: edge p closes the delays from its own to the next edge's
     const int64_t n = b - a;
-    uint16_t* T16 = static_cast<uint16_t*>(seg) + j * seg_stride;
-    uint32_t* T32 = static_cast<uint32_t*>(seg) + j * seg_stride;
+    unsigned char* row = static_cast<unsigned char*>(seg) + j * (int64_t)seg_bytes;
+    if (lane == 0) *reinterpret_cast<longlong2*>(row) = make_longlong2(row_ptr[j], row_ptr[j + 1]);
+    uint16_t* T16 = reinterpret_cast<uint16_t*>(row + kSegHead);
+    uint32_t* T32 = reinterpret_cast<uint32_t*>(row + kSegHead);
     for (int64_t p = lane; p < n; p += 32) {
       const int dp = (int)delay_in[a + p];
       const int dn = p + 1 < n ? (int)delay_in[a + p + 1] : dmax + 1;
@@ -1125,7 +1601,7 @@ void launch_init_state(const EngineDev& e, int inst, int n_tiles_inst, int first
 }
 
 void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s) {
-  const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads);
+  const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads) + (e.total_R + kUpdThreads - 1) / kUpdThreads;
   if (e.four) {
     if (e.any_ext) k_update<true, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
     else k_update<false, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
@@ -1167,45 +1643,58 @@ void launch_deliver(const EngineDev& e, int grid, StepRef sr, cudaStream_t s, in
   }
 }
 
+void launch_windows(const EngineDev& e, int grid, StepRef sr, bool first, cudaStream_t s) {
+  auto go = [&](auto kw, auto kr) {
+    if (first) kw<<<grid, kDelThreads, 0, s>>>(e, sr);
+    else kr<<<grid, kDelThreads, 0, s>>>(e, sr);
+  };
+  if (e.n_inst == 1) {
+    if (e.four) go(k_windows<true, true>, k_rest<true, true>);
+    else go(k_windows<false, true>, k_rest<false, true>);
+  } else {
+    if (e.four) go(k_windows<true, false>, k_rest<true, false>);
+    else go(k_windows<false, false>, k_rest<false, false>);
+  }
+}
+
+namespace {
+
+// f(kernel) for the stepper's variant that suits the engine
+template <bool EXT, bool FOUR, class F>
+auto with_persist(const EngineDev& e, F&& f) {
+  if (e.mode == kPerStep)
+    return e.n_inst == 1 ? f(k_persist<EXT, FOUR, true, true>) : f(k_persist<EXT, FOUR, false, true>);
+  return e.n_inst == 1 ? f(k_persist<EXT, FOUR, true, false>) : f(k_persist<EXT, FOUR, false, false>);
+}
+template <class F>
+auto with_persist(const EngineDev& e, F&& f) {
+  if (e.four) return e.any_ext ? with_persist<true, true>(e, f) : with_persist<false, true>(e, f);
+  return e.any_ext ? with_persist<true, false>(e, f) : with_persist<false, false>(e, f);
+}
+
+}  // namespace
+
 int persist_max_grid(const EngineDev& e) {
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const void* f = e.four ? (e.any_ext ? (const void*)k_persist<true, true, false>
-                                      : (const void*)k_persist<false, true, false>)
-                         : (e.any_ext ? (const void*)k_persist<true, false, false>
-                                      : (const void*)k_persist<false, false, false>);
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, f, kDelThreads, 0) != cudaSuccess) return 0;
-  return sms * occ;
-}
-
-template <bool EXT, bool FOUR, bool SINGLE>
-static cudaError_t coop_persist(const EngineDev& e, int grid, unsigned long long g0, int nsteps,
-                                unsigned* count, unsigned long long limit_ns, cudaStream_t s) {
-  EngineDev ea = e;
-  void* args[] = {&ea, &g0, &nsteps, &count, &limit_ns};
-  return cudaLaunchCooperativeKernel(k_persist<EXT, FOUR, SINGLE>, dim3(grid), dim3(kDelThreads),
-                                     args, 0, s);
+  const cudaError_t r = with_persist(e, [&](auto k) {
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kDelThreads, 0);
+  });
+  return r == cudaSuccess ? sms * occ : 0;
 }
 
 cudaError_t launch_persist(const EngineDev& e, int grid, unsigned long long g0, int nsteps,
                            unsigned* count, unsigned long long limit_ns, cudaStream_t s) {
-  if (grid < 2) grid = 2;  // with a segment ring, block 0 may take no items
-  cudaError_t r = cudaMemsetAsync(count, 0, sizeof(unsigned), s);
+  if (e.mode == kAtEmission) grid = grid < e.n_tiles ? grid : e.n_tiles;  // no work for more
+  else if (grid < 2) grid = 2;  // with a segment ring, block 0 may take no items
+  const cudaError_t r = cudaMemsetAsync(count, 0, sizeof(unsigned), s);
   if (r != cudaSuccess) return r;
-  const bool one = e.n_inst == 1;
-  if (e.four) {
-    if (e.any_ext)
-      return one ? coop_persist<true, true, true>(e, grid, g0, nsteps, count, limit_ns, s)
-                 : coop_persist<true, true, false>(e, grid, g0, nsteps, count, limit_ns, s);
-    return one ? coop_persist<false, true, true>(e, grid, g0, nsteps, count, limit_ns, s)
-               : coop_persist<false, true, false>(e, grid, g0, nsteps, count, limit_ns, s);
-  }
-  if (e.any_ext)
-    return one ? coop_persist<true, false, true>(e, grid, g0, nsteps, count, limit_ns, s)
-               : coop_persist<true, false, false>(e, grid, g0, nsteps, count, limit_ns, s);
-  return one ? coop_persist<false, false, true>(e, grid, g0, nsteps, count, limit_ns, s)
-             : coop_persist<false, false, false>(e, grid, g0, nsteps, count, limit_ns, s);
+  EngineDev ea = e;
+  void* args[] = {&ea, &g0, &nsteps, &count, &limit_ns};
+  return with_persist(e, [&](auto k) {
+    return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kDelThreads), args, 0, s);
+  });
 }
 
 cudaError_t launch_barrier_probe(int grid, unsigned extra, int rounds, unsigned long long limit_ns,
@@ -1218,22 +1707,38 @@ cudaError_t launch_barrier_probe(int grid, unsigned extra, int rounds, unsigned 
 
 void launch_ingest(int32_t N, int32_t j0, int32_t j1, int64_t e_base, const int64_t* row_ptr,
                    const int32_t* col_in, const void* w_in, const void* w2_in, int32_t w_dtype,
-                   const uint8_t* delay_in, uint16_t* rec, int32_t dmax, int32_t seg_stride,
-                   void* seg, int32_t seg_kind, int32_t* indeg, unsigned* wmax_bits, unsigned* err,
+                   const uint8_t* delay_in, uint16_t* rec, int32_t shift, int32_t dmax,
+                   int32_t seg_bytes, void* seg, int32_t seg_kind, int32_t* indeg, unsigned* wmax_bits, unsigned* err,
                    cudaStream_t s) {
   int64_t blocks = ((int64_t)(j1 - j0) * 32 + 255) / 256;
   if (blocks > 152 * 64) blocks = 152 * 64;
   if (blocks < 1) blocks = 1;
   k_ingest<<<(int)blocks, 256, 0, s>>>(N, j0, j1, e_base, row_ptr, col_in, w_in, w2_in, w_dtype,
-                                       delay_in, rec, dmax, seg_stride, seg, seg_kind, indeg,
+                                       delay_in, rec, shift, dmax, seg_bytes, seg, seg_kind, indeg,
                                        wmax_bits, err);
 }
 
 void launch_pending_events(const EngineDev& e, unsigned long long g, unsigned long long* out,
                            cudaStream_t s) {
-  if (g == 0) return;
-  const long long r0 = (long long)g - 1, r1 = (long long)g - 1 + e.bin_lead;
-  k_pending_events<<<152, 256, 0, s>>>(e, r0, r1, out);
+  if (g == 0 || e.mode == kAtEmission) return;
+  const long long window = ((long long)g - 1) & ~(long long)(e.mode == kWindows && !e.seg_cap ? e.wmask : 0);
+  launch_count_events(e, window > (long long)e.since ? window : (long long)e.since, (long long)g - 1 + e.bin_lead,
+                      out, s);
+}
+
+void launch_count_events(const EngineDev& e, long long r0, long long r1, unsigned long long* out, cudaStream_t s) {
+  if (r1 >= r0) k_pending_events<<<152, 256, 0, s>>>(e, r0, r1, out);
+}
+
+void launch_hand_over(const EngineDev& e, int grid, unsigned long long g, cudaStream_t s) {
+  EngineDev f = e;  // one window as long as the accumulator ring
+  f.mode = kWindows;
+  f.wmask = e.acc_slots - 1;
+  f.seg_cap = 0;
+  f.phases = 1;
+  f.keep_counts = 1;
+  f.since = g - 1ull;  // the spikes of step g - 1 are not counted yet
+  launch_windows(f, grid, StepRef{nullptr, g, nullptr}, true, s);
 }
 
 void launch_max_reduce(const int32_t* a, int64_t n, unsigned* out, cudaStream_t s) {

@@ -15,8 +15,11 @@
 // The same kernels as dbnet_step run here (init, deliver, update), so results
 // are identical to dbnet_create + dbnet_step on the same graph and options.
 // All calls share the scratch; each call clears it first; overlapping calls
-// race.  Without room for a per-graph segment table, the delivery finds each
-// spike's due segment by binary search over its row's delays.
+// race.  Where the accumulator ring fits the scratch (padded neurons x the
+// longest delay + 1 rounded up to a power of two <= 2^21) a spike's whole row
+// is added when it is emitted; else, without room for a per-graph segment
+// table, the delivery finds each spike's due segment by binary search over
+// its row's delays.
 #include <cuda_runtime.h>
 
 #include <climits>
@@ -46,7 +49,7 @@ constexpr int kMaxTiles = kMaxN / kTile;
 constexpr size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Byte offsets inside the scratch array.
-constexpr size_t kOffHist = 0;  // spike ring: kMaxLive entries
+constexpr size_t kOffHist = 0;  // spike ring: kMaxLive entries; or the accumulator ring
 constexpr size_t kOffAcc = align256(kOffHist + sizeof(uint32_t) * kMaxLive);
 constexpr size_t kOffIndeg = align256(kOffAcc + sizeof(int2) * kMaxN);
 constexpr size_t kOffRc = align256(kOffIndeg + sizeof(int32_t) * kMaxN);
@@ -56,7 +59,7 @@ constexpr size_t kOffDyn = align256(kOffDesc + sizeof(InstDesc));
 constexpr size_t kOffTiles = align256(kOffDyn + sizeof(InstDyn));
 constexpr size_t kOffRegInst = align256(kOffTiles + sizeof(int4) * kMaxTiles);
 constexpr size_t kOffCnt = align256(kOffRegInst + sizeof(int32_t) * kMaxR);
-constexpr size_t kOffBw = align256(kOffCnt + sizeof(int32_t) * kMaxR);
+constexpr size_t kOffBw = align256(kOffCnt + sizeof(int32_t) * 2 * kMaxR);
 constexpr size_t kOffYlast = align256(kOffBw + sizeof(double) * 4 * kMaxR);
 constexpr size_t kOffHcount = align256(kOffYlast + sizeof(double) * kMaxR);  // uint32[256]
 constexpr size_t kOffClosed = align256(kOffHcount + sizeof(uint32_t) * 256);  // int64[kMaxR]
@@ -161,7 +164,7 @@ extern "C" int dbnet_run_noalloc(const dbnet_device_graph_t* graph,
       raise(DBNET_EINVAL, "NULL argument");
     if (n_steps < 0 || raster_cap < 0 || (raster_cap > 0 && (!raster_step || !raster_id)))
       raise(DBNET_EINVAL, "bad step count or raster buffers");
-    // the update kernel moves whole tiles of V, J and ref with 16-byte bulk copies
+    // the update kernel moves V, J and ref as 16-byte vectors
     if ((reinterpret_cast<uintptr_t>(V) | reinterpret_cast<uintptr_t>(J) |
          reinterpret_cast<uintptr_t>(ref)) & 15u)
       raise(DBNET_EINVAL, "V, J and ref must be 16-byte aligned");
@@ -260,8 +263,8 @@ extern "C" int dbnet_run_noalloc(const dbnet_device_graph_t* graph,
     d.N = N;
     d.R = R;
     d.rbase = 0;
-    d.shift = 32;
-    d.tmask = 0xFFFFFFFFu;
+    d.shift = 24;  // targets lie below 2^24: the edge word is col | delay << 24
+    d.tmask = 0xFFFFFFu;
     d.two_S = std::ldexp(1.0f, S);
     d.inv_two_S = std::ldexp(1.0f, -S);
     d.spb = (int32_t)std::lrint(options->bin_ms / options->dt_ms);
@@ -303,9 +306,16 @@ extern "C" int dbnet_run_noalloc(const dbnet_device_graph_t* graph,
     e.V = V;
     e.J = J;
     e.ref = ref;
-    e.acc = reinterpret_cast<int2*>(at(kOffAcc));
+    // the spike ring's room holds the accumulator ring where that fits, and
+    // every edge is then added at emission
+    int32_t slots = 2;
+    while (slots < dmax + 1) slots *= 2;
+    const bool at_emission = (uint64_t)n_pad * (uint64_t)slots * sizeof(int2) <= sizeof(uint32_t) * kMaxLive;
+    e.mode = at_emission ? kAtEmission : kPerStep;
+    e.acc = reinterpret_cast<int2*>(at(at_emission ? kOffHist : kOffAcc));
     e.stride = n_pad;
-    e.acc_slots = 1;
+    e.acc_slots = at_emission ? slots : 1;
+    e.dmax = dmax;
     e.phases = 1;
     e.d_emit = dmax + 2;  // every delay at arrival time
     e.slot_emit = nullptr;
@@ -314,6 +324,7 @@ extern "C" int dbnet_run_noalloc(const dbnet_device_graph_t* graph,
     e.tile_info = reinterpret_cast<const int4*>(at(kOffTiles));
     e.closed = reinterpret_cast<long long*>(at(kOffClosed));
     e.cnt = reinterpret_cast<int32_t*>(at(kOffCnt));
+    e.cnt_stride = kMaxR;
     e.bw = reinterpret_cast<double*>(at(kOffBw));
     e.ylast = reinterpret_cast<double*>(at(kOffYlast));
     e.region_inst = reinterpret_cast<const int32_t*>(at(kOffRegInst));
@@ -331,7 +342,7 @@ extern "C" int dbnet_run_noalloc(const dbnet_device_graph_t* graph,
     const int grid = deliver_grid();
     for (int64_t k = 0; k < n_steps; ++k) {
       const StepRef sr{nullptr, (unsigned long long)k, nullptr};
-      launch_deliver(e, grid, sr, s);
+      if (!at_emission) launch_deliver(e, grid, sr, s);
       launch_update(e, sr, s);
     }
     launch_close(e, (unsigned long long)n_steps, s);

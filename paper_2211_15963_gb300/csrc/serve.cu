@@ -142,7 +142,7 @@ int32_t tiles_for(int32_t N) { return (N + kTile - 1) / kTile; }
 int64_t arena_estimate(const Req& r, int32_t dmax) {
   const dbnet_graph_t& g = r.graph;
   const int64_t N = g.n_neurons, E = g.row_ptr[N], R = g.n_regions;
-  const int64_t stride = (dmax + 7) / 8 * 8;
+  const int64_t stride = (dmax + 7) / 8 * 8 + kSegHead / 2;  // a table row, in counts
   const bool two = g.weight2 != nullptr;
   const int64_t stage = std::min<int64_t>(E, int64_t(1) << 27) * (two ? 13 : 9);
   return (two ? 8 : 6) * E + 8 * (N + 1) + 4 * stride * N + stage + 8 * N + 4 * (R + 1) +

@@ -36,7 +36,8 @@ def _equal(net, o):
 @pytest.mark.parametrize("form", ["plain", "current", "two_weights"])
 @pytest.mark.parametrize("sizes", [[1021, 6, 1025, 127, 130, 2050], [1024, 2048, 1021], [2051]])
 def test_update_region_edges(sizes, form):
-    g = synth.make_graph(sizes, 60, 31, k_within=5 if len(sizes) > 1 else 60, d_within=(1, 12), d_cross=(12, 40))
+    g = synth.make_graph(sizes, 40, 31, k_within=5 if len(sizes) > 1 else 40, d_within=(1, 12), d_cross=(12, 40),
+                         region_density=1.0)
     over = dict(ou_mu=0.05, ou_sigma=0.0, ou_tau=8.0, iext_shape=4.0) if form == "current" else {}
     p = [synth.default_region_params(I_ext=0.85 + 0.03 * r, **(over if r != 1 else {})) for r in range(len(sizes))]
     if form == "two_weights":
@@ -48,3 +49,58 @@ def test_update_region_edges(sizes, form):
     o.step(400)
     _equal(net, o)
     net.close()
+
+
+# Every delivery mode on the same spike trains: all edges at emission (small
+# ring), windows whose first edges the update adds, windows with the bounds
+# ring (forced by a large engine: many members), and one delay per step and
+# kernel (the pipelined schedule); step calls that start and end inside
+# windows and mix direct steps with replays; longest delays on and off a
+# multiple of the window, and shorter than one.
+@pytest.mark.parametrize("dmax,bin_ms", [(1, 0.0), (3, 0.0), (8, 0.0), (9, 0.0), (64, 0.0), (255, 0.0), (100, 0.7)])
+@pytest.mark.parametrize("schedule", [1, 2, 3])
+def test_delivery_modes(dmax, bin_ms, schedule):
+    from paper_2211_15963_gb300 import dbnet
+    sizes = [1500, 2300, 56_000] if dmax > 9 else [900, 1700]
+    g = synth.make_graph(sizes, 40, 7 + dmax, k_within=36, d_within=(1, max(1, dmax // 2)),
+                         d_cross=(max(1, dmax // 2), dmax), region_density=1.0)
+    p = [synth.default_region_params(I_ext=0.86 + 0.03 * r) for r in range(len(sizes))]
+    binned = dict(bin_spikes=1, bin_ms=bin_ms, tr_ms=10 * bin_ms) if bin_ms else dict(tr_ms=10.0)
+    net = dbnet.Network(g, p, dict(seed=9, raster_capacity=1 << 20, schedule=schedule, **binned))
+    o = oracle.Sim(g, p, seed=9, precision=32, **binned)
+    for n in (1, 3, 66, 1, 130, 5, 95):
+        net.step(n)
+        o.step(n)
+        assert net.stats()["events"] == o.info()["events"]
+    _equal(net, o)
+    net.close()
+
+
+def test_windows_of_a_large_engine():
+    """An ensemble wide enough that its delivery runs in windows with the
+    bounds ring and a kernel of its own for the rest of a window: the first,
+    a middle and the last member equal single networks (which add every edge
+    at emission)."""
+    from paper_2211_15963_gb300 import dbnet
+    g = synth.make_graph([700, 1100], 60, 3, k_within=48, d_within=(1, 20), d_cross=(20, 75))
+    base = [synth.default_region_params(I_ext=0.9)] * 2
+    M = 272
+    theta = np.random.default_rng(4).uniform(-0.5, 0.5, (M, 2, 2))
+    ens = dbnet.Ensemble(g, base, M, theta, dict(seed=8, net_id=40, raster_capacity=1 << 16))
+    for n in (5, 300, 1, 94):
+        ens.step(n)
+    for m in (0, 131, M - 1):
+        q = [dict(b) for b in base]
+        for r in range(2):
+            gu = list(q[r]["g_u"])
+            gu[0] *= float(np.exp(theta[m, r, 0]))
+            gu[2] *= float(np.exp(theta[m, r, 1]))
+            q[r]["g_u"] = tuple(gu)
+        net = dbnet.Network(g, q, dict(seed=8, net_id=40 + m, raster_capacity=1 << 16))
+        net.step(400)
+        for x, y in zip(ens.member_state(m), net.state()):
+            assert np.array_equal(x, y)
+        a, b = ens.member_spikes(m), net.spikes()
+        assert len(b[1]) > 500 and np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+        net.close()
+    ens.close()
