@@ -254,6 +254,15 @@ int deliver_grid();
 int persist_max_grid(const EngineDev& e);
 cudaError_t launch_persist(const EngineDev& e, int grid, unsigned long long g0, int nsteps,
                            unsigned* count, unsigned long long limit_ns, cudaStream_t s);
+// The resident stepper (kAtEmission): iterations g0 .. g0 + nsteps - 1 in one
+// launch of one thread-block cluster that holds the state in registers; also
+// closes the bin that ends with the last of them.  resident_fits(e): the
+// engine's tiles fit such a cluster on this device (call it before the first
+// launch and any capture: it opts the kernel in to 16 blocks).
+constexpr int kClusterBlocks = 16;
+constexpr int kResidentTiles = 4 * kClusterBlocks;
+bool resident_fits(const EngineDev& e);
+cudaError_t launch_resident(const EngineDev& e, unsigned long long g0, int nsteps, cudaStream_t s);
 // The grid barrier alone: rounds barriers over grid blocks of one
 // cooperative launch, each expecting extra arrivals more than the grid
 // makes (extra > 0: the first wait runs out and sets kFlagTimeout in *flags).

@@ -286,7 +286,7 @@ struct Engine {
   // a last turn weighs the best of those against it.
   Delivery rule{}, per_step{};
   int rule_grid = 0;
-  bool rule_persistent = false;
+  bool rule_persistent = false, rule_resident = false;
   bool weigh_rule = false;
   double best_ms = kDropped;          // the best per-step shape's last turn
   struct Shape {
@@ -316,6 +316,7 @@ struct Engine {
   static constexpr int kPersistSteps = 4096;
   static constexpr unsigned long long kBarrierLimitNs = 1000000000ull;
   bool persistent = false;
+  bool resident = false;  // by the resident stepper (then persistent, too)
   int persist_max = 0;
   bool persist_tunable = false;  // the tuner may weigh the persistent schedule
   DevBuf<unsigned> pbar;

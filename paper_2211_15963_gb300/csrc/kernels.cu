@@ -120,11 +120,11 @@ __device__ __forceinline__ void red_add_u64(unsigned long long* a, unsigned long
 #endif
 }
 
-// Forward-Euler step of the hemodynamic model for one region (FP64).
-__device__ double bw_euler(double* x, double z, const InstDesc& d) {
+// Forward-Euler step of the hemodynamic model for one region (FP64), from
+// its two powers fout = v^(1/alpha) and oe = (1 - rho)^(1/f).
+__device__ double bw_euler(double* x, double z, const InstDesc& d, double fout, double oe) {
   const double s = x[0], f = x[1], v = x[2], q = x[3];
-  const double fout = pow(v, 1.0 / d.alpha);
-  const double E = 1.0 - pow(1.0 - d.rho, 1.0 / f);
+  const double E = 1.0 - oe;
   const double ds = z - d.kappa * s - d.gamma * (f - 1.0);
   const double dv = (f - fout) / d.tau;
   const double dq = (f * E / d.rho - fout * q / v) / d.tau;
@@ -179,36 +179,55 @@ __device__ __forceinline__ unsigned long long step_of(const StepRef& sr) {
   return (sr.base ? *reinterpret_cast<const volatile unsigned long long*>(sr.base) : 0ull) + sr.off;
 }
 
-// Close the bin that ended with iteration g - 1 for region gr, once: the
+// Close the bins that ended with iteration g - 1, each once: the
 // Balloon-Windkessel step with that bin's activity, and the BOLD sample when
-// the bin ends a TR.
-__device__ void close_region(const EngineDev& e, int gr, unsigned long long g) {
-  const int k = e.region_inst[gr];
-  if (k < 0 || !e.dyn[k].active) return;  // unused region slot, or retired
-  const InstDesc& dk = e.insts[k];
-  if (g <= dk.g0) return;
-  const long long nk = (long long)(g - 1ull - dk.g0);  // step just completed
-  if (nk >= dk.n_end) return;                          // past the instance's last step
-  if ((nk + 1) % dk.spb != 0) return;
-  if (e.closed[gr] >= (long long)g) return;
-  const int r = gr - dk.rbase;
-  const double nr = (double)(dk.rc[r].end - dk.rc[r].start);
-  int32_t* const cnt = e.cnt + ((nk / dk.spb) & 1) * e.cnt_stride + gr;  // that bin's
-  const double z = dk.z_scale * (double)*cnt / nr;
-  *cnt = 0;
-  const double y = bw_euler(e.bw + 4 * gr, z, dk);
-  e.ylast[gr] = y;
-  const long long b = (nk + 1) / dk.spb;  // bins completed
-  if (b % dk.bins_per_tr == 0) {
-    const long long sidx = b / dk.bins_per_tr - 1;
-    if (sidx < dk.bold_cap) dk.bold[sidx * dk.R + r] = y;
+// the bin ends a TR.  Warps w, w + n, ... of the caller take 16 regions each,
+// a region on two lanes that compute one of its two powers (a power is some
+// 3 us of dependent FP64 operations, and on small networks everybody waits
+// for them).  Called by whole warps.
+__device__ void close_regions(const EngineDev& e, unsigned long long g, int w, int n) {
+  const int lane = threadIdx.x & 31;
+  for (int first = w * 16; first < e.total_R; first += n * 16) {
+    const int gr = first + (lane >> 1);
+    int k = -1;
+    long long nk = 0;
+    if (gr < e.total_R) {
+      k = e.region_inst[gr];
+      if (k >= 0 && !e.dyn[k].active) k = -1;  // unused region slot, or retired
+      if (k >= 0) {
+        const InstDesc& dk = e.insts[k];
+        nk = (long long)(g - 1ull - dk.g0);  // step just completed
+        if (g <= dk.g0 || nk >= dk.n_end || (nk + 1) % dk.spb != 0 || e.closed[gr] >= (long long)g) k = -1;
+      }
+    }
+    if (!__any_sync(kFull, k >= 0)) continue;
+    const InstDesc& dk = e.insts[k < 0 ? 0 : k];
+    double a = 1.0, x = 1.0;
+    if (k >= 0) {
+      a = (lane & 1) ? 1.0 - dk.rho : e.bw[4 * gr + 2];
+      x = 1.0 / ((lane & 1) ? e.bw[4 * gr + 1] : dk.alpha);
+    }
+    const double p = pow(a, x);
+    const double other = __shfl_xor_sync(kFull, p, 1);
+    if (k < 0 || (lane & 1)) continue;
+    const int r = gr - dk.rbase;
+    const double nr = (double)(dk.rc[r].end - dk.rc[r].start);
+    int32_t* const cnt = e.cnt + ((nk / dk.spb) & 1) * e.cnt_stride + gr;  // that bin's
+    const double z = dk.z_scale * (double)*cnt / nr;
+    *cnt = 0;
+    const double y = bw_euler(e.bw + 4 * gr, z, dk, p, other);
+    e.ylast[gr] = y;
+    const long long b = (nk + 1) / dk.spb;  // bins completed
+    if (b % dk.bins_per_tr == 0) {
+      const long long sidx = b / dk.bins_per_tr - 1;
+      if (sidx < dk.bold_cap) dk.bold[sidx * dk.R + r] = y;
+    }
+    e.closed[gr] = (long long)g;
   }
-  e.closed[gr] = (long long)g;
 }
 
 __global__ void k_close(EngineDev e, unsigned long long g) {
-  for (int gr = blockIdx.x * blockDim.x + threadIdx.x; gr < e.total_R; gr += gridDim.x * blockDim.x)
-    close_region(e, gr, g);
+  close_regions(e, g, (blockIdx.x * blockDim.x + threadIdx.x) >> 5, (gridDim.x * blockDim.x) >> 5);
 }
 
 __global__ void k_set_base(unsigned long long* base, unsigned long long g) { *base = g; }
@@ -261,6 +280,55 @@ struct EdgeView {
         two_w(d.two_w), two_S(d.two_S) {}
 };
 
+// One edge's additions: word and weights of a record of v, of a spike with
+// this key (handed on at a step with low bits key >> 1, class key & 1).
+//
+// FOUR: four accumulator channels per neuron; an edge adds its two weights
+// (the one weight twice for one-weight records) to the channel pair of the
+// source's class with one 64-bit atomic.  Every channel sum stays below 2^31
+// (the fixed-point scale is chosen so), so the low word never carries into
+// the high one.
+template <bool FOUR>
+__device__ __forceinline__ void add_edge(const EngineDev& e, const EdgeView& v, uint32_t word, uint32_t wts,
+                                         uint32_t key, unsigned long long pol_acc) {
+  const uint32_t slot = ((key >> 1) + (word >> v.shift)) & ((uint32_t)e.acc_slots - 1u);
+  const size_t at = (size_t)slot * (size_t)e.stride + (size_t)v.base + (word & v.tmask);
+  const int q = __float2int_rn(__fmul_rn(__uint_as_float(wts << 16), v.two_S));
+  if (FOUR) {
+    const int q2 = __float2int_rn(__fmul_rn(__uint_as_float(wts & 0xFFFF0000u), v.two_S));
+    red_add_u64(reinterpret_cast<unsigned long long*>(e.acc) + 2 * at + (key & 1u),
+                ((unsigned long long)(uint32_t)q2 << 32) | (uint32_t)q, pol_acc);
+  } else {
+    red_add_s32(reinterpret_cast<int*>(e.acc) + 2 * at + (key & 1u), q, pol_acc);
+  }
+}
+
+// Record ei of v: its word and its two weights (the one weight twice).
+template <bool FOUR>
+__device__ __forceinline__ void load_edge(const EdgeView& v, int64_t ei, uint32_t& word, uint32_t& wts,
+                                          unsigned long long pol_rec) {
+  if (FOUR && v.two_w) {  // 8-byte record: word, weight | second weight << 16
+    const uint2 r4 = ld_stream_u64(reinterpret_cast<const uint2*>(v.rec) + ei, pol_rec);
+    word = r4.x;
+    wts = r4.y;
+  } else if (v.rec) {
+    // 6-byte record at byte 6 ei: two aligned words cover it (the record
+    // array carries 8 bytes of padding at its end)
+    const size_t byte = 6 * (size_t)ei;
+    const uint32_t* w4 = reinterpret_cast<const uint32_t*>(
+        reinterpret_cast<const unsigned char*>(v.rec) + (byte & ~size_t(3)));
+    const uint32_t w0 = ld_stream_u32(w4, pol_rec), w1 = ld_stream_u32(w4 + 1, pol_rec);
+    const uint32_t sh = (uint32_t)(byte & 3u) * 8u;  // 0 or 16
+    word = __funnelshift_r(w0, w1, sh);
+    const uint32_t wb = (w1 >> sh) & 0xFFFFu;
+    wts = wb | (wb << 16);
+  } else {
+    word = __ldg(v.col + ei) | ((uint32_t)__ldg(v.delay + ei) << v.shift);
+    const uint32_t wb = __ldg(v.w + ei);
+    wts = wb | (wb << 16);
+  }
+}
+
 // Adds the warp's segments -- nseg edge records from e0 on, of a row of
 // instance inst (UNI: the first) whose spike was handed on at a step with low
 // bits key >> 1 and has class key & 1 -- each edge into the accumulator slot
@@ -273,12 +341,6 @@ struct EdgeView {
 // warp), so that an owner's data is one 16-byte read.  (A shuffle search per
 // chunk took 5 + 5 shuffles and more than twice the instructions, and the
 // walk is bound by its issue slots.)  Called by the whole warp.
-//
-// FOUR: four accumulator channels per neuron; an edge adds its two weights
-// (the one weight twice for one-weight records) to the channel pair of the
-// source's class with one 64-bit atomic.  Every channel sum stays below 2^31
-// (the fixed-point scale is chosen so), so the low word never carries into
-// the high one.
 template <bool FOUR, bool UNI>
 __device__ __forceinline__ void walk_segments(const EngineDev& e, const InstDesc* insts, int4* s_item,
                                               int64_t e0, uint32_t nseg, int inst, uint32_t key,
@@ -299,7 +361,6 @@ __device__ __forceinline__ void walk_segments(const EngineDev& e, const InstDesc
     s_item[__popc(full & ((1u << lane) - 1u))] = make_int4((int)(uint32_t)b, (int)(b >> 32), (int)key, inst);
   }
   __syncwarp();
-  const uint32_t smask = (uint32_t)e.acc_slots - 1u;
   const unsigned upto = 0xffffffffu >> (31 - lane);  // this lane and those before
   const EdgeView v0(insts[0]);
   int begun = -1;  // items that start before the chunk, less one
@@ -321,42 +382,13 @@ __device__ __forceinline__ void walk_segments(const EngineDev& e, const InstDesc
         ic[u] = UNI ? 0 : it.w;
         const int64_t ei = (int64_t)(((uint64_t)(uint32_t)it.y << 32) | (uint32_t)it.x) + (int64_t)fi;
         const EdgeView v(UNI ? v0 : EdgeView(insts[ic[u]]));
-        if (FOUR && v.two_w) {  // 8-byte record: word, weight | second weight << 16
-          const uint2 r4 = ld_stream_u64(reinterpret_cast<const uint2*>(v.rec) + ei, pol_rec);
-          tg[u] = r4.x;
-          wv[u] = r4.y;
-        } else if (v.rec) {
-          // 6-byte record at byte 6 ei: two aligned words cover it (the
-          // record array carries 8 bytes of padding at its end)
-          const size_t byte = 6 * (size_t)ei;
-          const uint32_t* w4 = reinterpret_cast<const uint32_t*>(
-              reinterpret_cast<const unsigned char*>(v.rec) + (byte & ~size_t(3)));
-          const uint32_t w0 = ld_stream_u32(w4, pol_rec), w1 = ld_stream_u32(w4 + 1, pol_rec);
-          const uint32_t sh = (uint32_t)(byte & 3u) * 8u;  // 0 or 16
-          tg[u] = __funnelshift_r(w0, w1, sh);
-          const uint32_t wb = (w1 >> sh) & 0xFFFFu;
-          wv[u] = wb | (wb << 16);
-        } else {
-          tg[u] = __ldg(v.col + ei) | ((uint32_t)__ldg(v.delay + ei) << v.shift);
-          const uint32_t wb = __ldg(v.w + ei);
-          wv[u] = wb | (wb << 16);
-        }
+        load_edge<FOUR>(v, ei, tg[u], wv[u], pol_rec);
       }
     }
 #pragma unroll
     for (int u = 0; u < kWalkU; ++u) {
       if (ic[u] < 0) continue;
-      const EdgeView v(UNI ? v0 : EdgeView(insts[ic[u]]));
-      const uint32_t slot = ((ky[u] >> 1) + (tg[u] >> v.shift)) & smask;
-      const size_t at = (size_t)slot * (size_t)e.stride + (size_t)v.base + (tg[u] & v.tmask);
-      const int q = __float2int_rn(__fmul_rn(__uint_as_float(wv[u] << 16), v.two_S));
-      if (FOUR) {
-        const int q2 = __float2int_rn(__fmul_rn(__uint_as_float(wv[u] & 0xFFFF0000u), v.two_S));
-        red_add_u64(reinterpret_cast<unsigned long long*>(e.acc) + 2 * at + (ky[u] & 1u),
-                    ((unsigned long long)(uint32_t)q2 << 32) | (uint32_t)q, pol_acc);
-      } else {
-        red_add_s32(reinterpret_cast<int*>(e.acc) + 2 * at + (ky[u] & 1u), q, pol_acc);
-      }
+      add_edge<FOUR>(e, UNI ? v0 : EdgeView(insts[ic[u]]), tg[u], wv[u], ky[u], pol_acc);
     }
   }
   __syncwarp();  // s_item is read
@@ -375,11 +407,27 @@ __device__ __forceinline__ uint32_t edges_up_to(const InstDesc& dd, const unsign
 
 // Region constants of a thread's four neurons: one region's for all (ONE), or
 // each neuron's own.
-template <bool ONE>
+// HELD: they may lie in shared memory (the resident steppers), else they are
+// read through the L1's read-only path.
+template <bool ONE, bool HELD>
 struct QuadConst {
   const RegionConst* p;  // the tile's first region
   int r[ONE ? 1 : 4];    // the neurons' regions, counted from it
   __device__ __forceinline__ const RegionConst& of(int k) const { return ONE ? *p : p[r[ONE ? 0 : k]]; }
+  template <class T>
+  static __device__ __forceinline__ T ld(const T* a) {
+    return HELD ? *a : __ldg(a);
+  }
+  // the regions of neurons li0 .. li0 + m - 1
+  __device__ __forceinline__ void find(int32_t li0, int m) {
+    int at = 0;
+#pragma unroll
+    for (int k = 0; k < (ONE ? 0 : 4); ++k) {
+      if (k < m)
+        while (li0 + k >= ld(&p[at].end)) ++at;
+      r[ONE ? 0 : k] = at;
+    }
+  }
 };
 
 // What the membrane step of a thread's four neurons leaves: bit k of spk and
@@ -388,85 +436,107 @@ struct QuadSpikes {
   unsigned spk = 0, cls = 0;
 };
 
-// One Euler step of the thread's four neurons (m of them exist).  The traces
-// go channel by channel over the four, so that only one channel's constants
-// and one float4 of traces are live at a time, and each float4 is stored as
-// soon as it is updated.
-template <bool EXT, bool FOUR, bool ONE>
-__device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDesc& d, const QuadConst<ONE>& rc,
-                                                int m, int64_t gi0, int32_t li0, long long n,
-                                                float4 V4, const float4 (&J4)[4], uchar4 rf, const int4 (&A)[FOUR ? 4 : 2]) {
+// A step's random draws of the thread's four neurons: what the background
+// drive adds to AMPA and NMDA, and the normals of the OU current where the
+// instance has it.  They depend on the step alone.
+struct QuadDraw {
+  int dq[4];
+  float xi[4];
+};
+template <bool EXT, bool ONE, bool HELD>
+__device__ __forceinline__ QuadDraw quad_draw(const InstDesc& d, const QuadConst<ONE, HELD>& rc, int32_t li0,
+                                              long long n) {
+  QuadDraw o;
   unsigned long long x[4] = {(unsigned long long)n, (unsigned long long)(li0 >> 2), 0ull, 0ull};
   philox4x64_10(x, d.seed, d.net_id);
   // background: Poisson count by integer inversion of 32 Philox bits (the
-  // thresholds are non-decreasing: count them up to the first miss), added
-  // to AMPA and NMDA
-  int dq[4];
+  // thresholds are non-decreasing: count them up to the first miss)
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     const RegionConst& p = rc.of(k);
     const uint32_t uu = (uint32_t)(x[k] >> 32);
-    const int n_thr = __ldg(&p.n_thr);
+    const int n_thr = rc.ld(&p.n_thr);
     int c = 0;
-    while (c < n_thr && uu >= __ldg(&p.thr[c])) ++c;
-    dq[k] = c * __ldg(&p.q_ext);
+    while (c < n_thr && uu >= rc.ld(&p.thr[c])) ++c;
+    o.dq[k] = c * rc.ld(&p.q_ext);
   }
-  const float v[4] = {V4.x, V4.y, V4.z, V4.w};
+  if (EXT && (d.ext & kExtOU)) {  // the OU noise: stream 4
+    unsigned long long xo[4] = {(unsigned long long)n, (unsigned long long)(li0 >> 2), 4ull, 0ull};
+    philox4x64_10(xo, d.seed, d.net_id);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) o.xi[k] = normal_from_word(xo[k]);
+  }
+  return o;
+}
+
+// State of the thread's four neurons.
+struct QuadState {
+  float4 V, J[4], B;  // B: the background current, where the instance has it
+  uchar4 ref;
+};
+__device__ __forceinline__ void quad_load(const EngineDev& e, int64_t gi0, QuadState& q) {
+  // (state is streamed once per step: evict-first, so that the delivery's
+  // working set keeps the L2)
+  q.V = __ldcs(reinterpret_cast<const float4*>(e.V + gi0));
+#pragma unroll
+  for (int u = 0; u < 4; ++u) q.J[u] = __ldcs(reinterpret_cast<const float4*>(e.J + u * e.stride + gi0));
+  q.ref = __ldcs(reinterpret_cast<const uchar4*>(e.ref + gi0));
+}
+
+// One Euler step of the thread's four neurons (m of them exist).  The traces
+// go channel by channel over the four, so that only one channel's constants
+// are live at a time.  HELD: the state stays in q (the resident steppers);
+// else each vector is stored as soon as it is updated.
+template <bool EXT, bool FOUR, bool ONE, bool HELD>
+__device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDesc& d, const QuadConst<ONE, HELD>& rc,
+                                                int m, int64_t gi0, int32_t li0, const QuadDraw& draw,
+                                                QuadState& q, const int4 (&A)[FOUR ? 4 : 2]) {
+  const float v[4] = {q.V.x, q.V.y, q.V.z, q.V.w};
   float Isyn[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
   for (int u = 0; u < 4; ++u) {  // the membrane sees the old V and traces
-    const float jo[4] = {J4[u].x, J4[u].y, J4[u].z, J4[u].w};
+    const float jo[4] = {q.J[u].x, q.J[u].y, q.J[u].z, q.J[u].w};
     float jn[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
       const RegionConst& p = rc.of(k);
-      const float gj = __fmul_rn(__ldg(&p.g[u]), jo[k]);
-      const float dv = __fsub_rn(__ldg(&p.Vu[u]), v[k]);
+      const float gj = __fmul_rn(rc.ld(&p.g[u]), jo[k]);
+      const float dv = __fsub_rn(rc.ld(&p.Vu[u]), v[k]);
       Isyn[k] = __fadd_rn(Isyn[k], __fmul_rn(gj, dv));
       // traces: decay, then this step's arrivals
       const int4 Ak = FOUR ? A[k] : A[k >> 1];
-      const int q = FOUR ? (u == 0 ? Ak.x : u == 1 ? Ak.y : u == 2 ? Ak.z : Ak.w)
+      const int a = FOUR ? (u == 0 ? Ak.x : u == 1 ? Ak.y : u == 2 ? Ak.z : Ak.w)
                          : ((k & 1) ? (u < 2 ? Ak.z : Ak.w) : (u < 2 ? Ak.x : Ak.y));
-      const float xu = __fmul_rn(__int2float_rn(u < 2 ? q + dq[k] : q), d.inv_two_S);
-      jn[k] = __fadd_rn(__fmul_rn(__ldg(&p.dec[u]), jo[k]), xu);
+      const float xu = __fmul_rn(__int2float_rn(u < 2 ? a + draw.dq[k] : a), d.inv_two_S);
+      jn[k] = __fadd_rn(__fmul_rn(rc.ld(&p.dec[u]), jo[k]), xu);
     }
-    if (m == 4) {
-      __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + gi0), make_float4(jn[0], jn[1], jn[2], jn[3]));
-    } else {  // the last neurons of an instance: the padding keeps its values
-      __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + gi0),
-             make_float4(jn[0], m > 1 ? jn[1] : jo[1], m > 2 ? jn[2] : jo[2], jo[3]));
-    }
+    // (the last neurons of an instance: the padding keeps its values)
+    q.J[u] = make_float4(jn[0], m > 1 ? jn[1] : jo[1], m > 2 ? jn[2] : jo[2], m > 3 ? jn[3] : jo[3]);
+    if (!HELD) __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + gi0), q.J[u]);
   }
   // the background current and the injected-current factors, only where the
   // instance has them (a request server's engine runs this variant for
   // every request)
   const bool ou = EXT && (d.ext & kExtOU), het = EXT && (d.ext & kExtHet);
-  float4 B4 = make_float4(0.f, 0.f, 0.f, 0.f), F4 = make_float4(1.f, 1.f, 1.f, 1.f);
-  if (ou) B4 = __ldcs(reinterpret_cast<const float4*>(e.Ibg + gi0));
+  float4 F4 = make_float4(1.f, 1.f, 1.f, 1.f);
+  if (ou && !HELD) q.B = __ldcs(reinterpret_cast<const float4*>(e.Ibg + gi0));
   if (het) F4 = __ldg(reinterpret_cast<const float4*>(e.fext + gi0));
-  float ib[4] = {B4.x, B4.y, B4.z, B4.w};
+  float ib[4] = {q.B.x, q.B.y, q.B.z, q.B.w};
   const float fe[4] = {F4.x, F4.y, F4.z, F4.w};
-  unsigned long long xo[4] = {0ull, 0ull, 0ull, 0ull};
-  if (ou) {  // the OU noise: stream 4
-    xo[0] = (unsigned long long)n;
-    xo[1] = (unsigned long long)(li0 >> 2);
-    xo[2] = 4ull;
-    philox4x64_10(xo, d.seed, d.net_id);
-  }
   float vo[4];
-  int rr[4] = {rf.x, rf.y, rf.z, rf.w};
+  int rr[4] = {q.ref.x, q.ref.y, q.ref.z, q.ref.w};
   QuadSpikes out;
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
     vo[k] = v[k];
     if (k >= m) continue;
     const RegionConst& p = rc.of(k);
-    const float4 M = __ldg(reinterpret_cast<const float4*>(&p.dtC));     // dtC gL VL Vth
-    const float4 Q = __ldg(reinterpret_cast<const float4*>(&p.Vreset));  // Vreset Iext n_ref q_ext
+    const float4 M = rc.ld(reinterpret_cast<const float4*>(&p.dtC));     // dtC gL VL Vth
+    const float4 Q = rc.ld(reinterpret_cast<const float4*>(&p.Vreset));  // Vreset Iext n_ref q_ext
     const float leak = __fmul_rn(M.y, __fsub_rn(v[k], M.z));
     float I = __fsub_rn(Isyn[k], leak);
     float4 OUc = make_float4(0.f, 0.f, 0.f, 0.f);  // mu, dt/tau, sigma sqrt(2 dt/tau), bits
-    if (EXT && d.ext) OUc = __ldg(reinterpret_cast<const float4*>(&p.ou_mu));
+    if (EXT && d.ext) OUc = rc.ld(reinterpret_cast<const float4*>(&p.ou_mu));
     const int xb = __float_as_int(OUc.w);
     // injected current, scaled by the neuron's factor where heterogeneous
     const float ie = (EXT && (xb & kExtHet)) ? __fmul_rn(Q.y, fe[k]) : Q.y;
@@ -474,10 +544,9 @@ __device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDe
     if (EXT && (xb & kExtOU)) I = __fadd_rn(I, ib[k]);  // I_bg before this step
     const float vn = __fadd_rn(v[k], __fmul_rn(I, M.x));
     if (EXT && (xb & kExtOU)) {  // Eq. 1, Euler-Maruyama
-      const float xi = normal_from_word(xo[k]);
       const float t1 = __fmul_rn(__fsub_rn(OUc.x, ib[k]), OUc.y);
       ib[k] = __fadd_rn(ib[k], t1);
-      ib[k] = __fadd_rn(ib[k], __fmul_rn(OUc.z, xi));
+      ib[k] = __fadd_rn(ib[k], __fmul_rn(OUc.z, draw.xi[k]));
     }
     // refractory clamp, threshold, reset
     if (rr[k] > 0) {
@@ -487,16 +556,165 @@ __device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDe
       vo[k] = Q.x;
       rr[k] = __float_as_int(Q.z);
       out.spk |= 1u << k;
-      if (li0 + k >= __ldg(&p.exc_end)) out.cls |= 1u << k;
+      if (li0 + k >= rc.ld(&p.exc_end)) out.cls |= 1u << k;
     } else {
       vo[k] = vn;
     }
   }
-  __stcs(reinterpret_cast<float4*>(e.V + gi0), make_float4(vo[0], vo[1], vo[2], vo[3]));
-  __stcs(reinterpret_cast<uchar4*>(e.ref + gi0),
-         make_uchar4((unsigned char)rr[0], (unsigned char)rr[1], (unsigned char)rr[2], (unsigned char)rr[3]));
-  if (ou) __stcs(reinterpret_cast<float4*>(e.Ibg + gi0), make_float4(ib[0], ib[1], ib[2], ib[3]));
+  q.V = make_float4(vo[0], vo[1], vo[2], vo[3]);
+  q.ref = make_uchar4((unsigned char)rr[0], (unsigned char)rr[1], (unsigned char)rr[2], (unsigned char)rr[3]);
+  if (ou) q.B = make_float4(ib[0], ib[1], ib[2], ib[3]);
+  if (!HELD) {
+    __stcs(reinterpret_cast<float4*>(e.V + gi0), q.V);
+    __stcs(reinterpret_cast<uchar4*>(e.ref + gi0), q.ref);
+    if (ou) __stcs(reinterpret_cast<float4*>(e.Ibg + gi0), q.B);
+  }
   return out;
+}
+
+// A warp's place: its tile's instance and regions, and its lanes' neurons.
+struct WarpPlace {
+  int inst, r0, nr, m;  // m: neurons of the thread that exist
+  int64_t gi0;
+  int32_t li0;
+};
+
+// What a block keeps of a tile in shared memory while its state is held: a
+// barrier between steps empties the L1, and every constant would come from
+// the L2 again.
+constexpr int kHeldRegions = 8;
+struct HeldTile {
+  InstDesc d;
+  RegionConst rc[kHeldRegions];
+  int64_t row0;             // first edge of the tile's rows, -1: not held
+  uint32_t row[kTile + 1];  // and of each row, from there
+};
+// The spikes of a warp's neurons in iteration g (step n of the instance):
+// counts, ring append, and the edges that are due soon.  Called by the whole
+// warp; s_item has 32 entries per warp of the block.
+template <bool FOUR>
+__device__ __forceinline__ void warp_spikes(const EngineDev& e, const InstDesc& d, const WarpPlace& w,
+                                            unsigned long long g, long long n, QuadSpikes qs, int4* s_item,
+                                            const HeldTile* held = nullptr) {
+  const int lane = threadIdx.x & 31;
+  const unsigned spk = qs.spk, cls_bits = qs.cls;
+  if (!__any_sync(kFull, spk != 0)) return;
+  const int nsp = __popc(spk);
+  int ps = nsp;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int t = __shfl_up_sync(kFull, ps, o);
+    if (lane >= o) ps += t;
+  }
+  const int total = __shfl_sync(kFull, ps, 31);
+  // the step at which these spikes are handed on: this step, or with spike
+  // binning the last step of its bin
+  const long long bin = div_steps(n, d.spb);
+  const unsigned long long rel = d.bin_sp ? d.g0 + (unsigned long long)((bin + 1) * d.spb - 1) : g;
+  const int slot = e.mode == kAtEmission ? 0
+                   : (int)((rel >> 32) ? rel % (unsigned long long)e.D : (uint32_t)rel % (uint32_t)e.D);
+  int32_t* const cnt = e.cnt + (bin & 1) * e.cnt_stride + d.rbase + w.r0;
+  uint32_t hbase = 0;
+  unsigned long long rbase = 0;
+  if (lane == 31) {
+    if (e.mode != kAtEmission) hbase = atomicAdd(e.hcount + slot, (uint32_t)ps);
+    atomicAdd(&e.dyn[w.inst].spikes, (unsigned long long)ps);
+    if (d.raster_cap > 0) rbase = atomicAdd(&e.dyn[w.inst].raster_count, (unsigned long long)ps);
+    if (w.nr == 1) atomicAdd(cnt, ps);
+  }
+  hbase = __shfl_sync(kFull, hbase, 31);
+  rbase = __shfl_sync(kFull, rbase, 31);
+  // the longest delay whose edges this warp adds: up to the end of the window
+  // in which the spikes are handed on, or every delay
+  const int dnow = e.mode == kAtEmission ? d.dmax
+                   : e.push_now ? min(e.wmask - (int)((unsigned)rel & (unsigned)e.wmask), d.dmax)
+                                : 0;
+  unsigned long long ev = 0;
+  // spike i of the warp goes to lane i mod 32: its owner by a shuffle search
+  // over the inclusive counts, its neuron the owner's bit of that rank
+  for (int i0 = 0; i0 < total; i0 += 32) {
+    const int i = i0 + lane;
+    int o = 0;
+#pragma unroll
+    for (int step = 16; step > 0; step >>= 1) {
+      const int v = __shfl_sync(kFull, ps, o + step - 1);
+      if (v <= i) o += step;
+    }
+    o = o < 32 ? o : 31;
+    unsigned bits = __shfl_sync(kFull, spk, o);
+    const unsigned inh = __shfl_sync(kFull, cls_bits, o);
+    int rank = i - (__shfl_sync(kFull, ps, o) - __popc(bits));
+    const int rk = w.nr == 1 ? 0 : -1;
+    int64_t e0 = 0;
+    uint32_t nseg = 0, key = 0;
+    int k = 0;
+    if (i < total) {
+      while (rank-- > 0) bits &= bits - 1u;
+      k = __ffs(bits) - 1;
+      const int32_t lo = w.li0 - lane * 4 + o * 4 + k;  // the neuron
+      const unsigned cl = (inh >> k) & 1u;
+      if (e.mode != kAtEmission) {
+        const uint64_t pos = (uint64_t)hbase + (uint32_t)i;
+        if (pos < (uint64_t)e.hist_cap)
+          e.hist[(size_t)slot * (size_t)e.hist_cap + pos] = (uint32_t)(d.base + lo) | (cl << 31);
+        else
+          atomicOr(e.flags, kFlagHistOverflow);
+      }
+      if (d.raster_cap > 0 && rbase + (unsigned)i < (unsigned long long)d.raster_cap) {
+        d.raster_step[rbase + (unsigned)i] = (int32_t)n;
+        d.raster_id[rbase + (unsigned)i] = lo;
+      }
+      if (rk < 0) {
+        int r = 0;
+        while (lo >= __ldg(&d.rc[w.r0 + r].end)) ++r;
+        atomicAdd(cnt + r, 1);
+      }
+      if (dnow > 0) {
+        key = ((uint32_t)rel << 1) | cl;
+        if (e.mode == kAtEmission) {  // the whole row
+          if (held && held->row0 >= 0) {
+            const uint32_t* row = held->row + (lo & (kTile - 1));  // (an instance starts on a tile)
+            e0 = held->row0 + row[0];
+            nseg = row[1] - row[0];
+          } else {
+            e0 = __ldg(d.row_ptr + lo);
+            nseg = (uint32_t)(__ldg(d.row_ptr + lo + 1) - e0);
+          }
+          ev += nseg;
+        } else {
+          const unsigned char* row = seg_row(d, lo);
+          e0 = __ldg(reinterpret_cast<const longlong2*>(row)).x;
+          nseg = edges_up_to(d, row, dnow);
+        }
+      }
+    }
+    if (dnow <= 0) continue;
+    if (total == 1) {  // most often: lane 0 has it, the lanes take its records in turn
+      e0 = __shfl_sync(kFull, e0, 0);
+      nseg = __shfl_sync(kFull, nseg, 0);
+      key = __shfl_sync(kFull, key, 0);
+      const EdgeView v(d);
+      const unsigned long long first = l2_policy_first(), last = l2_policy_last();
+      for (uint32_t f = lane; f < nseg; f += 32u * kWalkU) {
+        uint32_t word[kWalkU], wts[kWalkU];
+#pragma unroll
+        for (int u = 0; u < kWalkU; ++u)
+          if (f + 32u * u < nseg) load_edge<FOUR>(v, e0 + f + 32u * u, word[u], wts[u], first);
+#pragma unroll
+        for (int u = 0; u < kWalkU; ++u)
+          if (f + 32u * u < nseg) add_edge<FOUR>(e, v, word[u], wts[u], key, last);
+      }
+      __syncwarp();
+      continue;
+    }
+    walk_segments<FOUR, true>(e, &d, s_item + (threadIdx.x >> 5) * 32, e0, nseg, 0, key, l2_policy_first(),
+                              l2_policy_last());
+  }
+  if (e.mode == kAtEmission) {  // the synaptic events of these spikes
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
+    if (lane == 0 && ev) atomicAdd(e.events, ev);
+  }
 }
 
 // One warp's 128 neurons of a tile, in the iteration sr names.
@@ -522,158 +740,58 @@ __device__ __forceinline__ QuadSpikes quad_step(const EngineDev& e, const InstDe
 template <bool EXT, bool FOUR>
 __device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& sr, int tile, int warp,
                                             int4* s_item) {
-  const int lane = threadIdx.x & 31;
   // state loads first: they depend only on the tile, and the arrays cover
   // every padded tile
-  const int64_t gi0 = (int64_t)tile * kTile + warp * 128 + lane * 4;
-  // (state is streamed once per step: evict-first, so that the delivery's
-  // working set keeps the L2)
-  const float4 V4 = __ldcs(reinterpret_cast<const float4*>(e.V + gi0));
-  float4 J4[4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) J4[u] = __ldcs(reinterpret_cast<const float4*>(e.J + u * e.stride + gi0));
-  const uchar4 rf = __ldcs(reinterpret_cast<const uchar4*>(e.ref + gi0));
+  WarpPlace w;
+  w.gi0 = (int64_t)tile * kTile + warp * 128 + (threadIdx.x & 31) * 4;
+  QuadState q;
+  quad_load(e, w.gi0, q);
   const int4 ti = __ldg(e.tile_info + tile);  // instance, first region, regions touched
   // this step's arrivals: one int4 per neuron (AMPA, NMDA, GABA_A, GABA_B)
   // or per two (E, I of each), from the accumulator slot of this iteration
   const unsigned long long g = step_of(sr);
   constexpr int kA = FOUR ? 4 : 2;
-  int4* const accs = reinterpret_cast<int4*>(acc_of(e, g)) + (FOUR ? gi0 : gi0 / 2);
+  int4* const accs = reinterpret_cast<int4*>(acc_of(e, g)) + (FOUR ? w.gi0 : w.gi0 / 2);
   int4 A[kA];
 #pragma unroll
   for (int k = 0; k < kA; ++k) A[k] = __ldcg(accs + k);
 
   if (sr.next && threadIdx.x == 0) *sr.next = g + 1ull;
   if (ti.x < 0) return;  // unused tile
-  const int inst = ti.x, r0 = ti.y;
-  const InstDesc& d = e.insts[inst];
+  w.inst = ti.x;
+  w.r0 = ti.y;
+  w.nr = ti.z;
+  const InstDesc& d = e.insts[w.inst];
   const long long n = (long long)(g - d.g0);
-  if (e.dyn[inst].active == 0 || n >= d.n_end) return;
-  const int32_t li0 = (int32_t)(gi0 - d.base);
-  const int m = d.N - li0 < 4 ? d.N - li0 : 4;  // neurons of the thread that exist
-  const RegionConst* rcp = d.rc + r0;
-  QuadConst<true> one{rcp, {0}};
-  QuadConst<false> each{rcp, {0, 0, 0, 0}};
+  if (e.dyn[w.inst].active == 0 || n >= d.n_end) return;
+  w.li0 = (int32_t)(w.gi0 - d.base);
+  w.m = d.N - w.li0 < 4 ? d.N - w.li0 : 4;
+  const QuadConst<true, false> one{d.rc + w.r0, {0}};
+  QuadConst<false, false> each{d.rc + w.r0, {0, 0, 0, 0}};
   QuadSpikes qs;
-  if (m > 0) {
+  if (w.m > 0) {
 #pragma unroll
     for (int k = 0; k < kA; ++k) accs[k] = make_int4(0, 0, 0, 0);
-    if (ti.z == 1) {  // the whole tile lies in one region
-      qs = quad_step<EXT, FOUR, true>(e, d, one, m, gi0, li0, n, V4, J4, rf, A);
+    if (w.nr == 1) {  // the whole tile lies in one region
+      qs = quad_step<EXT, FOUR, true, false>(e, d, one, w.m, w.gi0, w.li0, quad_draw<EXT>(d, one, w.li0, n), q, A);
     } else {
-      int r = 0;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        if (k < m)
-          while (li0 + k >= __ldg(&rcp[r].end)) ++r;
-        each.r[k] = r;
-      }
-      qs = quad_step<EXT, FOUR, false>(e, d, each, m, gi0, li0, n, V4, J4, rf, A);
+      each.find(w.li0, w.m);
+      qs = quad_step<EXT, FOUR, false, false>(e, d, each, w.m, w.gi0, w.li0, quad_draw<EXT>(d, each, w.li0, n), q, A);
     }
   }
-  const unsigned spk = qs.spk, cls_bits = qs.cls;
+  warp_spikes<FOUR>(e, d, w, g, n, qs, s_item);
+}
 
-  // ---- spikes: counts, ring append, and the edges that are due soon -------
-  if (!__any_sync(kFull, spk != 0)) return;
-  const int nsp = __popc(spk);
-  int ps = nsp;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int t = __shfl_up_sync(kFull, ps, o);
-    if (lane >= o) ps += t;
-  }
-  const int total = __shfl_sync(kFull, ps, 31);
-  // the step at which these spikes are handed on: this step, or with spike
-  // binning the last step of its bin
-  const long long bin = div_steps(n, d.spb);
-  const unsigned long long rel = d.bin_sp ? d.g0 + (unsigned long long)((bin + 1) * d.spb - 1) : g;
-  const int slot = e.mode == kAtEmission ? 0
-                   : (int)((rel >> 32) ? rel % (unsigned long long)e.D : (uint32_t)rel % (uint32_t)e.D);
-  int32_t* const cnt = e.cnt + (bin & 1) * e.cnt_stride + d.rbase + r0;
-  uint32_t hbase = 0;
-  unsigned long long rbase = 0;
-  if (lane == 31) {
-    if (e.mode != kAtEmission) hbase = atomicAdd(e.hcount + slot, (uint32_t)ps);
-    atomicAdd(&e.dyn[inst].spikes, (unsigned long long)ps);
-    if (d.raster_cap > 0) rbase = atomicAdd(&e.dyn[inst].raster_count, (unsigned long long)ps);
-    if (ti.z == 1) atomicAdd(cnt, ps);
-  }
-  hbase = __shfl_sync(kFull, hbase, 31);
-  rbase = __shfl_sync(kFull, rbase, 31);
-  // the longest delay whose edges this warp adds: up to the end of the window
-  // in which the spikes are handed on, or every delay
-  const int dnow = e.mode == kAtEmission ? d.dmax
-                   : e.push_now ? min(e.wmask - (int)((unsigned)rel & (unsigned)e.wmask), d.dmax)
-                                : 0;
-  unsigned long long ev = 0;
-  // spike i of the warp goes to lane i mod 32: its owner by a shuffle search
-  // over the inclusive counts, its neuron the owner's bit of that rank
-  for (int i0 = 0; i0 < total; i0 += 32) {
-    const int i = i0 + lane;
-    int o = 0;
-#pragma unroll
-    for (int step = 16; step > 0; step >>= 1) {
-      const int v = __shfl_sync(kFull, ps, o + step - 1);
-      if (v <= i) o += step;
-    }
-    o = o < 32 ? o : 31;
-    unsigned bits = __shfl_sync(kFull, spk, o);
-    const unsigned inh = __shfl_sync(kFull, cls_bits, o);
-    int rank = i - (__shfl_sync(kFull, ps, o) - __popc(bits));
-    const int rk = ti.z == 1 ? 0 : -1;
-    int64_t e0 = 0;
-    uint32_t nseg = 0, key = 0;
-    int k = 0;
-    if (i < total) {
-      while (rank-- > 0) bits &= bits - 1u;
-      k = __ffs(bits) - 1;
-      const int32_t lo = li0 - lane * 4 + o * 4 + k;  // the neuron
-      const unsigned cl = (inh >> k) & 1u;
-      if (e.mode != kAtEmission) {
-        const uint64_t pos = (uint64_t)hbase + (uint32_t)i;
-        if (pos < (uint64_t)e.hist_cap)
-          e.hist[(size_t)slot * (size_t)e.hist_cap + pos] = (uint32_t)(d.base + lo) | (cl << 31);
-        else
-          atomicOr(e.flags, kFlagHistOverflow);
-      }
-      if (d.raster_cap > 0 && rbase + (unsigned)i < (unsigned long long)d.raster_cap) {
-        d.raster_step[rbase + (unsigned)i] = (int32_t)n;
-        d.raster_id[rbase + (unsigned)i] = lo;
-      }
-      if (rk < 0) {
-        int r = 0;
-        while (lo >= __ldg(&rcp[r].end)) ++r;
-        atomicAdd(cnt + r, 1);
-      }
-      if (dnow > 0) {
-        key = ((uint32_t)rel << 1) | cl;
-        if (e.mode == kAtEmission) {  // the whole row
-          e0 = __ldg(d.row_ptr + lo);
-          nseg = (uint32_t)(__ldg(d.row_ptr + lo + 1) - e0);
-          ev += nseg;
-        } else {
-          const unsigned char* row = seg_row(d, lo);
-          e0 = __ldg(reinterpret_cast<const longlong2*>(row)).x;
-          nseg = edges_up_to(d, row, dnow);
-        }
-      }
-    }
-    if (dnow > 0)
-      walk_segments<FOUR, true>(e, &d, s_item + (threadIdx.x >> 5) * 32, e0, nseg, 0, key, l2_policy_first(), l2_policy_last());
-  }
-  if (e.mode == kAtEmission) {  // the synaptic events of these spikes
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
-    if (lane == 0 && ev) atomicAdd(e.events, ev);
-  }
+// Blocks of the update that close bins: a warp for 16 regions.
+__host__ __device__ __forceinline__ int close_blocks(const EngineDev& e) {
+  return (e.total_R + 16 * (kUpdThreads / 32) - 1) / (16 * (kUpdThreads / 32));
 }
 
 template <bool EXT, bool FOUR>
 __global__ void __launch_bounds__(kUpdThreads, 7) k_update(EngineDev e, StepRef sr) {
-  const int n_close = (e.total_R + kUpdThreads - 1) / kUpdThreads;
+  const int n_close = close_blocks(e);
   if ((int)blockIdx.x < n_close) {  // close the bins that ended with the previous iteration
-    const int gr = blockIdx.x * kUpdThreads + threadIdx.x;
-    if (gr < e.total_R) close_region(e, gr, step_of(sr));
+    close_regions(e, step_of(sr), blockIdx.x * (kUpdThreads / 32) + (threadIdx.x >> 5), n_close * (kUpdThreads / 32));
     return;
   }
   const int w = (blockIdx.x - n_close) * (kUpdThreads / 32) + (threadIdx.x >> 5);
@@ -1394,12 +1512,14 @@ __device__ __forceinline__ void red_release_add_u32(unsigned* a, unsigned v) {
 // after limit_ns of the global timer, or as soon as another block has given
 // up (kFlagTimeout set in *flags), it gives up too, sets kFlagTimeout, and
 // every thread of the block gets false.
-__device__ bool grid_barrier(unsigned* count, unsigned target, unsigned long long limit_ns,
-                             unsigned* flags) {
-  __shared__ int s_ok;
+__device__ __forceinline__ void grid_arrive(unsigned* count) {
   __syncthreads();
+  if (threadIdx.x == 0) red_release_add_u32(count, 1u);
+}
+
+__device__ bool grid_wait(unsigned* count, unsigned target, unsigned long long limit_ns, unsigned* flags) {
+  __shared__ int s_ok;
   if (threadIdx.x == 0) {
-    red_release_add_u32(count, 1u);
     int ok = 1;
     const unsigned long long t0 = global_ns();
     for (unsigned spin = 0; (int)(ld_acquire_u32(count) - target) < 0; ++spin) {
@@ -1420,18 +1540,126 @@ __device__ bool grid_barrier(unsigned* count, unsigned target, unsigned long lon
   return s_ok != 0;
 }
 
+__device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, unsigned long long limit_ns,
+                                             unsigned* flags) {
+  grid_arrive(count);
+  return grid_wait(count, target, limit_ns, flags);
+}
+
+// by the tile's 256 threads, a block barrier after it
+__device__ __forceinline__ void held_load(const EngineDev& e, int tile, HeldTile& h) {
+  if (tile >= e.n_tiles) return;
+  const int4 ti = __ldg(e.tile_info + tile);
+  if (ti.x < 0) return;
+  const InstDesc& d = e.insts[ti.x];
+  const int t = threadIdx.x % (kTile / 4);
+  const uint32_t* from = reinterpret_cast<const uint32_t*>(&d);
+  for (int w = t; w < (int)(sizeof(InstDesc) / 4); w += kTile / 4) reinterpret_cast<uint32_t*>(&h.d)[w] = from[w];
+  if (e.mode == kAtEmission) {
+    const int32_t lo = (int32_t)((int64_t)tile * kTile - d.base);
+    const int rows = d.N - lo < kTile ? d.N - lo : kTile;
+    const int64_t r0 = d.row_ptr[lo];
+    const bool fits = (unsigned long long)(d.row_ptr[lo + rows] - r0) < (1ull << 32);
+    if (t == 0) h.row0 = fits ? r0 : -1;
+    for (int k = t; k <= rows; k += kTile / 4) h.row[k] = (uint32_t)(d.row_ptr[lo + k] - r0);
+  }
+  if (ti.z > kHeldRegions) return;
+  from = reinterpret_cast<const uint32_t*>(d.rc + ti.y);
+  for (int w = t; w < ti.z * (int)(sizeof(RegionConst) / 4); w += kTile / 4)
+    reinterpret_cast<uint32_t*>(h.rc)[w] = from[w];
+}
+
+// A warp's 128 neurons with their state in registers over many steps.
+template <bool EXT, bool FOUR>
+struct HeldWarp {
+  WarpPlace w;
+  QuadState q;
+  QuadConst<true, true> one;
+  QuadConst<false, true> each;
+  QuadDraw draw;
+  const InstDesc* d;
+  const HeldTile* tile;
+  bool ou;
+
+  __device__ __forceinline__ HeldWarp(const EngineDev& e, int t, int warp, const HeldTile& h) : tile(&h) {
+    w.inst = -1;
+    w.m = w.r0 = w.nr = 0;
+    w.li0 = 0;
+    w.gi0 = (int64_t)t * kTile + warp * 128 + (threadIdx.x & 31) * 4;
+    if (t < e.n_tiles) {
+      quad_load(e, w.gi0, q);
+      const int4 ti = __ldg(e.tile_info + t);
+      if (ti.x >= 0 && e.dyn[ti.x].active != 0) w.inst = ti.x;
+      w.r0 = ti.y;
+      w.nr = ti.z;
+    }
+    d = &h.d;
+    ou = false;
+    if (w.inst >= 0) {
+      one.p = each.p = w.nr <= kHeldRegions ? h.rc : d->rc + w.r0;
+      w.li0 = (int32_t)(w.gi0 - d->base);
+      w.m = d->N - w.li0 < 4 ? d->N - w.li0 : 4;
+      if (w.nr > 1) each.find(w.li0, w.m);
+      ou = EXT && (d->ext & kExtOU);
+      if (ou) q.B = __ldcs(reinterpret_cast<const float4*>(e.Ibg + w.gi0));
+    }
+  }
+  // the random draws of iteration g
+  __device__ __forceinline__ void prepare(unsigned long long g) {
+    if (w.m <= 0) return;
+    const long long n = (long long)(g - d->g0);
+    draw = w.nr == 1 ? quad_draw<EXT>(*d, one, w.li0, n) : quad_draw<EXT>(*d, each, w.li0, n);
+  }
+  // iteration g, prepared; the whole warp
+  __device__ __forceinline__ void step(const EngineDev& e, unsigned long long g, int4* s_item) {
+    if (w.inst < 0) return;  // warp-uniform, as the next
+    const long long n = (long long)(g - d->g0);
+    if (n >= d->n_end) return;
+    QuadSpikes qs;
+    if (w.m > 0) {
+      constexpr int kA = FOUR ? 4 : 2;
+      int4* const accs = reinterpret_cast<int4*>(acc_of(e, g)) + (FOUR ? w.gi0 : w.gi0 / 2);
+      int4 A[kA];
+#pragma unroll
+      for (int k = 0; k < kA; ++k) A[k] = __ldcg(accs + k);
+#pragma unroll
+      for (int k = 0; k < kA; ++k) accs[k] = make_int4(0, 0, 0, 0);
+      qs = w.nr == 1 ? quad_step<EXT, FOUR, true, true>(e, *d, one, w.m, w.gi0, w.li0, draw, q, A)
+                     : quad_step<EXT, FOUR, false, true>(e, *d, each, w.m, w.gi0, w.li0, draw, q, A);
+    }
+    __syncwarp();
+    warp_spikes<FOUR>(e, *d, w, g, n, qs, s_item, tile);
+  }
+  __device__ __forceinline__ void store(const EngineDev& e) {
+    if (w.m <= 0) return;
+    __stcs(reinterpret_cast<float4*>(e.V + w.gi0), q.V);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) __stcs(reinterpret_cast<float4*>(e.J + u * e.stride + w.gi0), q.J[u]);
+    __stcs(reinterpret_cast<uchar4*>(e.ref + w.gi0), q.ref);
+    if (ou) __stcs(reinterpret_cast<float4*>(e.Ibg + w.gi0), q.B);
+  }
+};
+
 // The persistent stepper: iterations g0 .. g0 + nsteps - 1 in one
 // cooperative launch, each the delivery where the mode has one (the whole
 // grid) and the update (tiles dealt round robin over the blocks), with a grid
 // barrier after each.  The same device functions as the launched step do
 // the work, so the results are identical bit for bit; a barrier that gives
 // up ends the launch (kFlagTimeout stays set for the host).
-template <bool EXT, bool FOUR, bool SINGLE, bool PER_STEP>
+template <bool EXT, bool FOUR, bool SINGLE, bool PER_STEP, bool HELD>
 __global__ void __launch_bounds__(kDelThreads, 2)
     k_persist(EngineDev e, unsigned long long g0, int nsteps, unsigned* count,
               unsigned long long limit_ns) {
   __shared__ int4 s_item[kDelThreads];
+  const int warp = threadIdx.x >> 5;
   unsigned target = 0;
+  __shared__ HeldTile s_tile;
+  if (HELD) {
+    held_load(e, blockIdx.x, s_tile);
+    __syncthreads();
+  }
+  HeldWarp<EXT, FOUR> h(e, HELD ? (int)blockIdx.x : e.n_tiles, warp, s_tile);
+  if (HELD) h.prepare(g0);
   for (int s = 0; s < nsteps; ++s) {
     const unsigned long long g = g0 + (unsigned long long)s;
     const StepRef sr{nullptr, g, nullptr};
@@ -1444,14 +1672,64 @@ __global__ void __launch_bounds__(kDelThreads, 2)
       target += gridDim.x;
       if (!grid_barrier(count, target, limit_ns, e.flags)) return;
     }
-    for (int gr = (gridDim.x - 1 - blockIdx.x) * kDelThreads + threadIdx.x; gr < e.total_R;
-         gr += gridDim.x * kDelThreads)
-      close_region(e, gr, g);  // the last blocks: the first ones have the most tiles
-    for (int t = blockIdx.x; t < e.n_tiles; t += gridDim.x)
-      update_warp<EXT, FOUR>(e, sr, t, threadIdx.x >> 5, s_item);
+    // the last blocks: the first ones have the most tiles
+    close_regions(e, g, (gridDim.x - 1 - blockIdx.x) * (kDelThreads / 32) + warp, gridDim.x * (kDelThreads / 32));
     target += gridDim.x;
-    if (!grid_barrier(count, target, limit_ns, e.flags)) return;
+    if (HELD) {
+      h.step(e, g, s_item);
+      grid_arrive(count);
+      h.prepare(g + 1ull);  // under the barrier
+      if (!grid_wait(count, target, limit_ns, e.flags)) return;
+    } else {
+      for (int t = blockIdx.x; t < e.n_tiles; t += gridDim.x)
+        update_warp<EXT, FOUR>(e, sr, t, warp, s_item);
+      if (!grid_barrier(count, target, limit_ns, e.flags)) return;
+    }
   }
+  if (HELD) h.store(e);
+}
+
+// The resident stepper of small networks (kAtEmission, at most 64 tiles):
+// iterations g0 .. g0 + nsteps - 1 in one launch of one thread-block cluster
+// of at most 16 blocks, each holding the state of its THREADS / 256 tiles in
+// registers.  A step is the arrivals' load from the L2, the membrane step,
+// the rows of the step's spikes and one hardware cluster barrier, under which
+// the next step's random draws are made; nothing else leaves the registers,
+// and nothing is launched between steps.
+//
+// Bound: the latency of that chain, not traffic.  4.4 us a step at 10,000
+// neurons and 8 spikes a step (2.0 the arrivals, the membrane step and the
+// barrier, some 2 the spikes' rows, 0.4 the bins), 6.6 at 30,000 and 9.1 at
+// 60,000 (four tiles a block: 64 registers, spills); with a launch per step
+// 7.4, 12.4 and 14, and 13.2, 25 and 27 with two.  The grid barrier of the
+// persistent stepper costs 1.1 to 1.2 us by itself.  Constants and row starts
+// in registers' reach (HeldTile) took 0.6 us off, a region's two powers on two
+// lanes and the short way for a lone spike 0.7.
+template <bool EXT, bool FOUR, int THREADS>
+__global__ void __launch_bounds__(THREADS, 1) k_resident(EngineDev e, unsigned long long g0, int nsteps) {
+  __shared__ int4 s_item[THREADS];
+  const int warp = threadIdx.x >> 5;
+  __shared__ HeldTile s_tile[THREADS / (kTile / 4)];
+  const int tile = blockIdx.x * (THREADS / (kTile / 4)) + warp / kTileWarps;
+  held_load(e, tile, s_tile[warp / kTileWarps]);
+  __syncthreads();
+  HeldWarp<EXT, FOUR> h(e, tile, warp % kTileWarps, s_tile[warp / kTileWarps]);
+  const auto close = [&](unsigned long long g) {  // one block closes the bins, the last: it has the fewest tiles
+    if (blockIdx.x == gridDim.x - 1) close_regions(e, g, warp, THREADS / 32);
+  };
+  h.prepare(g0);
+  for (int s = 0; s < nsteps; ++s) {
+    const unsigned long long g = g0 + (unsigned long long)s;
+    h.step(e, g, s_item);
+    close(g);
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    h.prepare(g + 1ull);
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  }
+  close(g0 + (unsigned long long)nsteps);
+  h.store(e);
 }
 
 // The grid barrier alone, rounds times, with extra arrivals expected per
@@ -1601,7 +1879,7 @@ void launch_init_state(const EngineDev& e, int inst, int n_tiles_inst, int first
 }
 
 void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s) {
-  const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads) + (e.total_R + kUpdThreads - 1) / kUpdThreads;
+  const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads) + close_blocks(e);
   if (e.four) {
     if (e.any_ext) k_update<true, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
     else k_update<false, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
@@ -1612,7 +1890,7 @@ void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s) {
 }
 
 void launch_close(const EngineDev& e, unsigned long long g, cudaStream_t s) {
-  const int blocks = (e.total_R + 127) / 128;
+  const int blocks = (e.total_R + 63) / 64;  // a warp for 16 regions
   k_close<<<blocks > 0 ? blocks : 1, 128, 0, s>>>(e, g);
 }
 
@@ -1659,17 +1937,20 @@ void launch_windows(const EngineDev& e, int grid, StepRef sr, bool first, cudaSt
 
 namespace {
 
-// f(kernel) for the stepper's variant that suits the engine
+// f(kernel) for the stepper's variant that suits the engine on grid blocks
 template <bool EXT, bool FOUR, class F>
-auto with_persist(const EngineDev& e, F&& f) {
+auto with_persist(const EngineDev& e, int grid, F&& f) {
+  const bool one = e.n_inst == 1;
   if (e.mode == kPerStep)
-    return e.n_inst == 1 ? f(k_persist<EXT, FOUR, true, true>) : f(k_persist<EXT, FOUR, false, true>);
-  return e.n_inst == 1 ? f(k_persist<EXT, FOUR, true, false>) : f(k_persist<EXT, FOUR, false, false>);
+    return one ? f(k_persist<EXT, FOUR, true, true, false>) : f(k_persist<EXT, FOUR, false, true, false>);
+  if (grid >= e.n_tiles)
+    return one ? f(k_persist<EXT, FOUR, true, false, true>) : f(k_persist<EXT, FOUR, false, false, true>);
+  return one ? f(k_persist<EXT, FOUR, true, false, false>) : f(k_persist<EXT, FOUR, false, false, false>);
 }
 template <class F>
-auto with_persist(const EngineDev& e, F&& f) {
-  if (e.four) return e.any_ext ? with_persist<true, true>(e, f) : with_persist<false, true>(e, f);
-  return e.any_ext ? with_persist<true, false>(e, f) : with_persist<false, false>(e, f);
+auto with_persist(const EngineDev& e, int grid, F&& f) {
+  if (e.four) return e.any_ext ? with_persist<true, true>(e, grid, f) : with_persist<false, true>(e, grid, f);
+  return e.any_ext ? with_persist<true, false>(e, grid, f) : with_persist<false, false>(e, grid, f);
 }
 
 }  // namespace
@@ -1678,10 +1959,15 @@ int persist_max_grid(const EngineDev& e) {
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  const cudaError_t r = with_persist(e, [&](auto k) {
-    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kDelThreads, 0);
-  });
-  return r == cudaSuccess ? sms * occ : 0;
+  int least = 1 << 20;  // of the variants it may take
+  for (int grid : {0, 1 << 30}) {
+    const cudaError_t r = with_persist(e, grid, [&](auto k) {
+      return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kDelThreads, 0);
+    });
+    if (r != cudaSuccess) return 0;
+    least = occ < least ? occ : least;
+  }
+  return sms * least;
 }
 
 cudaError_t launch_persist(const EngineDev& e, int grid, unsigned long long g0, int nsteps,
@@ -1692,8 +1978,66 @@ cudaError_t launch_persist(const EngineDev& e, int grid, unsigned long long g0, 
   if (r != cudaSuccess) return r;
   EngineDev ea = e;
   void* args[] = {&ea, &g0, &nsteps, &count, &limit_ns};
-  return with_persist(e, [&](auto k) {
+  return with_persist(e, grid, [&](auto k) {
     return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kDelThreads), args, 0, s);
+  });
+}
+
+namespace {
+
+// The resident stepper's variant for the engine's tiles: threads per block
+// (256, 512 or 1,024) and blocks (a power of two, the cluster).
+template <bool EXT, bool FOUR, class F>
+cudaError_t with_resident(const EngineDev& e, F&& f) {
+  int blocks = 1;
+  const int per = e.n_tiles <= kClusterBlocks ? 1 : e.n_tiles <= 2 * kClusterBlocks ? 2 : 4;
+  while (blocks * per < e.n_tiles) blocks *= 2;
+  if (per == 1) return f(k_resident<EXT, FOUR, 256>, blocks, 256);
+  if (per == 2) return f(k_resident<EXT, FOUR, 512>, blocks, 512);
+  return f(k_resident<EXT, FOUR, 1024>, blocks, 1024);
+}
+template <class F>
+cudaError_t with_resident(const EngineDev& e, F&& f) {
+  if (e.four) return e.any_ext ? with_resident<true, true>(e, f) : with_resident<false, true>(e, f);
+  return e.any_ext ? with_resident<true, false>(e, f) : with_resident<false, false>(e, f);
+}
+
+}  // namespace
+
+bool resident_fits(const EngineDev& e) {
+  if (e.mode != kAtEmission || e.n_tiles < 1 || e.n_tiles > kResidentTiles) return false;
+  int clusters = 0;
+  const cudaError_t r = with_resident(e, [&](auto k, int blocks, int threads) {
+    cudaError_t a = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    if (a != cudaSuccess) return a;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaOccupancyMaxActiveClusters(&clusters, k, &cfg);
+  });
+  if (r != cudaSuccess) cudaGetLastError();  // not a failure of the engine
+  return r == cudaSuccess && clusters > 0;
+}
+
+cudaError_t launch_resident(const EngineDev& e, unsigned long long g0, int nsteps, cudaStream_t s) {
+  return with_resident(e, [&](auto k, int blocks, int threads) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = blocks;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, e, g0, nsteps);
   });
 }
 

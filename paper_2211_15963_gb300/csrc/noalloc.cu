@@ -340,7 +340,14 @@ extern "C" int dbnet_run_noalloc(const dbnet_device_graph_t* graph,
 
     launch_init_state(e, 0, n_tiles, 0, s);
     const int grid = deliver_grid();
-    for (int64_t k = 0; k < n_steps; ++k) {
+    int64_t k = 0;
+    if (at_emission && resident_fits(e))  // (every size this entry point takes)
+      while (k < n_steps) {
+        const int c = (int)std::min<int64_t>(n_steps - k, 4096);
+        CK(launch_resident(e, (unsigned long long)k, c, s));
+        k += c;
+      }
+    for (; k < n_steps; ++k) {
       const StepRef sr{nullptr, (unsigned long long)k, nullptr};
       if (!at_emission) launch_deliver(e, grid, sr, s);
       launch_update(e, sr, s);

@@ -104,3 +104,31 @@ def test_windows_of_a_large_engine():
         assert len(b[1]) > 500 and np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
         net.close()
     ens.close()
+
+
+# The resident stepper holds one, two or four tiles a block on up to 16
+# blocks, the persistent one a tile a block on one or two blocks an SM: sizes
+# on and past each edge, more regions in a tile than a block keeps, every
+# form of the update, and calls of one step and of many.
+@pytest.mark.parametrize("sizes,form", [([40], "plain"), ([1024], "two_weights"), ([16_000, 384], "plain"),
+                                        ([16_385], "current"), ([90] * 30, "plain"), ([90] * 30, "current"),
+                                        ([32_768], "two_weights"), ([33_000], "plain"), ([65_536], "current"),
+                                        ([66_000], "plain"), ([156_000], "current"), ([100_000, 58_000], "two_weights")])
+def test_steppers_that_hold_the_state(sizes, form):
+    from paper_2211_15963_gb300 import dbnet
+    R = len(sizes)
+    k = min(24, sum(sizes) - 1)
+    g = synth.make_graph(sizes, k, 17, k_within=max(1, k - 2) if R > 1 else k, d_within=(1, 9), d_cross=(9, 14),
+                         region_density=1.0)
+    over = dict(ou_mu=0.05, ou_sigma=0.0, ou_tau=8.0, iext_shape=4.0) if form == "current" else {}
+    p = [synth.default_region_params(I_ext=0.86 + 0.01 * (r % 5), **(over if r != 1 else {})) for r in range(R)]
+    if form == "two_weights":
+        g = synth.with_second_weight(g, 5)
+    net = dbnet.Network(g, p, dict(seed=6, raster_capacity=1 << 21, tr_ms=5.0))
+    assert net.stats()["schedule"] == 3
+    o = oracle.Sim(g, p, seed=6, tr_ms=5.0, precision=32)
+    for n in (1, 9, 10, 1, 129, 50):
+        net.step(n)
+        o.step(n)
+    _equal(net, o)
+    net.close()
