@@ -350,7 +350,7 @@ int ens_create(const dbnet_graph_t* graph, const dbnet_region_params_t* base, in
     for (int64_t i = 0; i < (int64_t)M * R * 2; ++i)
       if (!std::isfinite(log_scale_init[i])) raise(DBNET_EINVAL, "non-finite initial log scale");
     cudaStream_t s = (cudaStream_t)cuda_stream;
-    auto g = upload_graph(graph, s);
+    auto g = upload_graph(graph, s, options->emit_delay == 0);
     std::vector<InstSpec> specs((size_t)M);
     for (int m = 0; m < M; ++m) {
       InstSpec& sp = specs[(size_t)m];

@@ -196,7 +196,8 @@ struct GraphDev {
   double w_max = 0.0;
   // the smallest delay from which every delay carries fewer than
   // kEmitSegEdges edges per row on average (estimated on a sample of rows),
-  // or 0 when there is none: those short segments are handed on at emission
+  // or 0 when there is none (or nobody asked): those short segments are handed
+  // on at emission
   int32_t emit_from = 0;
 };
 constexpr double kEmitSegEdges = 4.0;
@@ -382,7 +383,8 @@ struct Engine {
   int64_t bold_samples(int k) const;
 };
 
-std::shared_ptr<GraphDev> upload_graph(const dbnet_graph_t* g, cudaStream_t s);
+// emit_estimate: also estimate GraphDev::emit_from, which only emit_delay 0 uses
+std::shared_ptr<GraphDev> upload_graph(const dbnet_graph_t* g, cudaStream_t s, bool emit_estimate);
 // min_ref: the fewest refractory steps a region may have (spike binning)
 void check_params(const dbnet_region_params_t& p, double dt, int32_t min_ref);
 int32_t bin_lead(const dbnet_options_t& o);

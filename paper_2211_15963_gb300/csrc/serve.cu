@@ -256,7 +256,7 @@ bool admit(dbsrv* s, Req& r) {
   try {
     ArenaScope scope(&s->arena);
     if (!gd) {
-      gd = upload_graph(&r.graph, s->up);
+      gd = upload_graph(&r.graph, s->up, false);  // servers add nothing at emission by threshold
       if (r.rq.graph_key) s->shared[r.rq.graph_key] = gd;
     }
     double wext_max = 0.0;
