@@ -59,10 +59,14 @@ __device__ __forceinline__ int find_region(const int32_t* __restrict__ ro, int R
 #define DBNET_L2_HINTS 1
 #endif
 // 32-edge chunks of a warp's walk whose record loads are issued before the
-// first of their atomics (memory-level parallelism of the walk).
+// first of their atomics (memory-level parallelism of the walk): two measured
+// 97.8 / 129.5 us a step at 5 M neurons and for the 64-member ensemble, four
+// 99.1 / 131.4, eight 104.6 / 138.5.  A lone spike's row takes four at once:
+// nothing else covers its latency.
 #ifndef DBNET_WALK_CHUNKS
-#define DBNET_WALK_CHUNKS 4
+#define DBNET_WALK_CHUNKS 2
 #endif
+constexpr int kLoneU = 4;
 constexpr int kWalkU = DBNET_WALK_CHUNKS;
 constexpr int kSegGroup = 32;  // spikes per transposition group of the segment-ring copy
 constexpr int kTileWarps = kTile / 128;  // warps of an update tile, 128 neurons each
@@ -695,13 +699,13 @@ __device__ __forceinline__ void warp_spikes(const EngineDev& e, const InstDesc& 
       key = __shfl_sync(kFull, key, 0);
       const EdgeView v(d);
       const unsigned long long first = l2_policy_first(), last = l2_policy_last();
-      for (uint32_t f = lane; f < nseg; f += 32u * kWalkU) {
-        uint32_t word[kWalkU], wts[kWalkU];
+      for (uint32_t f = lane; f < nseg; f += 32u * kLoneU) {
+        uint32_t word[kLoneU], wts[kLoneU];
 #pragma unroll
-        for (int u = 0; u < kWalkU; ++u)
+        for (int u = 0; u < kLoneU; ++u)
           if (f + 32u * u < nseg) load_edge<FOUR>(v, e0 + f + 32u * u, word[u], wts[u], first);
 #pragma unroll
-        for (int u = 0; u < kWalkU; ++u)
+        for (int u = 0; u < kLoneU; ++u)
           if (f + 32u * u < nseg) add_edge<FOUR>(e, v, word[u], wts[u], key, last);
       }
       __syncwarp();
@@ -782,6 +786,15 @@ __device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& s
   warp_spikes<FOUR>(e, d, w, g, n, qs, s_item);
 }
 
+// Programmatic dependent launch: the kernels of a step are launched while
+// their predecessor still runs, wait here for its end and its writes, and let
+// their successor be launched in turn once all their blocks have started
+// (nothing, on an ordinary launch).
+__device__ __forceinline__ void step_after() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 // Blocks of the update that close bins: a warp for 16 regions.
 __host__ __device__ __forceinline__ int close_blocks(const EngineDev& e) {
   return (e.total_R + 16 * (kUpdThreads / 32) - 1) / (16 * (kUpdThreads / 32));
@@ -789,6 +802,7 @@ __host__ __device__ __forceinline__ int close_blocks(const EngineDev& e) {
 
 template <bool EXT, bool FOUR>
 __global__ void __launch_bounds__(kUpdThreads, 7) k_update(EngineDev e, StepRef sr) {
+  step_after();
   const int n_close = close_blocks(e);
   if ((int)blockIdx.x < n_close) {  // close the bins that ended with the previous iteration
     close_regions(e, step_of(sr), blockIdx.x * (kUpdThreads / 32) + (threadIdx.x >> 5), n_close * (kUpdThreads / 32));
@@ -1321,11 +1335,13 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
     s_items[threadIdx.x] = acc;
   }
   __syncthreads();
-  // items per unit: 32, or fewer when that would leave warps without one
+  // items per unit: 32, or fewer when that would leave some warps with one and
+  // others with two (100 -> 93 us a step at 4 M neurons with 50,000 spikes of
+  // 100 edges)
   uint32_t all = 0;
   for (int q = 0; q < Q; ++q) all += s_items[q];
   int ub = 5;
-  while (ub > 0 && (all >> ub) < (uint32_t)nblk * (kDelThreads / 32)) --ub;
+  while (ub > 0 && (all >> ub) < 2u * (uint32_t)nblk * (kDelThreads / 32)) --ub;
   if (threadIdx.x == 0) {
     s_unit[0] = 0u;
     for (int q = 0; q < kMaxPhases; ++q) s_unit[q + 1] = s_unit[q] + ((s_items[q] + (1u << ub) - 1u) >> ub);
@@ -1336,7 +1352,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
   const uint32_t n_units = s_unit[kMaxPhases];
   const unsigned long long pol_rec = l2_policy_first(), pol_acc = l2_policy_last();
 
-  // A unit of 32 items is four runs of eight consecutive ones, a quarter of
+  // A unit of 8 to 32 items is four runs of consecutive ones, a quarter of
   // the phase apart: the buckets hold segments of very different lengths
   // (short delays within a region, long ones across), so every unit gets an
   // even share, and a run's bounds lie side by side in the ring.
@@ -1353,7 +1369,8 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
     for (int step = kMaxPhases / 2; step > 0; step >>= 1)
       if (q + step < Q && s_unit[q + step] <= u) q += step;
     const uint32_t U = s_unit[q + 1] - s_unit[q], v = u - s_unit[q];
-    const uint32_t x = ub == 5 ? ((uint32_t)lane >> 3) * (U * 8u) + v * 8u + (lane & 7) : (v << ub) + lane;
+    const int rb = ub >= 3 ? ub - 2 : ub;  // a run's length, or the unit's
+    const uint32_t x = ((uint32_t)lane >> rb) * (U << rb) + (v << rb) + (lane & ((1 << rb) - 1));
     if (x >= s_items[q]) return it;
     int lo = 0;  // the bucket: the largest with s_pre[q][lo] <= x
 #pragma unroll
@@ -1404,7 +1421,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
     if (d0 > d1) return;
     const uint32_t a = d0 >= 2 ? edges_up_to(dd, row, d0 - 1) : 0u;
     e0 = r.x + a;
-    n = edges_up_to(dd, row, d1) - a;
+    n = (d1 == dd.dmax ? (uint32_t)(r.y - r.x) : edges_up_to(dd, row, d1)) - a;
   };
   const uint32_t stride = (uint32_t)nblk * (kDelThreads / 32);
   uint32_t u = (uint32_t)bid * (kDelThreads / 32) + warp;
@@ -1441,7 +1458,7 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
   const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
   const uint32_t warps = (uint32_t)nblk * (kDelThreads / 32);
   int ub = 5;
-  while (ub > 0 && (c >> ub) < warps) --ub;
+  while (ub > 0 && (c >> ub) < 2u * warps) --ub;
   const uint32_t n_units = (uint32_t)(((unsigned long long)c + (1u << ub) - 1u) >> ub);
   for (uint32_t u = (uint32_t)bid * (kDelThreads / 32) + warp; u < n_units; u += warps) {
     const uint32_t k = (u << ub) + lane;
@@ -1455,8 +1472,9 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
       if (inst >= 0) {
         const InstDesc& dd = e.insts[inst];
         const unsigned char* row = seg_row(dd, gidx - dd.base);
-        e0 = __ldg(reinterpret_cast<const longlong2*>(row)).x;
-        nseg = edges_up_to(dd, row, left < dd.dmax ? left : dd.dmax);
+        const longlong2 r = __ldg(reinterpret_cast<const longlong2*>(row));
+        e0 = r.x;
+        nseg = left < dd.dmax ? edges_up_to(dd, row, left) : (uint32_t)(r.y - r.x);
         key = ((uint32_t)(g - 1ull) << 1) | (ent >> 31);
       } else {
         inst = 0;
@@ -1473,12 +1491,14 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
 
 template <bool FOUR, bool SINGLE>
 __global__ void __launch_bounds__(kDelThreads, 4) k_windows(EngineDev e, StepRef sr) {
+  step_after();
   deliver_windows<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x);
 }
 
 template <bool FOUR, bool SINGLE>
 __global__ void __launch_bounds__(kDelThreads, 4) k_rest(EngineDev e, StepRef sr) {
   __shared__ int4 s_item[kDelThreads];
+  step_after();
   deliver_rest<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x, s_item);
 }
 
@@ -1878,14 +1898,36 @@ void launch_init_state(const EngineDev& e, int inst, int n_tiles_inst, int first
   if (n_tiles_inst > 0) k_init_state<<<n_tiles_inst, kTile / 4, 0, s>>>(e, inst, first_tile);
 }
 
+namespace {
+
+// A step kernel's launch.  Up to 2,048 tiles it need not wait for its
+// predecessor on the stream to end (step_after in the kernel does): that
+// took a step of 2 M neurons from 54.7 to 53.1 us and one of 500,000 in
+// columns from 19.2 to 18.4; at 4 and 5 M neurons it cost one of 98 us 1.2.
+template <class... Par, class... Arg>
+void launch_after(void (*k)(Par...), int grid, int threads, cudaStream_t s, const EngineDev& e, Arg... arg) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(threads);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = e.n_tiles <= 2048 ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, k, e, arg...);  // (errors by cudaGetLastError, as for <<<>>>)
+}
+
+}  // namespace
+
 void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s) {
   const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads) + close_blocks(e);
   if (e.four) {
-    if (e.any_ext) k_update<true, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
-    else k_update<false, true><<<blocks, kUpdThreads, 0, s>>>(e, sr);
+    if (e.any_ext) launch_after(k_update<true, true>, blocks, kUpdThreads, s, e, sr);
+    else launch_after(k_update<false, true>, blocks, kUpdThreads, s, e, sr);
   } else {
-    if (e.any_ext) k_update<true, false><<<blocks, kUpdThreads, 0, s>>>(e, sr);
-    else k_update<false, false><<<blocks, kUpdThreads, 0, s>>>(e, sr);
+    if (e.any_ext) launch_after(k_update<true, false>, blocks, kUpdThreads, s, e, sr);
+    else launch_after(k_update<false, false>, blocks, kUpdThreads, s, e, sr);
   }
 }
 
@@ -1923,8 +1965,7 @@ void launch_deliver(const EngineDev& e, int grid, StepRef sr, cudaStream_t s, in
 
 void launch_windows(const EngineDev& e, int grid, StepRef sr, bool first, cudaStream_t s) {
   auto go = [&](auto kw, auto kr) {
-    if (first) kw<<<grid, kDelThreads, 0, s>>>(e, sr);
-    else kr<<<grid, kDelThreads, 0, s>>>(e, sr);
+    launch_after(first ? kw : kr, grid, kDelThreads, s, e, sr);
   };
   if (e.n_inst == 1) {
     if (e.four) go(k_windows<true, true>, k_rest<true, true>);
