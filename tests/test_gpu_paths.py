@@ -132,3 +132,55 @@ def test_steppers_that_hold_the_state(sizes, form):
         o.step(n)
     _equal(net, o)
     net.close()
+
+
+def test_noalloc_beyond_the_accumulator_ring():
+    """Delays too long for the allocation-free scratch to hold an accumulator
+    slot each (40,960 padded neurons x 64 slots): it delivers per step, and
+    gives what a handle gives; two steps short of that ring it fits."""
+    from paper_2211_15963_gb300 import dbnet
+    for n, dmax in ((40_000, 60), (32_000, 62)):
+        g = synth.make_graph([n], 30, 23, d_within=(1, dmax))
+        p = synth.default_region_params(I_ext=0.9)
+        n_pad = -(-n // 1024) * 1024
+        t = lambda a: torch.from_numpy(np.ascontiguousarray(a)).cuda()  # noqa: E731
+        V, J = torch.empty(n_pad, device="cuda"), torch.empty(4, n_pad, device="cuda")
+        ref = torch.empty(n_pad, dtype=torch.uint8, device="cuda")
+        n_sp, n_ev = dbnet.dbnet_run_noalloc(n, g.region_offsets, g.n_exc, t(g.row_ptr), t(g.col),
+                                             t(np.asarray(g.w_bf16).view(np.int16)), t(g.delay), p, dict(seed=4), 250,
+                                             V, J, ref)
+        net = dbnet.Network(g, p, dict(seed=4))
+        net.step(250)
+        Vn, Jn, rn = net.state()
+        s = net.stats()
+        assert n_sp == s["spikes"] > 500 and n_ev == s["events"]
+        assert np.array_equal(V[:n].cpu().numpy(), Vn) and np.array_equal(J[:, :n].cpu().numpy(), Jn)
+        assert np.array_equal(ref[:n].cpu().numpy(), rn)
+        net.close()
+
+
+@pytest.mark.parametrize("max_neurons,max_delay", [(8_192, 40), (1 << 20, 200)])
+def test_server_tunes_with_requests_in_flight(max_neurons, max_delay):
+    """A server whose launch shapes are tuned from its first rounds on, while
+    requests come and go: its delivery changes from the mode of its size (at
+    emission; windows) to per step and back with spikes in flight, and every
+    request equals the same network alone."""
+    from paper_2211_15963_gb300 import dbnet
+    srv = dbnet.Server(max_neurons=max_neurons, max_requests=4, max_regions=16, max_delay=max_delay,
+                       chunk_steps=128, arena_bytes=1 << 30, run=dict(autotune_at=64, tr_ms=20.0))
+    nets = [synth.make_graph(z, 40, 50 + i, k_within=32 if len(z) > 1 else 40, d_within=(1, 20),
+                             d_cross=(20, 40), region_density=1.0)
+            for i, z in enumerate(([1500, 700], [2100], [900, 800, 700], [2600, 300]))]
+    p = synth.default_region_params(I_ext=0.92)
+    todo = [(g, n, i) for i, (g, n) in enumerate(zip(nets * 3, (700, 1500, 1100, 900, 2000, 640, 1300, 800, 1700,
+                                                                 1000, 1200, 760)))]
+    ids = {srv.submit(g, p, n, seed=30 + i, raster_capacity=1 << 18): (g, n, i) for g, n, i in todo}
+    srv.drain()
+    for rid, (g, n, i) in ids.items():
+        net = dbnet.Network(g, p, dict(seed=30 + i, raster_capacity=1 << 18, tr_ms=20.0, autotune_at=-1))
+        net.step(n)
+        a, b = srv.spikes(rid), net.spikes()
+        assert len(b[1]) > 100 and np.array_equal(np.stack(a), np.stack(b)), i
+        assert np.array_equal(srv.bold(rid), net.bold()), i
+        net.close()
+    srv.close()
