@@ -163,7 +163,7 @@ typedef struct {
  *                    emit_delay) does so before and after them, and one more
  *                    turn of 64 steps, after the tuning is reported done,
  *                    keeps it unless the best per-step shape was faster by
- *                    a tenth.
+ *                    a tenth than three such turns.
  *                    Results depend on none of these choices (integer
  *                    accumulation).  Default 2000 (200 ms at dt 0.1 ms, past
  *                    the onset).

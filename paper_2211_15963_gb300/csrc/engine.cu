@@ -1123,9 +1123,10 @@ void Engine::to_rule() {
   resident = rule_resident;
 }
 
-// The tuner's last turn: one chunk of the rule's mode against the chosen
+// The tuner's last turn: a chunk of the rule's mode against the chosen
 // per-step shape's last one (the activity grows over the first rounds); the
-// rule's mode stays unless that was faster by a tenth.
+// rule's mode stays unless that was faster by a tenth than three such turns
+// (the first one pays for the graph's upload).
 int64_t Engine::weigh_steps(int64_t n) {
   if (dev.mode == kPerStep) {
     if (!may_switch()) {
@@ -1149,6 +1150,7 @@ int64_t Engine::weigh_steps(int64_t n) {
   CK(cudaEventSynchronize(tune_ev[1]));
   float ms = 0.0f;
   CK(cudaEventElapsedTime(&ms, tune_ev[0], tune_ev[1]));
+  if ((double)ms > 1.1 * best_ms && ++weighed < 3) return kChunk;
   weigh_rule = false;
   if ((double)ms > 1.1 * best_ms && may_switch()) {
     to_per_step();

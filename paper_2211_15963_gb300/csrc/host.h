@@ -289,6 +289,7 @@ struct Engine {
   int rule_grid = 0;
   bool rule_persistent = false, rule_resident = false;
   bool weigh_rule = false;
+  int weighed = 0;          // turns in which the rule was the slower one
   double best_ms = kDropped;          // the best per-step shape's last turn
   struct Shape {
     int grid, sched;

@@ -1904,6 +1904,8 @@ namespace {
 // predecessor on the stream to end (step_after in the kernel does): that
 // took a step of 2 M neurons from 54.7 to 53.1 us and one of 500,000 in
 // columns from 19.2 to 18.4; at 4 and 5 M neurons it cost one of 98 us 1.2.
+// Per-step delivery keeps plain launches: its kernels' shares are what the
+// autotuner compares, a candidate by itself.
 template <class... Par, class... Arg>
 void launch_after(void (*k)(Par...), int grid, int threads, cudaStream_t s, const EngineDev& e, Arg... arg) {
   cudaLaunchConfig_t cfg{};
@@ -1914,7 +1916,7 @@ void launch_after(void (*k)(Par...), int grid, int threads, cudaStream_t s, cons
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = e.n_tiles <= 2048 ? 1 : 0;
+  cfg.numAttrs = e.mode != kPerStep && e.n_tiles <= 2048 ? 1 : 0;
   cudaLaunchKernelEx(&cfg, k, e, arg...);  // (errors by cudaGetLastError, as for <<<>>>)
 }
 
