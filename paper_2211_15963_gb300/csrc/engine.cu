@@ -512,9 +512,11 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
     // as long as its accumulators stay in the L2 (see k_windows).  Where the
     // update adds its own spikes' edges (small networks, bound by launches)
     // the longest; with spike binning, whose ring is a bin longer, four.
+    // Never longer than the longest delay: a window counts its earlier
+    // spikes' events as it goes over those that may still have edges due.
     dev.push_now = tiles <= kPushTiles;
     int32_t W = dev.push_now ? (lead > 0 ? 4 : kWindow) : 4 * slot_b <= kWindowRingBytes ? 4 : 2;
-    W = std::min(W, pow2(dev.dmax));
+    while (W > dev.dmax) W /= 2;
     const int32_t all = pow2(D), win = pow2(W + lead);
     if (fits(all) && all * slot_b <= kEmitRingBytes) {
       dev.mode = kAtEmission;

@@ -1,0 +1,56 @@
+"""Delivery modes and launch shapes at the edges of the rules that choose
+them: against the matched-FP32 oracle, or against another mode of the same
+network.  The arithmetic is the same in the same order and arrivals are exact
+integers, so the tolerance is zero."""
+import threading
+
+import numpy as np
+import pytest
+
+import oracle
+import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _device():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a GPU")
+    import __graft_entry__
+    __graft_entry__.build()
+    torch.cuda.set_device(0)
+
+
+def _net(g, p, **opts):
+    from paper_2211_15963_gb300 import dbnet
+    return dbnet.Network(g, p, opts)
+
+
+def _same(net, other):
+    for a, b in zip(net.state(), other.state()):
+        assert np.array_equal(np.asarray(a, np.float64), np.asarray(b, np.float64))
+
+
+# Windows on networks whose longest delay is short and no power of two: the
+# accumulators of every delay at once lie beyond the emission ring's 48 MB, by
+# four channels or by size; the update adds the edges due in the window (up to
+# 532 tiles) or a kernel of its own does, with two weights and with one.
+@pytest.mark.parametrize("n,dmax,two", [(400_000, 5, True), (400_000, 6, True), (400_000, 7, True),
+                                        (800_000, 3, True), (1_600_000, 3, False)])
+def test_windows_and_short_delays(n, dmax, two):
+    g = synth.make_graph([n // 2, n - n // 2], 20, 5, k_within=16, d_within=(1, dmax), d_cross=(1, dmax))
+    assert g.delay.max() == dmax
+    if two:
+        g = synth.with_second_weight(g, 5)
+    p = [synth.default_region_params(I_ext=0.88 + 0.03 * r) for r in range(2)]
+    net = _net(g, p, seed=3, tr_ms=5.0)
+    o = oracle.Sim(g, p, seed=3, tr_ms=5.0, precision=32)
+    for k in (1, 6, 66, 3, 9):
+        net.step(k)
+        o.step(k)
+        s, so = net.stats(), o.info()
+        assert s["events"] == so["events"] and s["spikes"] == so["spikes"] > 0, k
+    _same(net, o)
+    net.close()
