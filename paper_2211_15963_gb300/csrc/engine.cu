@@ -946,6 +946,10 @@ void Engine::step(int64_t n) {
       n -= tune_emit(n);
       continue;
     }
+    // (the persistent schedule by option on more tiles than it is weighed
+    // with: no candidate, so the shape stays)
+    if (tune_pending && g_host >= tune_at && fixed_schedule == DBNET_SCHEDULE_PERSISTENT && !persist_tunable)
+      tune_pending = false;
     if (tune_pending && g_host >= tune_at && (dev.mode == kPerStep || (n >= kChunk && may_switch()))) {  // then the grid
       if (dev.mode != kPerStep) to_per_step();
       n -= tune_steps(n);

@@ -54,3 +54,23 @@ def test_windows_and_short_delays(n, dmax, two):
         assert s["events"] == so["events"] and s["spikes"] == so["spikes"] > 0, k
     _same(net, o)
     net.close()
+
+
+def test_persistent_schedule_on_more_tiles_than_blocks():
+    """The persistent schedule by option on more tiles than its blocks: each
+    block takes several tiles of a step, in windows with their own kernel's
+    part for the rest of a window.  The autotuner has nothing to weigh there;
+    the schedule stays what the options say and nothing fails."""
+    g = synth.make_graph([300_000, 400_000], 10, 11, k_within=8, d_within=(1, 12), d_cross=(12, 60))
+    p = [synth.default_region_params(I_ext=0.88 + 0.03 * r) for r in range(2)]
+    net = _net(g, p, seed=5, schedule=3, autotune_at=64)
+    plain = _net(g, p, seed=5, schedule=1, autotune_at=-1)
+    for n in (30, 100, 130):
+        net.step(n)
+        plain.step(n)
+        _same(net, plain)
+        s, sp = net.stats(), plain.stats()
+        assert s["schedule"] == 3 and s["events"] == sp["events"] and s["spikes"] == sp["spikes"] > 0
+    assert s["autotuned"] == 1
+    net.close()
+    plain.close()
