@@ -1980,20 +1980,21 @@ void launch_windows(const EngineDev& e, int grid, StepRef sr, bool first, cudaSt
 
 namespace {
 
-// f(kernel) for the stepper's variant that suits the engine on grid blocks
+// f(kernel) for the engine's variant of the stepper; held: a block for every
+// tile keeps its state (not per step)
 template <bool EXT, bool FOUR, class F>
-auto with_persist(const EngineDev& e, int grid, F&& f) {
+auto with_persist(const EngineDev& e, bool held, F&& f) {
   const bool one = e.n_inst == 1;
   if (e.mode == kPerStep)
     return one ? f(k_persist<EXT, FOUR, true, true, false>) : f(k_persist<EXT, FOUR, false, true, false>);
-  if (grid >= e.n_tiles)
+  if (held)
     return one ? f(k_persist<EXT, FOUR, true, false, true>) : f(k_persist<EXT, FOUR, false, false, true>);
   return one ? f(k_persist<EXT, FOUR, true, false, false>) : f(k_persist<EXT, FOUR, false, false, false>);
 }
 template <class F>
-auto with_persist(const EngineDev& e, int grid, F&& f) {
-  if (e.four) return e.any_ext ? with_persist<true, true>(e, grid, f) : with_persist<false, true>(e, grid, f);
-  return e.any_ext ? with_persist<true, false>(e, grid, f) : with_persist<false, false>(e, grid, f);
+auto with_persist(const EngineDev& e, bool held, F&& f) {
+  if (e.four) return e.any_ext ? with_persist<true, true>(e, held, f) : with_persist<false, true>(e, held, f);
+  return e.any_ext ? with_persist<true, false>(e, held, f) : with_persist<false, false>(e, held, f);
 }
 
 }  // namespace
@@ -2002,9 +2003,9 @@ int persist_max_grid(const EngineDev& e) {
   int dev = 0, sms = 0, occ = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int least = 1 << 20;  // of the variants it may take
-  for (int grid : {0, 1 << 30}) {
-    const cudaError_t r = with_persist(e, grid, [&](auto k) {
+  int least = 1 << 20;  // of both variants: which one runs depends on the tiles in use
+  for (bool held : {false, true}) {
+    const cudaError_t r = with_persist(e, held, [&](auto k) {
       return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kDelThreads, 0);
     });
     if (r != cudaSuccess) return 0;
@@ -2021,7 +2022,7 @@ cudaError_t launch_persist(const EngineDev& e, int grid, unsigned long long g0, 
   if (r != cudaSuccess) return r;
   EngineDev ea = e;
   void* args[] = {&ea, &g0, &nsteps, &count, &limit_ns};
-  return with_persist(e, grid, [&](auto k) {
+  return with_persist(e, grid >= e.n_tiles, [&](auto k) {
     return cudaLaunchCooperativeKernel(k, dim3(grid), dim3(kDelThreads), args, 0, s);
   });
 }
