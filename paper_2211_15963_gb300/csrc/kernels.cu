@@ -837,10 +837,11 @@ struct ItemLoads {
 // read only spikes of steps <= g - 2 and so run beside the update of
 // iteration g - 1; then kPartShort after that update: the ring bookkeeping, the segment-ring copy of step g - 1's spikes, the
 // delay-1 items and the emission items.
-// Loads of the spike and segment rings: through the read-only path when
-// the rings are written only by earlier launches; from the L2 (coherent,
-// never a stale L1 line) in the persistent stepper, whose own blocks wrote
-// them earlier in the launch.
+// Per-step delivery's loads of the spike and segment rings: through the
+// read-only path where an entry was written by a launch that has ended
+// (k_deliver is launched plainly, never as a programmatic dependent); from the
+// L2 (coherent, never a stale L1 line) in the persistent stepper, whose own
+// blocks wrote them earlier in the launch.
 template <bool PERSIST, typename T>
 __device__ __forceinline__ T ld_ring(const T* p) {
   if (PERSIST) return __ldcg(p);
@@ -1222,18 +1223,21 @@ constexpr unsigned long long kNoRow = ~0ull;
 // 128 us were left without its edge reads and reductions).  Counts the
 // synaptic events of those spikes: the out-degree of each, once (Supp. Alg. 2
 // pushes every out-edge once).
-template <bool PERSIST>
+// Here and below the spike and bounds rings and their counts are read from the
+// L2: the update that writes them may still run when this kernel starts as its
+// programmatic dependent (or is a part of this one, in the persistent
+// stepper), so they are not read-only in the kernel's life.  The graph is.
 __device__ __forceinline__ void copy_bounds(const EngineDev& e, unsigned long long g, uint32_t w0, uint32_t n,
                                             unsigned long long& ev) {
   if (g == 0ull) return;
   const int lane = threadIdx.x & 31;
   const uint32_t sl = (uint32_t)((g - 1ull) % (unsigned long long)e.D);
-  const uint32_t h = PERSIST ? __ldcg(e.hcount + sl) : e.hcount[sl];
+  const uint32_t h = __ldcg(e.hcount + sl);
   const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap, cap = (uint32_t)e.seg_cap;
   const int W = e.wmask + 1;
   const int first = W - (int)((unsigned)(g - 1ull) & (unsigned)e.wmask);  // delay at the next window's start
   for (uint32_t k = w0; k < c; k += n) {
-    const uint32_t ent = ld_ring<PERSIST>(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
+    const uint32_t ent = __ldcg(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
     const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
     const int inst = e.n_inst == 1 ? 0 : e.tile_info[gidx / kTile].x;
     unsigned long long packed = kNoRow;
@@ -1268,7 +1272,7 @@ __device__ __forceinline__ void copy_bounds(const EngineDev& e, unsigned long lo
 // it: W = 4 / 2 / 1 measured 33.8 / 35.0 / 43.2 us a step at 2 M neurons and
 // in-degree 1,000 (16 MB of accumulators per step; 45.3 us with one delay per
 // step and kernel), 49.9 / 45.2 / 50.9 us at 5 M and 400 (40 MB; 60.2 us).
-template <bool FOUR, bool SINGLE, bool PERSIST>
+template <bool FOUR, bool SINGLE>
 __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned long long g, int bid, int nblk) {
   // items of phase q and bucket t start at s_pre[q][t] of the phase
   __shared__ uint32_t s_pre[kMaxPhases][256];
@@ -1299,7 +1303,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
   const int tme = threadIdx.x;
   if (tme < nb && g >= (unsigned long long)(t0 + tme) + 1ull) {
     const uint32_t sl = ring_of(t0 + tme);
-    const uint32_t h = PERSIST ? __ldcg(e.hcount + sl) : e.hcount[sl];
+    const uint32_t h = __ldcg(e.hcount + sl);
     c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
   }
   // Phases: the update appends each step's spikes roughly in tile order, so
@@ -1381,9 +1385,9 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
     if (it.t > 0 && it.k < cap && g - 1ull - (unsigned long long)it.t >= e.since) {  // window it.t / W of its slot
       const size_t sl = ring_of(it.t);
       const uint16_t* B = e.hseg + (sl * (size_t)e.dcap + (uint32_t)it.t / (uint32_t)W) * cap + it.k;
-      it.row = ld_ring<PERSIST>(reinterpret_cast<const unsigned long long*>(e.hr0) + sl * cap + it.k);
-      it.a = ld_ring<PERSIST>(B);
-      it.b = ld_ring<PERSIST>(B + cap);
+      it.row = __ldcg(reinterpret_cast<const unsigned long long*>(e.hr0) + sl * cap + it.k);
+      it.a = __ldcg(B);
+      it.b = __ldcg(B + cap);
     }
     return it;
   };
@@ -1403,7 +1407,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
       key |= (uint32_t)(it.row >> 47) & 1u;
       return;
     }
-    const uint32_t ent = ld_ring<PERSIST>(e.hist + (size_t)ring_of(it.t) * (size_t)e.hist_cap + it.k);
+    const uint32_t ent = __ldcg(e.hist + (size_t)ring_of(it.t) * (size_t)e.hist_cap + it.k);
     const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
     key |= ent >> 31;
     if (!SINGLE) {
@@ -1438,7 +1442,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
   __syncthreads();
   }
   if (e.seg_cap > 0)
-    copy_bounds<PERSIST>(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, (uint32_t)nblk * (kDelThreads / 32), ev);
+    copy_bounds(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, (uint32_t)nblk * (kDelThreads / 32), ev);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
   if (lane == 0 && ev) atomicAdd(e.events, ev);
@@ -1448,13 +1452,13 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
 // that come due by the window's end, the start of their rows.  A warp takes 32
 // of the spikes, or fewer when that would leave warps without one; four
 // dependent loads (count, ring entry, table row, records) bound it.
-template <bool FOUR, bool SINGLE, bool PERSIST>
+template <bool FOUR, bool SINGLE>
 __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long long g, int bid, int nblk,
                                              int4* s_item) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int left = e.wmask + 1 - (int)((unsigned)g & (unsigned)e.wmask);  // steps to the window's end
   const uint32_t sl = (uint32_t)((g - 1ull) % (unsigned long long)e.D);
-  const uint32_t h = PERSIST ? __ldcg(e.hcount + sl) : __ldg(e.hcount + sl);
+  const uint32_t h = __ldcg(e.hcount + sl);
   const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
   const uint32_t warps = (uint32_t)nblk * (kDelThreads / 32);
   int ub = 5;
@@ -1466,7 +1470,7 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
     uint32_t nseg = 0, key = 0;
     int inst = 0;
     if (lane < (1 << ub) && k < c) {
-      const uint32_t ent = ld_ring<PERSIST>(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
+      const uint32_t ent = __ldcg(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
       const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
       if (!SINGLE) inst = e.tile_info[gidx / kTile].x;
       if (inst >= 0) {
@@ -1485,21 +1489,21 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
   }
   if (e.seg_cap == 0) return;
   unsigned long long ev = 0;
-  copy_bounds<PERSIST>(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, warps, ev);
+  copy_bounds(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, warps, ev);
   if (lane == 0 && ev) atomicAdd(e.events, ev);
 }
 
 template <bool FOUR, bool SINGLE>
 __global__ void __launch_bounds__(kDelThreads, 4) k_windows(EngineDev e, StepRef sr) {
   step_after();
-  deliver_windows<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x);
+  deliver_windows<FOUR, SINGLE>(e, step_of(sr), blockIdx.x, gridDim.x);
 }
 
 template <bool FOUR, bool SINGLE>
 __global__ void __launch_bounds__(kDelThreads, 4) k_rest(EngineDev e, StepRef sr) {
   __shared__ int4 s_item[kDelThreads];
   step_after();
-  deliver_rest<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x, s_item);
+  deliver_rest<FOUR, SINGLE>(e, step_of(sr), blockIdx.x, gridDim.x, s_item);
 }
 
 template <bool FOUR, bool SINGLE>
@@ -1687,8 +1691,8 @@ __global__ void __launch_bounds__(kDelThreads, 2)
     if (due) {
       if (PER_STEP) deliver_body<FOUR, SINGLE, true>(e, sr, kPartAll, blockIdx.x, gridDim.x);
       else if (((unsigned)g & (unsigned)e.wmask) == 0u)
-        deliver_windows<FOUR, SINGLE, true>(e, g, blockIdx.x, gridDim.x);
-      else deliver_rest<FOUR, SINGLE, true>(e, g, blockIdx.x, gridDim.x, s_item);
+        deliver_windows<FOUR, SINGLE>(e, g, blockIdx.x, gridDim.x);
+      else deliver_rest<FOUR, SINGLE>(e, g, blockIdx.x, gridDim.x, s_item);
       target += gridDim.x;
       if (!grid_barrier(count, target, limit_ns, e.flags)) return;
     }
