@@ -955,7 +955,7 @@ void Engine::step(int64_t n) {
       n -= tune_steps(n);
       continue;
     }
-    if (weigh_rule) {  // and whether the best of them beats the mode the rule chose
+    if (verdict.is_open()) {  // and whether the best of them beats the mode the rule chose
       n -= weigh_steps(n);
       continue;
     }
@@ -1073,7 +1073,7 @@ void Engine::finish_turn(int C) {
     if (tune_ms[(size_t)k] < tune_ms[(size_t)best]) best = k;
   set_shape(tune_grid[(size_t)(best / 3)], best % 3);
   tune_pending = false;
-  weigh_rule = rule.mode != kPerStep;
+  if (rule.mode != kPerStep) verdict.open();
 }
 
 void Engine::use(const Delivery& m) {
@@ -1096,11 +1096,9 @@ void Engine::drop_graph() {
   gexec = nullptr;
 }
 
-// The mode may change before step g_host: a window starts there, and no
-// earlier spike waits for the end of its bin.
+// The mode may change before step g_host (and no long part is enqueued).
 bool Engine::may_switch() const {
-  return !long_pending && (g_host & (unsigned long long)rule.wmask) == 0ull &&
-         g_host % (unsigned long long)(dev.bin_lead + 1) == 0ull;
+  return !long_pending && steps_to_switch(g_host, rule.wmask, dev.bin_lead) == 0;
 }
 
 // From the rule's mode to per-step delivery (where the mode may change).
@@ -1130,10 +1128,20 @@ void Engine::to_rule() {
 }
 
 // The tuner's last turn: a chunk of the rule's mode against the chosen
-// per-step shape's last one (the activity grows over the first rounds); the
-// rule's mode stays unless that was faster by a tenth than three such turns
-// (the first one pays for the graph's upload).
+// per-step shape's last one (the activity grows over the first rounds), until
+// the verdict (RuleVerdict) is known and carried out.
 int64_t Engine::weigh_steps(int64_t n) {
+  if (verdict.leaving()) {
+    const int64_t k = std::min(n, steps_to_switch(g_host, rule.wmask, dev.bin_lead));
+    if (k > 0) {
+      run_plain(k);
+      return k;
+    }
+    to_per_step();
+    set_shape(best_shape.grid, best_shape.sched);
+    verdict.left();
+    return 0;
+  }
   if (dev.mode == kPerStep) {
     if (!may_switch()) {
       direct_step();
@@ -1156,12 +1164,7 @@ int64_t Engine::weigh_steps(int64_t n) {
   CK(cudaEventSynchronize(tune_ev[1]));
   float ms = 0.0f;
   CK(cudaEventElapsedTime(&ms, tune_ev[0], tune_ev[1]));
-  if ((double)ms > 1.1 * best_ms && ++weighed < 3) return kChunk;
-  weigh_rule = false;
-  if ((double)ms > 1.1 * best_ms && may_switch()) {
-    to_per_step();
-    set_shape(best_shape.grid, best_shape.sched);
-  }
+  verdict.turn((double)ms, best_ms);
   return kChunk;
 }
 

@@ -13,6 +13,7 @@
 #include "dbnet.h"
 #include "engine.h"
 #include "freelist.h"
+#include "turns.h"
 
 namespace dbn {
 
@@ -288,8 +289,7 @@ struct Engine {
   Delivery rule{}, per_step{};
   int rule_grid = 0;
   bool rule_persistent = false, rule_resident = false;
-  bool weigh_rule = false;
-  int weighed = 0;          // turns in which the rule was the slower one
+  RuleVerdict verdict;
   double best_ms = kDropped;          // the best per-step shape's last turn
   struct Shape {
     int grid, sched;

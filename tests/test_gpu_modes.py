@@ -74,3 +74,26 @@ def test_persistent_schedule_on_more_tiles_than_blocks():
     assert s["autotuned"] == 1
     net.close()
     plain.close()
+
+
+def test_a_losing_rule_is_left_with_binned_spikes():
+    """60,000 neurons at some 800,000 events a step, far above what one
+    cluster's SMs reduce: the resident stepper takes twice the time of the
+    best per-step shape, and the tuner's verdict to leave it holds although
+    its turns end inside a bin."""
+    k = 1000
+    g = synth.make_graph([30_000, 30_000], k, 27, k_within=800, d_within=(1, 10), d_cross=(10, 20))
+    p = synth.default_region_params(I_ext=97.0)
+    p["g_u"] = tuple(x * 100.0 / k for x in p["g_u"])
+    opts = dict(seed=4, bin_spikes=1)
+    rule = _net(g, p, autotune_at=-1, **opts)
+    net = _net(g, p, autotune_at=64, **opts)
+    net.step(6000)
+    rule.step(6000)
+    s, r = net.stats(), rule.stats()
+    assert s["events"] == r["events"] > 6000 * 500_000 and s["autotuned"] == 1
+    assert r["schedule"] == 3 and s["deliver_blocks"] != r["deliver_blocks"]  # of a per-step shape
+    for a, b in zip(net.state(), rule.state()):
+        assert np.array_equal(a, b)
+    net.close()
+    rule.close()
