@@ -961,7 +961,8 @@ void Engine::step(int64_t n) {
     }
     int64_t k = n;
     if ((tune_pending || emit_pending) && g_host < tune_at) k = std::min<int64_t>(n, (int64_t)(tune_at - g_host));
-    else if (tune_pending && n >= kChunk) k = 1;  // to the start of a window
+    else if (tune_pending && n >= kChunk)  // to the step where the turns may go on
+      k = std::min(n, std::max<int64_t>(1, steps_to_switch(g_host, rule.wmask, dev.bin_lead)));
     run_plain(k);
     n -= k;
   }
@@ -1017,14 +1018,22 @@ int64_t Engine::tune_emit(int64_t n) {
 // events (a captured graph, or one persistent launch, enqueued at once, so
 // the timing is the device's); the
 // smallest total wins, so that the network's own fluctuations of activity
-// from chunk to chunk average out.  Fewer than kChunk steps run plainly and
-// the tuning goes on at the next call.  Returns the steps run.
+// from chunk to chunk average out.  Fewer than kChunk steps run plainly, in
+// the mode of the engine's rule where it has one (a program that goes on with
+// short calls would stay in the last candidate: 13 us a step instead of 4.4 at
+// 10,000 neurons), and the tuning goes on at the next longer call.  Returns
+// the steps run.
 int64_t Engine::tune_steps(int64_t n) {
   const int C = (int)tune_grid.size() * 3;
   const int c = tune_done % C;
   if (n < kChunk) {
-    for (int64_t i = 0; i < n; ++i) direct_step();
-    return n;
+    if (rule.mode != kPerStep && may_switch()) {
+      to_rule();
+      return 0;
+    }
+    const int64_t k = rule.mode != kPerStep ? 1 : n;
+    for (int64_t i = 0; i < k; ++i) direct_step();
+    return k;
   }
   const int sched = c % 3, grid = tune_grid[(size_t)(c / 3)];
   if ((fixed_schedule != DBNET_SCHEDULE_AUTO && sched + 1 != fixed_schedule) ||

@@ -97,3 +97,28 @@ def test_a_losing_rule_is_left_with_binned_spikes():
         assert np.array_equal(a, b)
     net.close()
     rule.close()
+
+
+def test_calls_shorter_than_a_tuning_turn():
+    """A program that stops in the middle of the tuning and goes on with
+    calls too short for a turn steps in the mode of the engine's size, not
+    in the candidate that came last; longer calls finish the tuning."""
+    g = synth.small_network()
+    p = synth.default_region_params()
+    net = _net(g, p, seed=7, autotune_at=64, raster_capacity=1 << 20)
+    o = oracle.Sim(g, p, seed=7, precision=32)
+    for n in (64 + 64, 10, 1, 9, 200, 63, 64, 10):
+        net.step(n)
+        o.step(n)
+        s = net.stats()
+        if n < 64:
+            assert s["schedule"] == 3 and s["autotuned"] == 0
+        assert s["events"] == o.info()["events"]
+        _same(net, o)
+    for n in (5000, 10, 2000):
+        net.step(n)
+        o.step(n)
+    assert net.stats()["autotuned"] == 1 and net.stats()["events"] == o.info()["events"]
+    assert np.array_equal(np.stack(net.spikes()), np.stack(o.raster()))
+    _same(net, o)
+    net.close()
