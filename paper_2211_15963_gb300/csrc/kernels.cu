@@ -1738,8 +1738,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_resident(EngineDev e, unsigned l
   held_load(e, tile, s_tile[warp / kTileWarps]);
   __syncthreads();
   HeldWarp<EXT, FOUR> h(e, tile, warp % kTileWarps, s_tile[warp / kTileWarps]);
-  const auto close = [&](unsigned long long g) {  // one block closes the bins, the last: it has the fewest tiles
-    if (blockIdx.x == gridDim.x - 1) close_regions(e, g, warp, THREADS / 32);
+  // the last blocks close the bins, for they have the fewest tiles
+  const auto close = [&](unsigned long long g) {
+    close_regions(e, g, (gridDim.x - 1 - blockIdx.x) * (THREADS / 32) + warp, gridDim.x * (THREADS / 32));
   };
   h.prepare(g0);
   for (int s = 0; s < nsteps; ++s) {

@@ -122,3 +122,21 @@ def test_calls_shorter_than_a_tuning_turn():
     assert np.array_equal(np.stack(net.spikes()), np.stack(o.raster()))
     _same(net, o)
     net.close()
+
+
+# More regions than the warps of one block close at once, on one block and on
+# sixteen, closing every step and every tenth.
+@pytest.mark.parametrize("size,regions,dt", [(4, 1000, 0.1), (5, 1300, 1.0), (40, 1200, 0.1)])
+def test_many_regions_on_the_resident_stepper(size, regions, dt):
+    g = synth.make_graph([size] * regions, 20, 19, k_within=2, d_within=(1, 3), d_cross=(1, 9))
+    p = [synth.default_region_params(I_ext=0.86 + 0.01 * (r % 5)) for r in range(regions)]
+    over = dict(dt_ms=dt, bin_ms=1.0, tr_ms=2.0)
+    net = _net(g, p, seed=6, **over)
+    assert net.stats()["schedule"] == 3
+    o = oracle.Sim(g, p, seed=6, precision=32, **over)
+    for n in (1, 39, 60):
+        net.step(n)
+        o.step(n)
+    _same(net, o)
+    assert len(net.bold()) > 0 and np.allclose(net.bold(), o.bold(), rtol=1e-10, atol=1e-15)
+    net.close()
