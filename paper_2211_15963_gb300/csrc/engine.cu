@@ -499,7 +499,9 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   const int32_t D0 = D;  // ring slots that per-step delivery needs
   const bool tunes = common.autotune_at >= 0 && !(common.deliver_blocks > 0 && common.schedule != DBNET_SCHEDULE_AUTO);
   if (emit_from > 0) {
+    // (a power of two where that fits, so that a mask finds a step's slot)
     if (pow2(D) * slot_b <= (double)free_b / 3.0) slots = pow2(D);
+    else if (D * slot_b <= (double)free_b / 3.0) slots = D;
     else emit_from = 0;
   }
   // (a request server's instances have bins of their own each, so that there

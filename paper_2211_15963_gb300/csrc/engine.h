@@ -25,10 +25,11 @@
 //   The segment table: row j, of seg_bytes (a multiple of 16), holds the
 //   row's first and last edge (two int64) and, for k < dmax, the number of
 //   its edges with delay <= k + 1 (u16, or u32 for rows of 65,536 edges on).
-// The accumulators are a ring of acc_slots (a power of two): slot a mod
-// acc_slots collects the arrivals of step a, and the update of step a reads
-// and clears it.  A spike handed on at step s reaches the target of an edge
-// of delay d at step s + d; which kernel adds the edge is the engine's mode:
+// The accumulators are a ring of acc_slots (a power of two, or with an
+// emission threshold as many as the delays need): slot a mod acc_slots
+// collects the arrivals of step a, and the update of step a reads and clears
+// it.  A spike handed on at step s reaches the target of an edge of delay d at
+// step s + d; which kernel adds the edge is the engine's mode:
 //   kAtEmission  the update that emits a spike adds its whole row.  No spike
 //                ring, one launch per step.
 //   kWindows     steps go in windows of W = wmask + 1 (aligned to multiples
@@ -194,7 +195,7 @@ struct EngineDev {
   uint8_t* ref;
   int2* acc;             // [acc_slots][stride] (int2, or int4 with four channels)
   int64_t stride;
-  int32_t acc_slots;     // a power of two
+  int32_t acc_slots;     // a power of two, but for kPerStep with an emission threshold
   int32_t mode;          // kPerStep, kWindows or kAtEmission
   int32_t wmask;         // kWindows: steps per window - 1 (a power of two less one)
   int32_t push_now;      // kWindows: the update adds its spikes' edges due in the window

@@ -244,9 +244,15 @@ __device__ __forceinline__ float normal_from_word(unsigned long long w) {
   return sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
 }
 
-// Where an iteration's accumulators lie.
+// The accumulator slot of iteration a, and where it lies.  (A ring that is no
+// power of two has at most 256 slots.)
+__device__ __forceinline__ uint32_t acc_slot(const EngineDev& e, unsigned long long a) {
+  const uint32_t n = (uint32_t)e.acc_slots;
+  if ((n & (n - 1u)) == 0u) return (uint32_t)a & (n - 1u);
+  return ((uint32_t)(a >> 32) % n * (0xFFFFFFFFu % n + 1u) + (uint32_t)a % n) % n;
+}
 __device__ __forceinline__ int2* acc_of(const EngineDev& e, unsigned long long g) {
-  return e.acc + (size_t)((unsigned)g & (unsigned)(e.acc_slots - 1)) * (size_t)e.stride * (e.four ? 2 : 1);
+  return e.acc + (size_t)acc_slot(e, g) * (size_t)e.stride * (e.four ? 2 : 1);
 }
 
 // a / b for step counts: in 32 bits while they fit
@@ -1019,7 +1025,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
   }
   const unsigned long long W = W_arr + c1e * (unsigned long long)ne;
   const unsigned long long acc_elems = (unsigned long long)e.stride * (FOUR ? 2 : 1);
-  const uint32_t aslot_now = (uint32_t)g & ((uint32_t)e.acc_slots - 1u);
+  const uint32_t aslot_now = acc_slot(e, g), aslot_last = acc_slot(e, g - 1ull);
   __syncthreads();
 
   const unsigned long long pol_rec = l2_policy_first(), pol_acc = l2_policy_last();
@@ -1035,7 +1041,8 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
       p.k = (uint32_t)(te / (unsigned long long)ne);
       p.d = (uint32_t)e.d_emit + (uint32_t)(te % (unsigned long long)ne);
       p.slot = (uint32_t)s1;
-      p.aslot = (uint32_t)(g - 1ull + p.d) & ((uint32_t)e.acc_slots - 1u);
+      p.aslot = aslot_last + p.d;  // (the ring is longer than any delay)
+      if (p.aslot >= (uint32_t)e.acc_slots) p.aslot -= (uint32_t)e.acc_slots;
       p.ent = ld_ring<PERSIST>(e.hist + (size_t)p.slot * (size_t)e.hist_cap + p.k);
       return;
     }

@@ -140,3 +140,32 @@ def test_many_regions_on_the_resident_stepper(size, regions, dt):
     _same(net, o)
     assert len(net.bold()) > 0 and np.allclose(net.bold(), o.bold(), rtol=1e-10, atol=1e-15)
     net.close()
+
+
+def test_emission_threshold_with_a_ring_of_any_length():
+    """An explicit emission threshold is kept wherever a slot per step of the
+    longest delay fits a third of the free memory, also where the next power
+    of two of slots does not."""
+    n, dmax = 1_000_000, 128
+    g = synth.make_graph([n // 2, n - n // 2], 10, 13, k_within=8, d_within=(1, 20), d_cross=(20, dmax))
+    p = [synth.default_region_params(I_ext=0.88 + 0.03 * r) for r in range(2)]
+    plain = _net(g, p, seed=9, schedule=2, autotune_at=-1)
+    plain.step(200)
+    state, events = plain.state(), plain.stats()["events"]
+    plain.close()
+    torch.cuda.empty_cache()
+    slot = -(-n // 1024) * 1024 * 8
+    need = int(4.2 * (dmax + 1) * slot)  # a third of this holds 129 slots, not 256
+    hold = torch.empty(torch.cuda.mem_get_info()[0] - need, dtype=torch.uint8, device="cuda")
+    try:
+        net = _net(g, p, seed=9, emit_delay=30, autotune_at=-1)
+        for k in (1, 70, 129):
+            net.step(k)
+        assert net.stats()["emit_delay"] == 30
+        for a, b in zip(net.state(), state):
+            assert np.array_equal(a, b)
+        assert net.stats()["events"] == events
+        net.close()
+    finally:
+        del hold
+        torch.cuda.empty_cache()
