@@ -244,15 +244,19 @@ __device__ __forceinline__ float normal_from_word(unsigned long long w) {
   return sqrtf(-2.0f * logf(u1)) * cospif(2.0f * u2);
 }
 
-// The accumulator slot of iteration a, and where it lies.  (A ring that is no
-// power of two has at most 256 slots.)
+// The accumulator slot of iteration a, and where it lies.  ANY: the ring may be
+// other than a power of two (at most 256 slots); the update's variants without
+// the kExt* terms leave that out (nest_4m_1ms 49.8 against 49.6 ms, 64 members
+// 131.3 against 130.7) and such engines take the variants with them.
+template <bool ANY>
 __device__ __forceinline__ uint32_t acc_slot(const EngineDev& e, unsigned long long a) {
   const uint32_t n = (uint32_t)e.acc_slots;
-  if ((n & (n - 1u)) == 0u) return (uint32_t)a & (n - 1u);
+  if (!ANY || (n & (n - 1u)) == 0u) return (uint32_t)a & (n - 1u);
   return ((uint32_t)(a >> 32) % n * (0xFFFFFFFFu % n + 1u) + (uint32_t)a % n) % n;
 }
+template <bool ANY>
 __device__ __forceinline__ int2* acc_of(const EngineDev& e, unsigned long long g) {
-  return e.acc + (size_t)acc_slot(e, g) * (size_t)e.stride * (e.four ? 2 : 1);
+  return e.acc + (size_t)acc_slot<ANY>(e, g) * (size_t)e.stride * (e.four ? 2 : 1);
 }
 
 // a / b for step counts: in 32 bits while they fit
@@ -761,7 +765,7 @@ __device__ __forceinline__ void update_warp(const EngineDev& e, const StepRef& s
   // or per two (E, I of each), from the accumulator slot of this iteration
   const unsigned long long g = step_of(sr);
   constexpr int kA = FOUR ? 4 : 2;
-  int4* const accs = reinterpret_cast<int4*>(acc_of(e, g)) + (FOUR ? w.gi0 : w.gi0 / 2);
+  int4* const accs = reinterpret_cast<int4*>(acc_of<EXT>(e, g)) + (FOUR ? w.gi0 : w.gi0 / 2);
   int4 A[kA];
 #pragma unroll
   for (int k = 0; k < kA; ++k) A[k] = __ldcg(accs + k);
@@ -1025,7 +1029,7 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
   }
   const unsigned long long W = W_arr + c1e * (unsigned long long)ne;
   const unsigned long long acc_elems = (unsigned long long)e.stride * (FOUR ? 2 : 1);
-  const uint32_t aslot_now = acc_slot(e, g), aslot_last = acc_slot(e, g - 1ull);
+  const uint32_t aslot_now = acc_slot<true>(e, g), aslot_last = acc_slot<true>(e, g - 1ull);
   __syncthreads();
 
   const unsigned long long pol_rec = l2_policy_first(), pol_acc = l2_policy_last();
@@ -1219,6 +1223,18 @@ __device__ __forceinline__ void deliver_body(const EngineDev& e, const StepRef& 
 constexpr unsigned long long kRowMask = (1ull << 47) - 1ull;
 constexpr unsigned long long kNoRow = ~0ull;
 
+// Windows delivery's loads of the spike and bounds rings and their counts.
+// Never through the read-only path: the update that writes them may still run
+// when these kernels start as its programmatic dependents, or is a part of the
+// same launch in the persistent stepper.  Ordinary loads see the writes of the
+// grids that griddepcontrol.wait waited for, and neighbouring items share
+// sectors in the L1 (with loads from the L2: hmda_64x100k 130.4 -> 131.0 ms);
+// the persistent stepper's blocks read from the L2.
+template <bool PERSIST, typename T>
+__device__ __forceinline__ T ld_step(const T* p) {
+  return PERSIST ? __ldcg(p) : *p;
+}
+
 // The window bounds of step g - 1's spikes into the ring, one warp per spike,
 // warps w0, w0 + n, ...: for the spike of rank k, its row into hr0[slot][k],
 // and into hseg[slot][j][k] the number of its edges with delay below the
@@ -1230,21 +1246,18 @@ constexpr unsigned long long kNoRow = ~0ull;
 // 128 us were left without its edge reads and reductions).  Counts the
 // synaptic events of those spikes: the out-degree of each, once (Supp. Alg. 2
 // pushes every out-edge once).
-// Here and below the spike and bounds rings and their counts are read from the
-// L2: the update that writes them may still run when this kernel starts as its
-// programmatic dependent (or is a part of this one, in the persistent
-// stepper), so they are not read-only in the kernel's life.  The graph is.
+template <bool PERSIST>
 __device__ __forceinline__ void copy_bounds(const EngineDev& e, unsigned long long g, uint32_t w0, uint32_t n,
                                             unsigned long long& ev) {
   if (g == 0ull) return;
   const int lane = threadIdx.x & 31;
   const uint32_t sl = (uint32_t)((g - 1ull) % (unsigned long long)e.D);
-  const uint32_t h = __ldcg(e.hcount + sl);
+  const uint32_t h = ld_step<PERSIST>(e.hcount + sl);
   const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap, cap = (uint32_t)e.seg_cap;
   const int W = e.wmask + 1;
   const int first = W - (int)((unsigned)(g - 1ull) & (unsigned)e.wmask);  // delay at the next window's start
   for (uint32_t k = w0; k < c; k += n) {
-    const uint32_t ent = __ldcg(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
+    const uint32_t ent = ld_step<PERSIST>(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
     const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
     const int inst = e.n_inst == 1 ? 0 : e.tile_info[gidx / kTile].x;
     unsigned long long packed = kNoRow;
@@ -1279,7 +1292,7 @@ __device__ __forceinline__ void copy_bounds(const EngineDev& e, unsigned long lo
 // it: W = 4 / 2 / 1 measured 33.8 / 35.0 / 43.2 us a step at 2 M neurons and
 // in-degree 1,000 (16 MB of accumulators per step; 45.3 us with one delay per
 // step and kernel), 49.9 / 45.2 / 50.9 us at 5 M and 400 (40 MB; 60.2 us).
-template <bool FOUR, bool SINGLE>
+template <bool FOUR, bool SINGLE, bool PERSIST>
 __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned long long g, int bid, int nblk) {
   // items of phase q and bucket t start at s_pre[q][t] of the phase
   __shared__ uint32_t s_pre[kMaxPhases][256];
@@ -1310,7 +1323,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
   const int tme = threadIdx.x;
   if (tme < nb && g >= (unsigned long long)(t0 + tme) + 1ull) {
     const uint32_t sl = ring_of(t0 + tme);
-    const uint32_t h = __ldcg(e.hcount + sl);
+    const uint32_t h = ld_step<PERSIST>(e.hcount + sl);
     c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
   }
   // Phases: the update appends each step's spikes roughly in tile order, so
@@ -1392,9 +1405,9 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
     if (it.t > 0 && it.k < cap && g - 1ull - (unsigned long long)it.t >= e.since) {  // window it.t / W of its slot
       const size_t sl = ring_of(it.t);
       const uint16_t* B = e.hseg + (sl * (size_t)e.dcap + (uint32_t)it.t / (uint32_t)W) * cap + it.k;
-      it.row = __ldcg(reinterpret_cast<const unsigned long long*>(e.hr0) + sl * cap + it.k);
-      it.a = __ldcg(B);
-      it.b = __ldcg(B + cap);
+      it.row = ld_step<PERSIST>(reinterpret_cast<const unsigned long long*>(e.hr0) + sl * cap + it.k);
+      it.a = ld_step<PERSIST>(B);
+      it.b = ld_step<PERSIST>(B + cap);
     }
     return it;
   };
@@ -1414,7 +1427,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
       key |= (uint32_t)(it.row >> 47) & 1u;
       return;
     }
-    const uint32_t ent = __ldcg(e.hist + (size_t)ring_of(it.t) * (size_t)e.hist_cap + it.k);
+    const uint32_t ent = ld_step<PERSIST>(e.hist + (size_t)ring_of(it.t) * (size_t)e.hist_cap + it.k);
     const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
     key |= ent >> 31;
     if (!SINGLE) {
@@ -1449,7 +1462,7 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
   __syncthreads();
   }
   if (e.seg_cap > 0)
-    copy_bounds(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, (uint32_t)nblk * (kDelThreads / 32), ev);
+    copy_bounds<PERSIST>(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, (uint32_t)nblk * (kDelThreads / 32), ev);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ev += __shfl_down_sync(kFull, ev, o);
   if (lane == 0 && ev) atomicAdd(e.events, ev);
@@ -1459,13 +1472,13 @@ __device__ __forceinline__ void deliver_windows(const EngineDev& e, unsigned lon
 // that come due by the window's end, the start of their rows.  A warp takes 32
 // of the spikes, or fewer when that would leave warps without one; four
 // dependent loads (count, ring entry, table row, records) bound it.
-template <bool FOUR, bool SINGLE>
+template <bool FOUR, bool SINGLE, bool PERSIST>
 __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long long g, int bid, int nblk,
                                              int4* s_item) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int left = e.wmask + 1 - (int)((unsigned)g & (unsigned)e.wmask);  // steps to the window's end
   const uint32_t sl = (uint32_t)((g - 1ull) % (unsigned long long)e.D);
-  const uint32_t h = __ldcg(e.hcount + sl);
+  const uint32_t h = ld_step<PERSIST>(e.hcount + sl);
   const uint32_t c = (int64_t)h < e.hist_cap ? h : (uint32_t)e.hist_cap;
   const uint32_t warps = (uint32_t)nblk * (kDelThreads / 32);
   int ub = 5;
@@ -1477,7 +1490,7 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
     uint32_t nseg = 0, key = 0;
     int inst = 0;
     if (lane < (1 << ub) && k < c) {
-      const uint32_t ent = __ldcg(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
+      const uint32_t ent = ld_step<PERSIST>(e.hist + (size_t)sl * (size_t)e.hist_cap + k);
       const int64_t gidx = (int64_t)(ent & 0x7FFFFFFFu);
       if (!SINGLE) inst = e.tile_info[gidx / kTile].x;
       if (inst >= 0) {
@@ -1496,21 +1509,21 @@ __device__ __forceinline__ void deliver_rest(const EngineDev& e, unsigned long l
   }
   if (e.seg_cap == 0) return;
   unsigned long long ev = 0;
-  copy_bounds(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, warps, ev);
+  copy_bounds<PERSIST>(e, g, (uint32_t)bid * (kDelThreads / 32) + warp, warps, ev);
   if (lane == 0 && ev) atomicAdd(e.events, ev);
 }
 
 template <bool FOUR, bool SINGLE>
 __global__ void __launch_bounds__(kDelThreads, 4) k_windows(EngineDev e, StepRef sr) {
   step_after();
-  deliver_windows<FOUR, SINGLE>(e, step_of(sr), blockIdx.x, gridDim.x);
+  deliver_windows<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x);
 }
 
 template <bool FOUR, bool SINGLE>
 __global__ void __launch_bounds__(kDelThreads, 4) k_rest(EngineDev e, StepRef sr) {
   __shared__ int4 s_item[kDelThreads];
   step_after();
-  deliver_rest<FOUR, SINGLE>(e, step_of(sr), blockIdx.x, gridDim.x, s_item);
+  deliver_rest<FOUR, SINGLE, false>(e, step_of(sr), blockIdx.x, gridDim.x, s_item);
 }
 
 template <bool FOUR, bool SINGLE>
@@ -1649,7 +1662,7 @@ struct HeldWarp {
     QuadSpikes qs;
     if (w.m > 0) {
       constexpr int kA = FOUR ? 4 : 2;
-      int4* const accs = reinterpret_cast<int4*>(acc_of(e, g)) + (FOUR ? w.gi0 : w.gi0 / 2);
+      int4* const accs = reinterpret_cast<int4*>(acc_of<false>(e, g)) + (FOUR ? w.gi0 : w.gi0 / 2);
       int4 A[kA];
 #pragma unroll
       for (int k = 0; k < kA; ++k) A[k] = __ldcg(accs + k);
@@ -1698,8 +1711,8 @@ __global__ void __launch_bounds__(kDelThreads, 2)
     if (due) {
       if (PER_STEP) deliver_body<FOUR, SINGLE, true>(e, sr, kPartAll, blockIdx.x, gridDim.x);
       else if (((unsigned)g & (unsigned)e.wmask) == 0u)
-        deliver_windows<FOUR, SINGLE>(e, g, blockIdx.x, gridDim.x);
-      else deliver_rest<FOUR, SINGLE>(e, g, blockIdx.x, gridDim.x, s_item);
+        deliver_windows<FOUR, SINGLE, true>(e, g, blockIdx.x, gridDim.x);
+      else deliver_rest<FOUR, SINGLE, true>(e, g, blockIdx.x, gridDim.x, s_item);
       target += gridDim.x;
       if (!grid_barrier(count, target, limit_ns, e.flags)) return;
     }
@@ -1934,13 +1947,17 @@ void launch_after(void (*k)(Par...), int grid, int threads, cudaStream_t s, cons
 
 }  // namespace
 
+// The update's variant with the kExt* terms: they act only on instances that
+// have them, and it takes accumulator rings of any length.
+static bool ext_variant(const EngineDev& e) { return e.any_ext || (e.acc_slots & (e.acc_slots - 1)) != 0; }
+
 void launch_update(const EngineDev& e, StepRef sr, cudaStream_t s) {
   const int blocks = e.n_tiles * (kTile / 4 / kUpdThreads) + close_blocks(e);
   if (e.four) {
-    if (e.any_ext) launch_after(k_update<true, true>, blocks, kUpdThreads, s, e, sr);
+    if (ext_variant(e)) launch_after(k_update<true, true>, blocks, kUpdThreads, s, e, sr);
     else launch_after(k_update<false, true>, blocks, kUpdThreads, s, e, sr);
   } else {
-    if (e.any_ext) launch_after(k_update<true, false>, blocks, kUpdThreads, s, e, sr);
+    if (ext_variant(e)) launch_after(k_update<true, false>, blocks, kUpdThreads, s, e, sr);
     else launch_after(k_update<false, false>, blocks, kUpdThreads, s, e, sr);
   }
 }
@@ -2005,8 +2022,9 @@ auto with_persist(const EngineDev& e, bool held, F&& f) {
 }
 template <class F>
 auto with_persist(const EngineDev& e, bool held, F&& f) {
-  if (e.four) return e.any_ext ? with_persist<true, true>(e, held, f) : with_persist<false, true>(e, held, f);
-  return e.any_ext ? with_persist<true, false>(e, held, f) : with_persist<false, false>(e, held, f);
+  const bool ext = ext_variant(e);
+  if (e.four) return ext ? with_persist<true, true>(e, held, f) : with_persist<false, true>(e, held, f);
+  return ext ? with_persist<true, false>(e, held, f) : with_persist<false, false>(e, held, f);
 }
 
 }  // namespace

@@ -142,7 +142,8 @@ def test_many_regions_on_the_resident_stepper(size, regions, dt):
     net.close()
 
 
-def test_emission_threshold_with_a_ring_of_any_length():
+@pytest.mark.parametrize("schedule", [1, 2, 3])
+def test_emission_threshold_with_a_ring_of_any_length(schedule):
     """An explicit emission threshold is kept wherever a slot per step of the
     longest delay fits a third of the free memory, also where the next power
     of two of slots does not."""
@@ -158,7 +159,7 @@ def test_emission_threshold_with_a_ring_of_any_length():
     need = int(4.2 * (dmax + 1) * slot)  # a third of this holds 129 slots, not 256
     hold = torch.empty(torch.cuda.mem_get_info()[0] - need, dtype=torch.uint8, device="cuda")
     try:
-        net = _net(g, p, seed=9, emit_delay=30, autotune_at=-1)
+        net = _net(g, p, seed=9, emit_delay=30, autotune_at=-1, schedule=schedule)
         for k in (1, 70, 129):
             net.step(k)
         assert net.stats()["emit_delay"] == 30
