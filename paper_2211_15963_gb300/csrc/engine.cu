@@ -573,39 +573,41 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
   if (dev.mode != kAtEmission || tunes) hist.alloc((int64_t)D * stride);
   hcount.alloc(D);
   CK(cudaMemsetAsync(hcount.p, 0, sizeof(uint32_t) * D, stream));
-  // delay-major segment ring: room for seg_cap spikes per step -- a 64th of
-  // the neurons (at least 4096), within a sixteenth of the free memory; a
-  // step's spikes beyond seg_cap (and instances with u32 tables) take the
-  // direct path
-  auto ring = [&](int32_t per, DevBuf<uint16_t>& counts, DevBuf<int64_t>& rows, bool wanted) {
-    CK(cudaMemGetInfo(&free_b, &total_b));
+  // segment ring: room for seg_cap spikes per step -- a 64th of the neurons (at
+  // least 4096), within a sixteenth of the free memory; a step's spikes beyond
+  // seg_cap (and instances with u32 tables) take the direct path.  Per-step
+  // delivery (the engine's mode, or while the launch shapes are tuned) keeps a
+  // count per delay, windows a bound per window and one more.  One buffer
+  // serves both: a mode reads only what it has copied itself (EngineDev::since).
+  CK(cudaMemGetInfo(&free_b, &total_b));
+  int64_t ring_counts = 0, ring_rows = 0;
+  auto ring = [&](int32_t per, bool wanted) {
     const int64_t budget = (int64_t)(free_b / 16);
     const int64_t per_spike = (int64_t)D * per * 2 + (int64_t)D * 8;
     const int64_t want = std::max<int64_t>(4096, stride / 64);
     int64_t cap = std::min<int64_t>(std::min(stride, want), budget / per_spike) / 32 * 32;
     if (cap < 1024) cap = 0;  // too little room to be worth it
-    if (cap > 0 && wanted) {
-      counts.alloc((int64_t)D * per * cap);
-      rows.alloc((int64_t)D * cap);
+    if (wanted) {
+      ring_counts = std::max(ring_counts, (int64_t)D * per * cap);
+      ring_rows = std::max(ring_rows, (int64_t)D * cap);
     }
     return cap;
   };
-  // per-step delivery (the engine's mode, or while the launch shapes are
-  // tuned) and windows each have a ring of their own
   Delivery per{kPerStep, 0, 0, 1, D0 - 1, 0, nullptr, nullptr};
-  ring_cap = ring(per.dcap, hseg, hr0, dev.mode == kPerStep || tunes);
+  ring_cap = ring(per.dcap, dev.mode == kPerStep || tunes);
   per.seg_cap = ring_cap;
-  per.hseg = hseg.p;
-  per.hr0 = hr0.p;
   Delivery fast{dev.mode, dev.wmask, dev.push_now, 1, 0, 0, nullptr, nullptr};
-  if (dev.mode == kWindows) {  // a bound per window and one more
+  if (dev.mode == kWindows) {
     fast.dcap = (dev.dmax + dev.wmask) / (dev.wmask + 1) + 1;
     // (where most items lie beyond the first windows)
-    if (!dev.push_now && dev.dmax > 2 * (dev.wmask + 1) && n_inst <= 65535)
-      fast.seg_cap = ring(fast.dcap, wseg, wr0, true);
-    fast.hseg = wseg.p;
-    fast.hr0 = wr0.p;
+    if (!dev.push_now && dev.dmax > 2 * (dev.wmask + 1) && n_inst <= 65535) fast.seg_cap = ring(fast.dcap, true);
   }
+  if (ring_rows > 0) {
+    hseg.alloc(ring_counts);
+    hr0.alloc(ring_rows);
+  }
+  per.hseg = fast.hseg = hseg.p;
+  per.hr0 = fast.hr0 = hr0.p;
   base.alloc(2);
   events.alloc(2);  // [0] events counted by the deliveries, [1] scratch for the pending ones
   flags.alloc(1);

@@ -266,8 +266,8 @@ struct Engine {
   DevBuf<long long> closed;
   DevBuf<double> bw, ylast;
   DevBuf<uint32_t> hist, hcount;
-  DevBuf<uint16_t> hseg, wseg;  // segment rings of per-step delivery and of windows
-  DevBuf<int64_t> hr0, wr0;
+  DevBuf<uint16_t> hseg;  // segment ring of per-step delivery and of windows
+  DevBuf<int64_t> hr0;
   int64_t ring_cap = 0;  // spikes per step that the segment ring holds, where the mode has one
   DevBuf<unsigned long long> base, events;  // base: the two graph-half iteration words
   DevBuf<unsigned> flags;

@@ -170,3 +170,30 @@ def test_emission_threshold_with_a_ring_of_any_length(schedule):
     finally:
         del hold
         torch.cuda.empty_cache()
+
+
+def test_one_segment_ring():
+    """An engine that delivers in windows and may be tuned holds one segment
+    ring, not one for the windows and one for the tuner's per-step turns."""
+    g = synth.make_graph([600_000], 10, 15, d_within=(1, 200))
+    p = synth.default_region_params(I_ext=0.9)
+
+    def held(**opts):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        net = _net(g, p, seed=2, **opts)
+        used = before - torch.cuda.mem_get_info()[0]
+        for n in (300, 4000, 100):
+            net.step(n)
+        state = net.state()
+        net.close()
+        return used, state
+
+    held(schedule=2)  # what the first use of each path takes once
+    held(autotune_at=128)
+    per_step, a = held(schedule=2, autotune_at=-1)
+    windows, b = held(autotune_at=128)
+    # the ring alone: a 64th of the neurons x 204 slots x 51 bounds of 2 bytes
+    assert windows - per_step < 9376 * 204 * 51 * 2 // 2
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
