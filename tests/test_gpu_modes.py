@@ -33,12 +33,14 @@ def _same(net, other):
         assert np.array_equal(np.asarray(a, np.float64), np.asarray(b, np.float64))
 
 
-# Windows on networks whose longest delay is short and no power of two: the
-# accumulators of every delay at once lie beyond the emission ring's 48 MB, by
-# four channels or by size; the update adds the edges due in the window (up to
-# 532 tiles) or a kernel of its own does, with two weights and with one.
-@pytest.mark.parametrize("n,dmax,two", [(400_000, 5, True), (400_000, 6, True), (400_000, 7, True),
-                                        (800_000, 3, True), (1_600_000, 3, False)])
+# Windows on networks whose longest delay is below, at and just above a
+# window's eight steps: the accumulators of every delay at once (a power of two
+# of slots, 8 bytes a neuron, 16 with two weights) lie beyond the emission
+# ring's 48 MB; the update adds the edges due in the window (up to 532 tiles)
+# or a kernel of its own does, with two weights and with one.
+@pytest.mark.parametrize("n,dmax,two", [(400_000, 5, True), (400_000, 6, True), (400_000, 7, True), (200_000, 8, True),
+                                        (200_000, 9, True), (1_600_000, 1, True), (800_000, 3, True),
+                                        (1_600_000, 3, False)])
 def test_windows_and_short_delays(n, dmax, two):
     g = synth.make_graph([n // 2, n - n // 2], 20, 5, k_within=16, d_within=(1, dmax), d_cross=(1, dmax))
     assert g.delay.max() == dmax
@@ -197,3 +199,40 @@ def test_one_segment_ring():
     assert windows - per_step < 9376 * 204 * 51 * 2 // 2
     for x, y in zip(a, b):
         assert np.array_equal(x, y)
+
+
+def test_persistent_networks_on_two_threads():
+    """Two networks on the persistent stepper, stepped at the same time from
+    two threads, each with a grid that fills the device: their launches take
+    turns, no barrier gives up, and each equals the same network alone."""
+    p = synth.default_region_params(I_ext=0.9)
+    nets, alone = [], []
+    for k in range(2):
+        g = synth.make_graph([290_000], 10, 21 + k, d_within=(1, 60))
+        a = _net(g, p, seed=30 + k, autotune_at=-1)
+        a.step(600)
+        alone.append((a.state(), a.stats()["events"]))
+        a.close()
+        nets.append(_net(g, p, seed=30 + k, autotune_at=-1))
+        assert nets[k].stats()["schedule"] == 3
+    failed = []
+
+    def run(net):
+        try:
+            for n in (1, 99, 300, 200):
+                net.step(n)
+            net.sync()
+        except Exception as e:  # noqa: BLE001 (reported below)
+            failed.append(e)
+
+    th = [threading.Thread(target=run, args=(net,)) for net in nets]
+    for t in th:
+        t.start()
+    for t in th:
+        t.join()
+    assert not failed, failed
+    for net, (state, events) in zip(nets, alone):
+        for x, y in zip(net.state(), state):
+            assert np.array_equal(x, y)
+        assert net.stats()["events"] == events
+        net.close()
