@@ -163,7 +163,8 @@ typedef struct {
  *                    emit_delay) does so before and after them, and one more
  *                    turn of 64 steps, after the tuning is reported done,
  *                    keeps it unless the best per-step shape was faster by
- *                    a tenth than three such turns.
+ *                    a tenth than three such turns.  Calls too short for a
+ *                    turn go back to it in between.
  *                    Results depend on none of these choices (integer
  *                    accumulation).  Default 2000 (200 ms at dt 0.1 ms, past
  *                    the onset).
@@ -184,7 +185,8 @@ typedef struct {
  *                    (spike, delay) segment of a row on its own, which pays
  *                    when segments are long; at emission the accumulators
  *                    form a ring of D slots (D x N x 8 bytes, taken only when
- *                    it fits a third of the free device memory) and a
+ *                    it fits a third of the free device memory; a power of
+ *                    two of slots where that fits) and a
  *                    spike's edges of delay >= emit_delay go straight into
  *                    the slot of their arrival step, its short segments read
  *                    in one pass.  -1 (default): the engine's own rule --

@@ -1610,8 +1610,9 @@ int dbnet_stats(dbnet_t* h, dbnet_stats_t* out) {
     Engine& e = *h->eng;
     const InstHost& ih = e.inst[h->inst];
     InstDyn d = e.read_dyn(h->inst);
-    // the deliveries count a spike's events at its delay-1 item; those of
-    // the spikes handed on at the last step are added here
+    // counted at emission, by the window (or the bounds copy) that reaches the
+    // spike first, or at its delay-1 item (per step); those of the spikes that
+    // nothing has reached yet are added here
     CK(cudaMemsetAsync(e.events.p + 1, 0, sizeof(unsigned long long), e.stream));
     launch_pending_events(e.dev, e.g_host, e.events.p + 1, e.stream);
     CK(cudaGetLastError());

@@ -45,7 +45,7 @@
 //                graphs of more than 2^28 neurons).
 // Iteration g runs [k_windows or k_deliver,] k_update; the bin that ends
 // with iteration g - 1 is closed (Balloon-Windkessel step, BOLD sample) by
-// the first blocks of k_update(g), one region per thread; bins count into
+// the first blocks of k_update(g), a region on two lanes; bins count into
 // two sets of region counters in turn.
 // An engine may change between kPerStep and another mode at the start of a
 // window: arrivals before that step are in the accumulators, later ones are

@@ -242,7 +242,12 @@ struct Engine {
   static constexpr int kWindow = 8;
   // The accumulator ring up to which every edge is added at emission: it
   // stays in the L2 beside the state (one kernel a step: 7.8 against 13.2 us
-  // a step at 10,000 neurons, 12.4 against 16.6 at 30,000).
+  // a step at 10,000 neurons, 12.4 against 16.6 at 30,000).  Near the limit, at
+  // emission against in windows: 23.8 / 27.4 us at 1.5 M neurons and a longest
+  // delay of 3 (in-degree 100), 16.6 / 18.9 at 750,000 and 7, 12.0 / 11.6 at
+  // 390,000 and 15.  With one-step delays alone windows would be the better
+  // way from some 0.6 M neurons on: 25.3 / 24.5 us there, 55.7 / 51.6 at 2 M,
+  // 102 / 71.7 at 3 M (a delivery kernel a step for either took 94 to 141).
   static constexpr double kEmitRingBytes = 48.0 * 1048576.0;
   // A window's accumulators up to which it is four steps long (half the L2).
   static constexpr double kWindowRingBytes = 64.0 * 1048576.0;
@@ -357,8 +362,8 @@ struct Engine {
   // any_ext: launch the update variant with the OU current and the
   // per-neuron injected-current factors; four: four accumulator channels
   // per neuron, so that instances may carry two weights per edge.
-  // emit_from: delays >= it may be handed on at emission (0: never; the
-  // accumulators then have one slot).  n_tiles_fixed: every tile is placed
+  // emit_from: delays >= it may be handed on at emission (0: never, which
+  // leaves the accumulators' slots to the engine's rule).  n_tiles_fixed: every tile is placed
   // before the first step and stays.
   void init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D,
                  const dbnet_options_t& common, void* user_stream, bool any_ext,
