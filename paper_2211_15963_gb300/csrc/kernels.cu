@@ -1591,11 +1591,19 @@ __device__ __forceinline__ bool grid_barrier(unsigned* count, unsigned target, u
   return grid_wait(count, target, limit_ns, flags);
 }
 
-// by the tile's 256 threads, a block barrier after it
-__device__ __forceinline__ void held_load(const EngineDev& e, int tile, HeldTile& h) {
+// Whether the instance of a tile (its tile_info) has steps to run from
+// iteration g0 on.  Where not, nothing of it is read: a server may have given
+// its constants and graph to the next request while a launch is in flight.
+__device__ __forceinline__ bool runs_from(const EngineDev& e, const int4& ti, unsigned long long g0) {
+  return ti.x >= 0 && e.dyn[ti.x].active != 0 && (long long)(g0 - e.insts[ti.x].g0) < e.insts[ti.x].n_end;
+}
+
+// by the tile's 256 threads, a block barrier after it; g0: the launch's first
+// iteration
+__device__ __forceinline__ void held_load(const EngineDev& e, int tile, unsigned long long g0, HeldTile& h) {
   if (tile >= e.n_tiles) return;
   const int4 ti = __ldg(e.tile_info + tile);
-  if (ti.x < 0) return;
+  if (!runs_from(e, ti, g0)) return;
   const InstDesc& d = e.insts[ti.x];
   const int t = threadIdx.x % (kTile / 4);
   const uint32_t* from = reinterpret_cast<const uint32_t*>(&d);
@@ -1626,7 +1634,8 @@ struct HeldWarp {
   const HeldTile* tile;
   bool ou;
 
-  __device__ __forceinline__ HeldWarp(const EngineDev& e, int t, int warp, const HeldTile& h) : tile(&h) {
+  __device__ __forceinline__ HeldWarp(const EngineDev& e, int t, int warp, unsigned long long g0, const HeldTile& h)
+      : tile(&h) {
     w.inst = -1;
     w.m = w.r0 = w.nr = 0;
     w.li0 = 0;
@@ -1634,7 +1643,7 @@ struct HeldWarp {
     if (t < e.n_tiles) {
       quad_load(e, w.gi0, q);
       const int4 ti = __ldg(e.tile_info + t);
-      if (ti.x >= 0 && e.dyn[ti.x].active != 0) w.inst = ti.x;
+      if (runs_from(e, ti, g0)) w.inst = ti.x;
       w.r0 = ti.y;
       w.nr = ti.z;
     }
@@ -1700,10 +1709,10 @@ __global__ void __launch_bounds__(kDelThreads, 2)
   unsigned target = 0;
   __shared__ HeldTile s_tile;
   if (HELD) {
-    held_load(e, blockIdx.x, s_tile);
+    held_load(e, blockIdx.x, g0, s_tile);
     __syncthreads();
   }
-  HeldWarp<EXT, FOUR> h(e, HELD ? (int)blockIdx.x : e.n_tiles, warp, s_tile);
+  HeldWarp<EXT, FOUR> h(e, HELD ? (int)blockIdx.x : e.n_tiles, warp, g0, s_tile);
   if (HELD) h.prepare(g0);
   for (int s = 0; s < nsteps; ++s) {
     const unsigned long long g = g0 + (unsigned long long)s;
@@ -1758,9 +1767,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_resident(EngineDev e, unsigned l
   const int warp = threadIdx.x >> 5;
   __shared__ HeldTile s_tile[THREADS / (kTile / 4)];
   const int tile = blockIdx.x * (THREADS / (kTile / 4)) + warp / kTileWarps;
-  held_load(e, tile, s_tile[warp / kTileWarps]);
+  held_load(e, tile, g0, s_tile[warp / kTileWarps]);
   __syncthreads();
-  HeldWarp<EXT, FOUR> h(e, tile, warp % kTileWarps, s_tile[warp / kTileWarps]);
+  HeldWarp<EXT, FOUR> h(e, tile, warp % kTileWarps, g0, s_tile[warp / kTileWarps]);
   // the last blocks close the bins, for they have the fewest tiles
   const auto close = [&](unsigned long long g) {
     close_regions(e, g, (gridDim.x - 1 - blockIdx.x) * (THREADS / 32) + warp, gridDim.x * (THREADS / 32));

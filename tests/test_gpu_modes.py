@@ -236,3 +236,29 @@ def test_persistent_networks_on_two_threads():
             assert np.array_equal(x, y)
         assert net.stats()["events"] == events
         net.close()
+
+
+@pytest.mark.parametrize("max_neurons,max_delay,tune_at", [(8_192, 40, -1), (8_192, 40, 64), (200_000, 200, 64)])
+def test_server_on_the_persistent_schedule(max_neurons, max_delay, tune_at):
+    """A server by option on the persistent stepper, whose blocks hold their
+    tiles' state and constants: short requests of several regions come and
+    go, so that graphs and constants of finished ones pass to others while
+    launches are in flight.  Every request equals the same network alone."""
+    from paper_2211_15963_gb300 import dbnet
+    p = synth.default_region_params(I_ext=0.92)
+    nets = [synth.make_graph(z, 40, 50 + i, k_within=32 if len(z) > 1 else 40, d_within=(1, 20), d_cross=(20, 40),
+                             region_density=1.0)
+            for i, z in enumerate(([1500, 700], [2100], [900, 800, 700], [100] * 12))]
+    srv = dbnet.Server(max_neurons=max_neurons, max_requests=4, max_regions=40, max_delay=max_delay, chunk_steps=100,
+                       arena_bytes=1 << 29, run=dict(autotune_at=tune_at, tr_ms=20.0, schedule=3))
+    todo = [(k % 4, 150 + 137 * ((5 * k) % 11), k) for k in range(24)]
+    ids = {srv.submit(nets[j], p, n, seed=30 + i, raster_capacity=1 << 18): (j, n, i) for j, n, i in todo}
+    srv.drain()
+    for rid, (j, n, i) in ids.items():
+        net = _net(nets[j], p, seed=30 + i, raster_capacity=1 << 18, tr_ms=20.0, autotune_at=-1, schedule=2)
+        net.step(n)
+        a, b = srv.spikes(rid), net.spikes()
+        assert len(b[1]) > 100 and np.array_equal(np.stack(a), np.stack(b)), i
+        assert np.array_equal(srv.bold(rid), net.bold()), i
+        net.close()
+    srv.close()
