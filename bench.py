@@ -57,18 +57,34 @@ UNIT = "events/s"
 # (regions, neurons per region) of the two network workloads
 WORKLOAD_DIMS = {"large": (200, 100_000), "mid": (100, 20_000)}
 # kernels launched per dbnet_step(10,000): 156 replays of the 64-step graph
-# (128 launches each; 192 on the pipelined schedule, whose steps are three
-# launches, plus the long part launched ahead of the first replay) + 16
-# direct steps (2 each) + the graph's base word + the bin close at the end of
-# the call; on the persistent schedule one launch per 4,096 steps + the bin
-# close
+# (128 launches each, a delivery and an update per step; 192 on the pipelined
+# schedule, whose steps are three launches, plus the long part launched ahead
+# of the first replay) + 16 direct steps (2 each) + the graph's base word + the
+# bin close at the end of the call; on the persistent schedule one launch per
+# 4,096 steps + the bin close (which the resident stepper's launch does itself)
 LAUNCHES_PER_BIO_S = 156 * 128 + 16 * 2 + 2
 SCHEDULES = {1: "sequential", 2: "pipelined", 3: "persistent"}
 
 
-def launches_per_call(n_steps, schedule):
+# What a step's delivery is: k_windows and k_rest (windows), k_deliver (where
+# the tuner chose per-step delivery or the options ask for it), none where the
+# update adds every edge of the spikes it emits
+DELIVERY_KERNELS = "k_windows and k_rest, or k_deliver per step"
+
+
+def adds_at_emission(neurons, max_delay, two_weights=False):
+    """Whether the library adds every edge at emission by default: the
+    accumulators of a slot per step of the longest delay, a power of two of
+    them, stay within 48 MB."""
+    slots = 1
+    while slots < max_delay + 1:
+        slots *= 2
+    return slots * -(-neurons // 1024) * 1024 * (16 if two_weights else 8) <= 48 << 20
+
+
+def launches_per_call(n_steps, schedule, resident=False):
     if schedule == "persistent":
-        return -(-n_steps // 4096) + 1
+        return -(-n_steps // 4096) + (0 if resident else 1)
     pipelined = schedule == "pipelined"
     chunks, rest = divmod(n_steps, 64)
     return chunks * (192 if pipelined else 128) + 2 * rest + (2 if chunks else 1) + (
@@ -251,17 +267,19 @@ def measured_traffic(kernel, summary="traffic_mid_network_15hz.md"):
 
 
 def profiled_shape():
-    """Occupancy and issue figures of both kernels from the committed ncu
-    full sets (profiles/k_deliver_400k_grid608.md, k_update_400k.md), when
-    they were taken on the current kernel source, else None."""
+    """Occupancy and issue figures of the step's kernels from the committed
+    ncu full sets (those of profiles/k_update_400k.md, k_windows_400k.md and
+    k_deliver_400k_grid608.md that exist), when they were taken on the current
+    kernel source, else None."""
     import re
     out = {}
     for kernel, name, what in (("k_deliver", "k_deliver_400k_grid608.md", "608 blocks"),
+                               ("k_windows", "k_windows_400k.md", "608 blocks"),
                                ("k_update", "k_update_400k.md", "391 tiles")):
         try:
             txt = open(os.path.join(ROOT, "profiles", name)).read()
         except OSError:
-            return None
+            continue
         m = re.search(r"kernels\.cu sha256\[:16\]\s+([0-9a-f]+)", txt)
         if not m or m.group(1) != kernels_sha():
             return None
@@ -271,7 +289,7 @@ def profiled_shape():
             return None
         out[kernel] = {"warps_active_pct": float(warps.group(1)), "issue_active_pct": float(issue.group(1)),
                        "source": "profiles/%s (ncu full set, 400,000 neurons, %s)" % (name, what)}
-    return out
+    return out or None
 
 
 def peaks():
@@ -446,15 +464,16 @@ def run_network(args, dims, stream, dev, world, rank, seed, timed_steps, warmup,
         events, spikes, g.n_neurons, dev_ms, world, dev)
     ms_per_step = ms_all / timed_steps
 
-    # per-kernel device time (each kernel between CUDA events on the stream)
+    # device time of a step's delivery and update (each between CUDA events on
+    # the stream)
     p0 = net.stats()
     t_del, t_upd = net.step_timed(profile_steps)
     p1 = net.stats()
-    ev_per_launch = (p1["events"] - p0["events"]) / profile_steps
+    ev_per_step = (p1["events"] - p0["events"]) / profile_steps
     hbm, peak_kind = peaks()
     two = args.two_weights
     upd_bytes = g.n_neurons * (UPDATE_BYTES_PER_NEURON_FOUR if two else UPDATE_BYTES_PER_NEURON)
-    del_bytes = ev_per_launch * (DELIVER_BYTES_PER_EVENT_TWO if two else DELIVER_BYTES_PER_EVENT)
+    del_bytes = ev_per_step * (DELIVER_BYTES_PER_EVENT_TWO if two else DELIVER_BYTES_PER_EVENT)
     # a traffic summary exists only for the two standard networks
     sizes = {tuple(WORKLOAD_DIMS["large"]): "large_network", tuple(WORKLOAD_DIMS["mid"]): "mid_network"}
     name = sizes.get((g.n_regions, g.n_neurons // max(g.n_regions, 1)), "other_network")
@@ -463,14 +482,14 @@ def run_network(args, dims, stream, dev, world, rank, seed, timed_steps, warmup,
         "k_update": {"avg_us": 1e3 * t_upd / profile_steps, "algorithmic_bytes": upd_bytes,
                      "achieved_gbs": upd_bytes / (t_upd / profile_steps * 1e-3) / 1e9,
                      "traffic": measured_traffic("k_update", "traffic_%s.md" % tag)},
-        "k_deliver": {"avg_us": 1e3 * t_del / profile_steps, "algorithmic_bytes": del_bytes,
-                      "events_per_launch": ev_per_launch,
-                      "achieved_gbs": del_bytes / (t_del / profile_steps * 1e-3) / 1e9,
-                      "traffic": measured_traffic("k_deliver", "traffic_%s.md" % tag)},
+        "delivery": {"avg_us": 1e3 * t_del / profile_steps, "algorithmic_bytes": del_bytes,
+                     "events_per_step": ev_per_step, "kernels": DELIVERY_KERNELS,
+                     "achieved_gbs": del_bytes / (t_del / profile_steps * 1e-3) / 1e9,
+                     "traffic": measured_traffic("delivery", "traffic_%s.md" % tag)},
     }
     for k in kern.values():
         k["frac"] = k["achieved_gbs"] / hbm
-    dom = "k_update" if t_upd >= t_del else "k_deliver"
+    dom = "k_update" if t_upd >= t_del else "delivery"
     step_bytes = upd_bytes + del_bytes
     roof = {"bound": "hbm", "kernel": dom, "achieved": kern[dom]["achieved_gbs"], "peak": hbm,
             "unit": "GB/s", "frac": kern[dom]["frac"], "traffic": kern[dom]["traffic"],
@@ -644,8 +663,8 @@ def run_extras(args, stream, dev):
                   "mean_rate_hz": m["mean_rate_hz"], "deliver_blocks": m["deliver_blocks"],
                   "schedule": m["schedule"],
                   "k_update_us": kern["k_update"]["avg_us"], "k_update_frac": kern["k_update"]["frac"],
-                  "k_deliver_us": kern["k_deliver"]["avg_us"],
-                  "k_deliver_frac": kern["k_deliver"]["frac"],
+                  "delivery_us": kern["delivery"]["avg_us"],
+                  "delivery_frac": kern["delivery"]["frac"],
                   "path_frac": m["roofline"]["path"]["frac"], "clocks": m["clocks"]}
     if not args.no_cpu_baseline:  # the oracle at full size on the host cores
         out["mid"]["cpu_baseline"] = oracle_full_mid(args)
@@ -663,7 +682,7 @@ def run_extras(args, stream, dev):
     small_args = argparse.Namespace(**dict(vars(args), steps=3, warmup=2, profile_steps=2000))
     s = run_small(small_args, stream)
     out["small"] = {k: s[k] for k in ("config", "value", "unit", "rtf", "events_per_s",
-                                      "mean_rate_hz", "kernels_us", "clocks")}
+                                      "mean_rate_hz", "stepper", "kernels_us", "gpu_launches", "clocks")}
     out["small"]["config"] = s["config"]["workload"]
     ens_args = argparse.Namespace(**dict(vars(args), steps=3, warmup=1, members=64, separate_trs=1))
     e = run_ensemble(ens_args, stream)
@@ -1077,7 +1096,8 @@ def run_nest(args, stream=None):
                                "20,000, in-degree 100, delay 1 step, dt 1 ms, ~4.1 and ~12.1 Hz; "
                                "3 s simulated, the last second timed; value = 10 M at 12.1 Hz",
                    "step": "the timed biological second"},
-        "table": table, "clocks": clk, "gpu_launches": 2 * 1000 * len(table),
+        "table": table, "clocks": clk,
+        "gpu_launches": sum(1000 if adds_at_emission(t["neurons"], 1) else 2000 for t in table),
         "paper_context": "Supplementary Table 4: one GPU with 16 GB HBM2 (10.8 TFLOPS), "
                          "their own connectome-derived networks",
     }
@@ -1118,7 +1138,14 @@ def run_small(args, stream=None):
     clk = clocks.stop()
     ms = a.elapsed_time(b)
     s1 = net.stats()
-    t_del, t_upd = net.step_timed(args.profile_steps)
+    # (the resident stepper has no delivery grid: the default of four blocks
+    # per SM stays in the stats, which the persistent stepper never has)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    schedule = SCHEDULES[s1["schedule"]]
+    resident = schedule == "persistent" and s1["deliver_blocks"] > 2 * sms
+    # one launch per step between events, for its update (with the edges of
+    # the spikes it emits) alone; the steps above have no such launches
+    _, t_upd = net.step_timed(args.profile_steps)
     net.close()
     n_steps = STEPS_PER_BIO_S * args.steps
     line = {
@@ -1135,9 +1162,9 @@ def run_small(args, stream=None):
         "rtf": ms / args.steps / 1e3,
         "events_per_s": (s1["events"] - s0["events"]) / (ms * 1e-3),
         "mean_rate_hz": (s1["spikes"] - s0["spikes"]) / g.n_neurons / args.steps,
-        "kernels_us": {"k_deliver": 1e3 * t_del / args.profile_steps,
-                       "k_update": 1e3 * t_upd / args.profile_steps},
-        "clocks": clk, "gpu_launches": 2 * n_steps,
+        "stepper": "k_resident" if resident else schedule,
+        "kernels_us": {"k_update launched step by step": 1e3 * t_upd / args.profile_steps},
+        "clocks": clk, "gpu_launches": args.steps * launches_per_call(STEPS_PER_BIO_S, schedule, resident),
     }
     return line
 
@@ -1253,7 +1280,7 @@ def run_dt_study(args, stream=None):
         "table": table,
         "paper_context": "Extended Data Fig. 1 / Results: about 5 % relative membrane-potential "
                          "error at dt 1 ms against 0.001 ms over one second",
-        "gpu_launches": int(sum(2 * DT_STUDY_STEPS * round(1.0 / x) for x in DT_STUDY_MS)),
+        "gpu_launches": DT_STUDY_STEPS * len(DT_STUDY_MS),  # one resident launch a call
     }
     return line
 
@@ -1316,7 +1343,7 @@ def run_columns(args, stream=None):
         "drive_I_ext": drive, "sub_network_rate_hz": rate_sub,
         "out_degree": {"max": int(deg.max()), "p99": float(np.percentile(deg, 99)),
                        "median": float(np.median(deg))},
-        "kernels_us": {"k_deliver": 1e3 * t_del / args.profile_steps,
+        "kernels_us": {"delivery": 1e3 * t_del / args.profile_steps,
                        "k_update": 1e3 * t_upd / args.profile_steps},
         "generate_s": t_gen, "gpu_launches": 2 * STEPS_PER_BIO_S * args.steps,
     }

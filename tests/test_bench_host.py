@@ -135,3 +135,14 @@ def test_arm_cpu_part_names():
     import bench
     assert bench.ARM_PARTS["0xd4f"] == "Arm Neoverse V2"
     assert isinstance(bench.cpu_model(), str) and bench.cpu_model()
+
+
+def test_delivery_mode_and_resident_launches():
+    """The default delivery by size (48 MB of accumulators in a power of two
+    of slots) and the resident stepper's launches, which close the last bin
+    themselves."""
+    import bench
+    assert bench.adds_at_emission(3_145_728, 1) and not bench.adds_at_emission(3_145_729, 1)
+    assert bench.adds_at_emission(10_000, 20) and not bench.adds_at_emission(2_000_000, 200)
+    assert bench.adds_at_emission(1_572_864, 1, True) and not bench.adds_at_emission(1_572_865, 1, True)
+    assert bench.launches_per_call(10_000, "persistent", True) == 3
