@@ -418,7 +418,10 @@ void Engine::init(const std::vector<InstSpec>& specs, void* user_stream) {
   // layout: instances end to end, each on whole tiles
   int64_t tiles = 0;
   int32_t regions = 0, dmax_all = 1;
+  double neurons = 0.0, edges = 0.0;
   for (const auto& sp : specs) {
+    neurons += (double)sp.graph->N;
+    edges += (double)sp.graph->E;
     tiles += (sp.graph->N + kTile - 1) / kTile;
     regions += sp.graph->R;
     dmax_all = std::max(dmax_all, sp.graph->max_delay);
@@ -441,7 +444,7 @@ void Engine::init(const std::vector<InstSpec>& specs, void* user_stream) {
   }
   // with spike binning a spike waits up to spb - 1 steps for its bin to end
   init_pool(n, tiles, regions, dmax_all + 1 + bin_lead(specs[0].opt), specs[0].opt, user_stream,
-            any_ext, four, emit_from > dmax_all ? 0 : emit_from, true);
+            any_ext, four, emit_from > dmax_all ? 0 : emit_from, true, edges / neurons);
   int64_t t = 0;
   int32_t r = 0;
   for (int k = 0; k < n; ++k) {
@@ -455,7 +458,7 @@ void Engine::init(const std::vector<InstSpec>& specs, void* user_stream) {
 
 void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D,
                        const dbnet_options_t& common, void* user_stream, bool any_ext,
-                       bool four, int32_t emit_from, bool n_tiles_fixed) {
+                       bool four, int32_t emit_from, bool n_tiles_fixed, double mean_row) {
   if (user_stream) {
     stream = (cudaStream_t)user_stream;
     own_stream = false;
@@ -492,8 +495,9 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
     while (p < n) p *= 2;
     return p;
   };
-  // (two slots at least: the pipelined schedule delivers into step g + 1's
-  // slot while the update reads step g's)
+  // (two slots: the pipelined schedule delivers into step g + 1's slot while the
+  // update reads step g's; windows of one step have one and are not tuned for
+  // that schedule)
   int32_t slots = 2;
   dev.mode = kPerStep;
   const int32_t D0 = D;  // ring slots that per-step delivery needs
@@ -517,13 +521,16 @@ void Engine::init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D
     // Never longer than the longest delay: a window counts its earlier
     // spikes' events as it goes over those that may still have edges due.
     dev.push_now = tiles <= kPushTiles;
-    int32_t W = dev.push_now ? (lead > 0 ? 4 : kWindow) : 4 * slot_b <= kWindowRingBytes ? 4 : 2;
+    int32_t W = dev.push_now                     ? (lead > 0 ? 4 : kWindow)
+                : 4 * slot_b <= kWindowRingBytes ? 4
+                : 2 * slot_b <= kWindowPairBytes ? 2
+                                                 : 1;
     while (W > dev.dmax) W /= 2;
     const int32_t all = pow2(D), win = pow2(W + lead);
     if (fits(all) && all * slot_b <= kEmitRingBytes) {
       dev.mode = kAtEmission;
       slots = all;
-    } else if (fits(win)) {
+    } else if (fits(win) && !(slot_b > kLongRowSlotBytes && mean_row >= kLongRow)) {
       dev.mode = kWindows;
       dev.wmask = W - 1;
       slots = win;
@@ -1041,9 +1048,11 @@ int64_t Engine::tune_steps(int64_t n) {
   }
   const int sched = c % 3, grid = tune_grid[(size_t)(c / 3)];
   if ((fixed_schedule != DBNET_SCHEDULE_AUTO && sched + 1 != fixed_schedule) ||
+      (sched == 1 && dev.acc_slots < 2 && dev.dmax > 1) ||
       (sched == 2 && (grid > persist_max || !persist_tunable)) || tune_ms[(size_t)c] >= kDropped) {
-    // not a candidate (another schedule, too many blocks to be co-resident),
-    // or dropped after the first round
+    // not a candidate (another schedule, no second accumulator slot for the
+    // long part to go into beside the update, too many blocks to be
+    // co-resident), or dropped after the first round
     tune_ms[(size_t)c] = kDropped;
     finish_turn(C);
     return 0;

@@ -249,8 +249,19 @@ struct Engine {
   // way from some 0.6 M neurons on: 25.3 / 24.5 us there, 55.7 / 51.6 at 2 M,
   // 102 / 71.7 at 3 M (a delivery kernel a step for either took 94 to 141).
   static constexpr double kEmitRingBytes = 48.0 * 1048576.0;
-  // A window's accumulators up to which it is four steps long (half the L2).
+  // A window's accumulators up to which it is four steps long (half the L2),
+  // and two (a little more than the L2); else one, which reads shorter pieces
+  // but refetches fewer accumulators.  Two steps against one, us a step: 156.9 /
+  // 158.3 at 8 M neurons and in-degree 400 (128 MB), 200.8 / 199.1 at 10 M,
+  // 339.5 / 319.6 at 16 M; 211 / 194 at 8 M and 1,000, 279 / 247 at 10 M.
   static constexpr double kWindowRingBytes = 64.0 * 1048576.0;
+  static constexpr double kWindowPairBytes = 144.0e6;
+  // One step's accumulators beyond the L2 and rows as long as this: per-step
+  // delivery from the start.  Against windows of one step: 619 / 649 us a step
+  // at 20 M neurons and in-degree 1,000, 15 Hz (839 in windows of two), 411 / 410
+  // at 17 M and 800, 372 / 354 at 17 M and 500, 425 / 389 at 20 M and 300.
+  static constexpr double kLongRowSlotBytes = 128.0 * 1048576.0;
+  static constexpr double kLongRow = 800.0;
   // Tiles up to which the update adds its own spikes' edges due in the window
   // (a separate kernel else): while all its blocks are resident at once, the
   // few warps that stay for their spikes delay no other.  Inside / outside
@@ -364,10 +375,10 @@ struct Engine {
   // per neuron, so that instances may carry two weights per edge.
   // emit_from: delays >= it may be handed on at emission (0: never, which
   // leaves the accumulators' slots to the engine's rule).  n_tiles_fixed: every tile is placed
-  // before the first step and stays.
+  // before the first step and stays.  mean_row: edges per neuron (0: unknown).
   void init_pool(int32_t n_inst, int64_t tiles, int32_t regions, int32_t D,
                  const dbnet_options_t& common, void* user_stream, bool any_ext,
-                 bool four = false, int32_t emit_from = 0, bool n_tiles_fixed = false);
+                 bool four = false, int32_t emit_from = 0, bool n_tiles_fixed = false, double mean_row = 0.0);
   int64_t tune_emit(int64_t n);
   // Put instance k on tiles [first_tile, +tiles of its graph) and region
   // slots [rbase, +R): its constants, buffers and initial state; its step 0

@@ -262,3 +262,21 @@ def test_server_on_the_persistent_schedule(max_neurons, max_delay, tune_at):
         assert np.array_equal(srv.bold(rid), net.bold()), i
         net.close()
     srv.close()
+
+
+def test_windows_of_one_step():
+    """Two steps' accumulators beyond the L2: windows of one step on one
+    accumulator slot, whose bounds ring keeps a bound for every delay, against
+    per-step delivery, through the tuner and back."""
+    g = synth.make_graph([4_700_000, 4_900_000], 4, 29, k_within=3, d_within=(1, 5), d_cross=(5, 11))
+    p = [synth.default_region_params(I_ext=0.9 + 0.03 * r) for r in range(2)]
+    net = _net(g, p, seed=3, autotune_at=90)
+    plain = _net(g, p, seed=3, schedule=2, autotune_at=-1)
+    for n in (1, 2, 70, 17, 300, 20, 2500):
+        net.step(n)
+        plain.step(n)
+        s, sp = net.stats(), plain.stats()
+        assert s["events"] == sp["events"] and s["spikes"] == sp["spikes"] > 0
+    _same(net, plain)
+    net.close()
+    plain.close()
