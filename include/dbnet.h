@@ -155,7 +155,9 @@ typedef struct {
  *                    two 1,024-neuron tiles per SM also an eighth, a quarter
  *                    and half of the SMs) on each schedule the schedule
  *                    option admits (the persistent one only while its blocks
- *                    hold at most one tile each) -- runs 64 steps timed by
+ *                    hold at most one tile each, the pipelined one not where
+ *                    windows of one step left one accumulator slot) -- runs
+ *                    64 steps timed by
  *                    CUDA events, three times each in turn (after the first
  *                    round those over twice the best drop out), and the
  *                    smallest total is kept.  These turns time per-step
@@ -191,8 +193,10 @@ typedef struct {
  *                    the slot of their arrival step, its short segments read
  *                    in one pass.  -1 (default): the engine's own rule --
  *                    every edge at emission where that ring stays in the L2
- *                    (48 MB), else in windows of a few steps, a row's edges
- *                    due in a window read as one segment --; d >= 1: delays
+ *                    (48 MB), else in windows of one to eight steps, a row's
+ *                    edges due in a window read as one segment, or in their
+ *                    own step where one step's accumulators exceed the L2 and
+ *                    rows average 800 edges or more --; d >= 1: delays
  *                    >= d at emission, the others in their own step;
  *                    0: the delays from which every (row, delay) segment
  *                    holds fewer than 4 edges on average (estimated from a
